@@ -224,6 +224,7 @@ StageArgs base_args(const cvweno_mesh_s* m) {
   a.nu_scale = (float)(m->h / (2.0 * m->p));
   a.h_e = (float)m->h;
   a.tab_img = m->d_tabimg;
+  a.pk_img = m->d_pkimg;
   a.mlp = m->surrogate;
   a.mlp_conf_min = m->surrogate_conf_min;
   a.mlp_fallbacks = m->surrogate_fallbacks;
@@ -431,6 +432,7 @@ cvweno_status cvweno_mesh_destroy(cvweno_mesh m) {
   cudaFree(m->d_cg_xg);
   cudaFree(m->d_cg_ml);
   cudaFree(m->d_tabimg);
+  cudaFree(m->d_pkimg);
   cudaFreeHost(m->h_status);
   cudaFreeHost(m->h_red);
   for (int i = 0; i < kMaxMarks; ++i)
@@ -509,6 +511,8 @@ cvweno_status cvweno_mesh_create(const cvweno_mesh_desc* d, cvweno_mesh* out) {
   if (e == cudaSuccess) e = cudaMalloc(&m->d_lambda, sizeof(float) * (size_t)m->ncell);
   if (e == cudaSuccess) e = cudaMalloc(&m->d_tabimg, sizeof(float) * (size_t)tab_image_floats(m->dim, m->p));
   if (e == cudaSuccess) e = launch_tab_image(m->dim, m->p, m->tables, m->d_tabimg, 0);
+  if (e == cudaSuccess) e = cudaMalloc(&m->d_pkimg, sizeof(float) * (size_t)packed_image_floats(m->dim, m->p));
+  if (e == cudaSuccess) e = launch_packed_image(m->dim, m->p, m->tables, m->d_pkimg, 0);
   if (e == cudaSuccess) e = cudaStreamSynchronize(0);
   if (m->kind == CVWENO_CG) {
     if (e == cudaSuccess) e = cudaMalloc(&m->d_rloc, sizeof(float) * (size_t)m->ncell * m->nd);

@@ -26,15 +26,15 @@ struct BatchTile {
 // all meshes of that degree (only tscale, the vertex-output scaling, depends on h, and
 // the RK and residual modes do not read it).
 struct AllTables {
-  DgTables<2, 1> t1;
-  DgTables<2, 2> t2;
-  DgTables<2, 3> t3;
-  DgTables<2, 4> t4;
+  PackedTables<2, 1> t1;
+  PackedTables<2, 2> t2;
+  PackedTables<2, 3> t3;
+  PackedTables<2, 4> t4;
 };
 
 template <int PSEL>
 struct BatchTab {
-  using type = DgTables<2, PSEL>;
+  using type = PackedTables<2, PSEL>;
 };
 template <>
 struct BatchTab<0> {
@@ -42,28 +42,28 @@ struct BatchTab<0> {
 };
 
 template <int P>
-__device__ __forceinline__ const DgTables<2, P>& pick(const AllTables& T);
+__device__ __forceinline__ const PackedTables<2, P>& pick(const AllTables& T);
 template <>
-__device__ __forceinline__ const DgTables<2, 1>& pick<1>(const AllTables& T) { return T.t1; }
+__device__ __forceinline__ const PackedTables<2, 1>& pick<1>(const AllTables& T) { return T.t1; }
 template <>
-__device__ __forceinline__ const DgTables<2, 2>& pick<2>(const AllTables& T) { return T.t2; }
+__device__ __forceinline__ const PackedTables<2, 2>& pick<2>(const AllTables& T) { return T.t2; }
 template <>
-__device__ __forceinline__ const DgTables<2, 3>& pick<3>(const AllTables& T) { return T.t3; }
+__device__ __forceinline__ const PackedTables<2, 3>& pick<3>(const AllTables& T) { return T.t3; }
 template <>
-__device__ __forceinline__ const DgTables<2, 4>& pick<4>(const AllTables& T) { return T.t4; }
+__device__ __forceinline__ const PackedTables<2, 4>& pick<4>(const AllTables& T) { return T.t4; }
 template <int P>
-__device__ __forceinline__ const DgTables<2, P>& pick(const DgTables<2, P>& T) {
+__device__ __forceinline__ const PackedTables<2, P>& pick(const PackedTables<2, P>& T) {
   return T;
 }
 
 template <int P, int SYS, int TX, int TY, class TT>
 __device__ __forceinline__ void batch_tile(const StageArgs& a, const TT& T, const BatchTile& bt, float* smem,
                                            int& cur_p) {
-  const DgTables<2, P>& t = pick<P>(T);
+  const PackedTables<2, P>& t = pick<P>(T);
   // a new degree needs its tabulations in shared memory; the previous tile's readers
   // have passed the barrier that ends it, and the tile's first barrier publishes them
   if (cur_p != P) {
-    stage_tables_to_smem<2, P, TX, TY>(a.tab_img, smem);
+    stage_tables_to_smem<2, P, TX, TY>(a.pk_img, smem);
     cur_p = P;
   }
   scalar_tile<2, P, SYS, TX, TY>(a, t, bt.i0, bt.j0, smem);
@@ -380,17 +380,17 @@ void free_batch(cvweno_batch b) {
 }
 
 template <int P>
-bool same_tables(const DgTables<2, P>& x, const DgTables<2, P>& y) {
+bool same_tables(const PackedTables<2, P>& x, const PackedTables<2, P>& y) {
   // everything but tscale (vertex-output scaling, not read by the batch)
-  DgTables<2, P> a = x, c = y;
+  PackedTables<2, P> a = x, c = y;
   memset(a.tscale, 0, sizeof(a.tscale));
   memset(c.tscale, 0, sizeof(c.tscale));
   return memcmp(&a, &c, sizeof(a)) == 0;
 }
 
 template <int P>
-bool take_tables(DgTables<2, P>& dst, bool have, const cvweno_mesh m) {
-  const DgTables<2, P>& src = *static_cast<const DgTables<2, P>*>(m->tables);
+bool take_tables(PackedTables<2, P>& dst, bool have, const cvweno_mesh m) {
+  const PackedTables<2, P>& src = static_cast<const DgTables<2, P>*>(m->tables)->pk;
   if (!have) {
     dst = src;
     return true;

@@ -46,6 +46,28 @@ __device__ __forceinline__ bool cvw_span(int* status, long long first, long long
 #define CVW_EXTENT(a, field) int64_t(0)
 #endif
 
+// What the packed kernels read with compile-time indices, by value (constant bank).  Modes are
+// paired (2i, 2i + 1) in x (dg_packed.cuh); the padded mode of an odd N has zero entries.
+//   sigma2[ky][p]  sigma of the derivative pair
+//   R2[e]          the nonzero blocks of R, in the order norm_coords2 walks them: row pair
+//                  (my, p), then the column pairs (my, p), (my, p + 1) ..., (my + 2, 0) ...;
+//                  R couples only modes of equal parity in x and in y.  The mean's row is zero.
+//   tscale[k]      reference -> physical derivative
+template <int DIM, int P>
+struct PackedTables {
+  static constexpr int N = P + 1, NY1 = DIM == 2 ? N : 1, MP = (N + 1) / 2, ND = DIM == 2 ? N * N : N;
+  static constexpr int nr2() {
+    int n = 0;
+    for (int my = 0; my < NY1; ++my)
+      for (int p = 0; p < MP; ++p) n += (NY1 - 1 - my) / 2 * MP + MP - p;
+    return n;
+  }
+  static constexpr int NR2 = nr2();
+  float2 sigma2[NY1][MP];
+  float2 R2[NR2];
+  float tscale[ND];
+};
+
 // Reference-cell tabulations of one (dim, p) pair, FP64 on the host rounded once to
 // FP32, passed to the kernels by value (__grid_constant__), so that every warp reads
 // them through the constant bank with uniform addresses (the entries read with per-lane
@@ -76,7 +98,30 @@ struct DgTables {
   float tscale[ND];
   float R[NS][NS];
   float A[NC][NS][NS];
+  PackedTables<DIM, P> pk;
 };
+
+template <int DIM, int P>
+inline void pack_tables(DgTables<DIM, P>& t) {
+  using K = PackedTables<DIM, P>;
+  K& k = t.pk;
+  constexpr int N = K::N, NY1 = K::NY1, MP = K::MP, ND = K::ND;
+  auto r = [&](int i, int j) { return i > 0 && j > 0 ? t.R[i - 1][j - 1] : 0.0f; };  // by mode
+  int e = 0;
+  for (int my = 0; my < NY1; ++my)
+    for (int p = 0; p < MP; ++p) {
+      const bool pad = 2 * p + 1 >= N;
+      k.sigma2[my][p] = make_float2(t.sigma[2 * p + N * my], pad ? 0.0f : t.sigma[2 * p + 1 + N * my]);
+      for (int qy = my; qy < NY1; qy += 2)
+        for (int q = 0; q < MP; ++q) {
+          if (qy == my && q < p) continue;
+          const bool padq = 2 * q + 1 >= N;
+          k.R2[e++] = make_float2(r(2 * p + N * my, 2 * q + N * qy),
+                                  pad || padq ? 0.0f : r(2 * p + 1 + N * my, 2 * q + 1 + N * qy));
+        }
+    }
+  for (int m = 0; m < ND; ++m) k.tscale[m] = t.tscale[m];
+}
 
 // Device image of the tabulations that the stage kernels index with a different value in
 // every lane (A padded to NSP columns, B, Bd, Bk, w), in the order they take in shared
@@ -114,6 +159,46 @@ inline int tab_image_floats(int dim, int p) {
     case 22: return TabImage<2, 2>::FLOATS_ALL;
     case 23: return TabImage<2, 3>::FLOATS_ALL;
     case 24: return TabImage<2, 4>::FLOATS_ALL;
+    default: return 0;
+  }
+}
+
+// Device image of the node tabulations, in the order they take in shared memory.  Node
+// group g holds the Gauss nodes g and N - 1 - g (= -+xi; the middle node of an odd rule is
+// its own partner): rows of mode pairs for the x direction, every entry doubled for the y
+// direction, where both halves (two x nodes) take the same factor.
+template <int DIM, int P>
+struct PackedImage {
+  static constexpr int N = P + 1, NY1 = DIM == 2 ? N : 1, MP = (N + 1) / 2, NG = (N + 1) / 2;
+  static constexpr int NS = DgTables<DIM, P>::NS, NC = DgTables<DIM, P>::NC;
+  static constexpr int BX = 0;                               // [NG][MP] P_m(xi_g)
+  static constexpr int DX = BX + 2 * NG * MP;                // [NG][MP] P_m'(xi_g)
+  static constexpr int BY = DX + 2 * NG * MP;                // [NG][N] doubled P_m
+  static constexpr int DY = BY + (DIM == 2 ? 2 * NG * N : 0);
+  static constexpr int KX = DY + (DIM == 2 ? 2 * NG * N : 0);  // [N][NG][MP] P_m^(k)(xi_g)
+  static constexpr int KY = KX + 2 * N * NG * MP;            // [N][NG][N] doubled
+  static constexpr int WX = KY + (DIM == 2 ? 2 * N * NG * N : 0);  // [NG] weight (half at the middle node)
+  static constexpr int WY = WX + NG;                         // [NG] weight
+  static constexpr int FLOATS = (WY + NG + 3) / 4 * 4;
+  // The tensor-core form of the sensor's corner products (2D, p = 3): R C_l split into TF32
+  // hi and lo parts, zero-padded to TCK x TCK, in the canonical K-major operand layout
+  // [part][corner l][K chunk of 4][row i][4] (tc_tf32.cuh).
+  static constexpr bool HAS_TC = DIM == 2 && P == 3;
+  static constexpr int TCK = (NS + 15) / 16 * 16;
+  static constexpr int TC = FLOATS;
+  static constexpr int FLOATS_ALL = FLOATS + (HAS_TC ? 2 * NC * TCK * TCK : 0);
+};
+constexpr int kMaxPackedImage = imax(PackedImage<2, kMaxP>::FLOATS_ALL, PackedImage<2, 3>::FLOATS_ALL);
+inline int packed_image_floats(int dim, int p) {
+  switch (dim * 10 + p) {
+    case 11: return PackedImage<1, 1>::FLOATS_ALL;
+    case 12: return PackedImage<1, 2>::FLOATS_ALL;
+    case 13: return PackedImage<1, 3>::FLOATS_ALL;
+    case 14: return PackedImage<1, 4>::FLOATS_ALL;
+    case 21: return PackedImage<2, 1>::FLOATS_ALL;
+    case 22: return PackedImage<2, 2>::FLOATS_ALL;
+    case 23: return PackedImage<2, 3>::FLOATS_ALL;
+    case 24: return PackedImage<2, 4>::FLOATS_ALL;
     default: return 0;
   }
 }
@@ -179,6 +264,7 @@ struct StageArgs {
   float* norm_out;     // kModeFeatures: ||u^e||_e per cell (may be null)
   float h_e;           // cell diameter
   const float* tab_img;  // TabImage of the mesh's tabulations (device)
+  const float* pk_img;   // PackedImage of the mesh's tabulations (device)
   float adv_vx, adv_vy;
   float gas_gamma;
   // CG only: nodal lattice and the per-stage work arrays
@@ -241,6 +327,7 @@ struct cvweno_mesh_s {
   void* tables;            // host copy of DgTables<dim, p>
   size_t tables_bytes;
   float* d_tabimg;         // TabImage<dim, p> (device)
+  float* d_pkimg;          // PackedImage<dim, p> (device)
   // CG: nodal lattice, tabulations and stage work arrays
   int kind;
   int nnx, nny;
@@ -299,6 +386,8 @@ cudaError_t launch_positivity(const cvweno_mesh_s* m, const StageArgs& a, float*
 // dg_scalar_2d.cu: writes TabImage<dim, p> of the host tables t (DgTables<dim, p>) to
 // dst (device, tab_image_floats(dim, p) floats), stream-ordered on s
 cudaError_t launch_tab_image(int dim, int p, const void* t, float* dst, cudaStream_t s);
+// dg_scalar_2d.cu: likewise PackedImage<dim, p> (packed_image_floats(dim, p) floats)
+cudaError_t launch_packed_image(int dim, int p, const void* t, float* dst, cudaStream_t s);
 // cg_scalar.cu
 cudaError_t launch_stage_cg(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t s);
 // api.cu: the stage arguments common to every launch on mesh m (no state pointers, no RK)

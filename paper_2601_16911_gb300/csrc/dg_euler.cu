@@ -16,9 +16,10 @@
 //           so FP32 rounding is relative to the variation inside the cell.
 // Non-positive density or pressure at any node raises the positivity bit of the
 // status word (the computation continues; nothing traps).
-#include "dg_scalar_kernel.cuh"
+#include "cg_tile.cuh"
 
 namespace cvw {
+using namespace legacy;
 namespace {
 
 constexpr int NV = 4;

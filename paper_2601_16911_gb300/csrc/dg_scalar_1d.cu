@@ -26,7 +26,7 @@ static cudaError_t launch_steps_tile(const cvweno_mesh_s* m, const StepArgs& a, 
   static_assert(Lay::BYTES <= 48 * 1024, "a 1D tile fits the default shared memory");
   if (m->tables_bytes != sizeof(DgTables<1, P>)) return cudaErrorInvalidValue;
   return launch_pdl(dg_scalar_steps_tile<P, SYS, TX>, dim3(1), dim3(stage_block_threads<1, P, TX, 1>()), Lay::BYTES,
-                    s, a, *static_cast<const DgTables<1, P>*>(m->tables));
+                    s, a, static_cast<const DgTables<1, P>*>(m->tables)->pk);
 }
 
 cudaError_t launch_steps_1d_tile(const cvweno_mesh_s* m, const StepArgs& a, cudaStream_t s) {

@@ -37,23 +37,23 @@ cudaError_t launch_stage(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_
 
 namespace {
 template <int DIM, int P>
-cudaError_t tab_image(const void* t, float* dst, cudaStream_t s) {
-  tab_image_kernel<DIM, P><<<1, 256, 0, s>>>(*static_cast<const DgTables<DIM, P>*>(t), dst);
+cudaError_t packed_image(const void* t, float* dst, cudaStream_t s) {
+  packed_image_kernel<DIM, P><<<1, 256, 0, s>>>(*static_cast<const DgTables<DIM, P>*>(t), dst);
   return cudaGetLastError();
 }
 }  // namespace
 
-cudaError_t launch_tab_image(int dim, int p, const void* t, float* dst, cudaStream_t s) {
+cudaError_t launch_packed_image(int dim, int p, const void* t, float* dst, cudaStream_t s) {
   if (!t || !dst) return cudaErrorInvalidValue;
   switch (dim * 10 + p) {
-    case 11: return tab_image<1, 1>(t, dst, s);
-    case 12: return tab_image<1, 2>(t, dst, s);
-    case 13: return tab_image<1, 3>(t, dst, s);
-    case 14: return tab_image<1, 4>(t, dst, s);
-    case 21: return tab_image<2, 1>(t, dst, s);
-    case 22: return tab_image<2, 2>(t, dst, s);
-    case 23: return tab_image<2, 3>(t, dst, s);
-    case 24: return tab_image<2, 4>(t, dst, s);
+    case 11: return packed_image<1, 1>(t, dst, s);
+    case 12: return packed_image<1, 2>(t, dst, s);
+    case 13: return packed_image<1, 3>(t, dst, s);
+    case 14: return packed_image<1, 4>(t, dst, s);
+    case 21: return packed_image<2, 1>(t, dst, s);
+    case 22: return packed_image<2, 2>(t, dst, s);
+    case 23: return packed_image<2, 3>(t, dst, s);
+    case 24: return packed_image<2, 4>(t, dst, s);
     default: return cudaErrorNotSupported;
   }
 }
@@ -62,17 +62,14 @@ cudaError_t launch_tab_image(int dim, int p, const void* t, float* dst, cudaStre
 
 namespace cvw {
 namespace {
-// sin d and cos d - 1 as the KPP flux forms them: the series up to |d| = 1, the reduced
-// series beyond (ScalarLaw<KPP>::flux_dev).
+// sin d and cos d - 1 as the KPP flux forms them (sin_cosm1_2, both halves).
 __global__ void kpp_sincos_kernel(const float* __restrict__ d, float* __restrict__ out, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float s, cm1;
-    if (fabsf(d[i]) <= 1.0f)
-      sin_cosm1_small(d[i], s, cm1);
-    else
-      sin_cosm1_reduced(d[i], s, cm1);
-    out[i] = s;
-    out[n + i] = cm1;
+  for (int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x); i < n; i += 2 * gridDim.x * blockDim.x) {
+    f2 s, cm1;
+    sin_cosm1_2(mk2(d[i], i + 1 < n ? d[i + 1] : 0.0f), s, cm1);
+    out[i] = s.x;
+    out[n + i] = cm1.x;
+    if (i + 1 < n) out[i + 1] = s.y, out[n + i + 1] = cm1.y;
   }
 }
 }  // namespace

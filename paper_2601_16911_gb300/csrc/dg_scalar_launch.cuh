@@ -27,7 +27,7 @@ cudaError_t launch_scalar(const cvweno_mesh_s* m, const StageArgs& a, cudaStream
   if (m->tables_bytes != sizeof(Tb)) return cudaErrorInvalidValue;
   dim3 grid((a.nx + TX - 1) / TX, DIM == 2 ? (a.ny + TY - 1) / TY : 1);
   const int threads = stage_block_threads<DIM, P, TX, TY>();
-  return launch_pdl(kern, grid, dim3(threads), smem, s, a, *static_cast<const Tb*>(m->tables));
+  return launch_pdl(kern, grid, dim3(threads), smem, s, a, static_cast<const Tb*>(m->tables)->pk);
 }
 
 // The tensor-core form of the 2D Q3 stage kernel (8 x 16 tiles, TileLayout<..., true>).
@@ -41,7 +41,7 @@ cudaError_t launch_scalar_tc(const cvweno_mesh_s* m, const StageArgs& a, cudaStr
   if (e != cudaSuccess) return e;
   if (m->tables_bytes != sizeof(Tb)) return cudaErrorInvalidValue;
   dim3 grid((a.nx + 7) / 8, (a.ny + 15) / 16);
-  return launch_pdl(kern, grid, dim3(128), Lay::BYTES, s, a, *static_cast<const Tb*>(m->tables));
+  return launch_pdl(kern, grid, dim3(128), Lay::BYTES, s, a, static_cast<const Tb*>(m->tables)->pk);
 }
 
 }  // namespace cvw

@@ -33,7 +33,7 @@ constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) float g_stage_scratch[2 * kStaticStateFloats];
 static __device__ __align__(256) int g_static_status;
-static __device__ __align__(256) float g_static_tab_image[cvw::kMaxTabImage];
+static __device__ __align__(256) float g_static_tab_image[cvw::kMaxPackedImage];
 
 struct DeviceSlots {
   float* scratch;
@@ -145,7 +145,7 @@ extern "C" cvweno_status cvweno_step_static(const cvweno_mesh_desc* d, float* u,
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   // the tabulation image first: the stage kernels read it before their dependent-launch
   // wait, so a stream operation that is not one of them (the status reset) separates them
-  if (launch_tab_image(m.dim, m.p, m.tables, slots.tab_image, s) != cudaSuccess) return CVWENO_ERR_CUDA;
+  if (launch_packed_image(m.dim, m.p, m.tables, slots.tab_image, s) != cudaSuccess) return CVWENO_ERR_CUDA;
   // the status word must start at zero for this step; the stage buffers are fully
   // written before they are read
   if (cudaMemsetAsync(slots.status, 0, sizeof(int), s) != cudaSuccess) return CVWENO_ERR_CUDA;
@@ -163,7 +163,7 @@ extern "C" cvweno_status cvweno_step_static(const cvweno_mesh_desc* d, float* u,
   a.two_dy = (float)(2.0 / m.dy);
   a.nu_scale = (float)(m.h / (2.0 * m.p));
   a.h_e = (float)m.h;
-  a.tab_img = slots.tab_image;
+  a.pk_img = slots.tab_image;
   a.eps = (float)p.eps;
   a.r = (int)p.r;
   a.q = (float)p.q;

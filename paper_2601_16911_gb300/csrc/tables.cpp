@@ -220,6 +220,7 @@ cvweno_status fill_into(DgTables<DIM, P>* t, double dx, double dy) {
         t->A[l][i][j] = (float)acc;
       }
   }
+  pack_tables<DIM, P>(*t);
   return CVWENO_OK;
 }
 
