@@ -16,10 +16,9 @@
 //           so FP32 rounding is relative to the variation inside the cell.
 // Non-positive density or pressure at any node raises the positivity bit of the
 // status word (the computation continues; nothing traps).
-#include "cg_tile.cuh"
+#include "dg_scalar_kernel.cuh"
 
 namespace cvw {
-using namespace legacy;
 namespace {
 
 constexpr int NV = 4;
@@ -47,629 +46,563 @@ __device__ __forceinline__ EulerMean euler_mean(float g, const float* Ub) {
 
 // a*b - c*d with the rounding of c*d compensated (Kahan's FMA form): the result is
 // accurate relative to itself even when the two products nearly cancel.
-__device__ __forceinline__ float diff_of_products(float a, float b, float c, float d) {
-  const float w = c * d;
-  const float e = fmaf(-c, d, w);  // w - c*d, exactly
-  const float f = fmaf(a, b, -w);  // a*b - w, one rounding
-  return f + e;
+__device__ __forceinline__ f2 diff_of_products(f2 a, f2 b, float c, f2 d) {
+  const f2 nw = mul2(dup2(-c), d);       // -w
+  const f2 ne = fma2(dup2(c), d, nw);    // c*d - w, exactly
+  return sub2(fma2(a, b, nw), ne);
 }
 
-// F(Ubar + d) - F(Ubar) in x and y, written as sums of (mean quantity) x (deviation)
-// so that FP32 rounding is relative to |d|:
+// F(Ubar + d) - F(Ubar) in x and y at a pair of nodes, written as sums of (mean quantity) x
+// (deviation) so that FP32 rounding is relative to |d|:
 //   dv = (dm rhobar - mbar drho) / (rho rhobar),
 //   dE - dK = (dE rhobar - dm . mbar / 2) / rhobar - (mbar + dm) . dv / 2,
 //   dp = (g - 1)(dE - dK),  dH = dE + dp.
 // The two differences that cancel exactly in uniform flow (dv for a uniform velocity,
 // dE - dK for a uniform pressure) are formed with compensated products.
-__device__ __forceinline__ void euler_dflux(float g, const EulerMean& M, const float* d, float* dFx, float* dFy) {
-  const float rb = M.U[0];
-  const float ir = rcp_fast(rb * (rb + d[0]));
-  const float dvx = diff_of_products(d[1], rb, M.U[1], d[0]) * ir;
-  const float dvy = diff_of_products(d[2], rb, M.U[2], d[0]) * ir;
+__device__ __forceinline__ void euler_dflux(float g, const EulerMean& M, const f2 (&d)[NV], f2 (&dFx)[NV], f2 (&dFy)[NV]) {
+  const f2 rb = dup2(M.U[0]);
+  const f2 rr = mul2(rb, add2(rb, d[0]));
+  const f2 ir = mk2(rcp_fast(rr.x), rcp_fast(rr.y));
+  const f2 dvx = mul2(diff_of_products(d[1], rb, M.U[1], d[0]), ir);
+  const f2 dvy = mul2(diff_of_products(d[2], rb, M.U[2], d[0]), ir);
   // dE rhobar - (dmx mbarx + dmy mbary) / 2, compensated
-  const float x1 = diff_of_products(d[3], rb, 0.5f * d[1], M.U[1]);
-  const float p2 = 0.5f * d[2] * M.U[2];
-  const float e2 = fmaf(0.5f * d[2], M.U[2], -p2);
-  const float x = (x1 - p2) - e2;
-  const float dEmK = x * M.irho - 0.5f * ((M.U[1] + d[1]) * dvx + (M.U[2] + d[2]) * dvy);
-  const float dp = (g - 1.0f) * dEmK;
-  const float dH = d[3] + dp;
+  const f2 x1 = diff_of_products(d[3], rb, 0.5f * M.U[1], d[1]);
+  const f2 np2 = mul2(dup2(-0.5f * M.U[2]), d[2]);
+  const f2 x = sub2(add2(x1, np2), fma2(dup2(0.5f * M.U[2]), d[2], np2));
+  const f2 m1 = add2(dup2(M.U[1]), d[1]), m2 = add2(dup2(M.U[2]), d[2]);
+  const f2 k = fma2(m1, dvx, mul2(m2, dvy));
+  const f2 dEmK = fma2(dup2(-0.5f), k, mul2(x, dup2(M.irho)));
+  const f2 dp = mul2(dup2(g - 1.0f), dEmK);
+  const f2 dH = add2(d[3], dp), H = add2(dup2(M.H), dH);
+  const f2 vx = dup2(M.vx), vy = dup2(M.vy);
   dFx[0] = d[1];
-  dFx[1] = M.U[1] * dvx + d[1] * M.vx + d[1] * dvx + dp;
-  dFx[2] = M.U[2] * dvx + d[2] * M.vx + d[2] * dvx;
-  dFx[3] = M.H * dvx + dH * M.vx + dH * dvx;
+  dFx[1] = add2(fma2(m1, dvx, mul2(d[1], vx)), dp);
+  dFx[2] = fma2(m2, dvx, mul2(d[2], vx));
+  dFx[3] = fma2(H, dvx, mul2(dH, vx));
   dFy[0] = d[2];
-  dFy[1] = M.U[1] * dvy + d[1] * M.vy + d[1] * dvy;
-  dFy[2] = M.U[2] * dvy + d[2] * M.vy + d[2] * dvy + dp;
-  dFy[3] = M.H * dvy + dH * M.vy + dH * dvy;
+  dFy[1] = fma2(m1, dvy, mul2(d[1], vy));
+  dFy[2] = add2(fma2(m2, dvy, mul2(d[2], vy)), dp);
+  dFy[3] = fma2(H, dvy, mul2(dH, vy));
 }
 
-__device__ __forceinline__ float euler_pressure(float g, const float* U) {
-  return (g - 1.0f) * (U[3] - 0.5f * (U[1] * U[1] + U[2] * U[2]) / U[0]);
-}
-
-// |v| + c at a node of full state U, with the velocity along x (dir 0) or y (dir 1) and
-// the sound speed c; flags non-positive density or pressure
-__device__ __forceinline__ float euler_wave(float g, const float* U, int dir, float& vn, float& c, bool& bad) {
-  const float rho = U[0], ir = rcp_fast(rho);
-  const float vx = U[1] * ir, vy = U[2] * ir;
-  const float p = (g - 1.0f) * (U[3] - 0.5f * (U[1] * vx + U[2] * vy));
-  bad |= !(rho > 0.0f) || !(p > 0.0f);
-  c = sqrt_fast(g * fmaxf(p, 0.0f) * fabsf(ir));
+// |v| + c at a pair of nodes of full state U, with the velocity along x (dir 0) or y (dir 1)
+// and the sound speed c; flags non-positive density or pressure
+__device__ __forceinline__ float euler_wave(float g, const f2 (&U)[NV], int dir, f2& vn, f2& c, bool& bad) {
+  const f2 ir = mk2(rcp_fast(U[0].x), rcp_fast(U[0].y));
+  const f2 vx = mul2(U[1], ir), vy = mul2(U[2], ir);
+  const f2 p = mul2(dup2(g - 1.0f), fma2(dup2(-0.5f), fma2(U[1], vx, mul2(U[2], vy)), U[3]));
+  bad |= !(U[0].x > 0.0f) || !(U[0].y > 0.0f) || !(p.x > 0.0f) || !(p.y > 0.0f);
+  c = mk2(sqrt_fast(g * fmaxf(p.x, 0.0f) * fabsf(ir.x)), sqrt_fast(g * fmaxf(p.y, 0.0f) * fabsf(ir.y)));
   vn = dir == 0 ? vx : vy;
-  return sqrt_fast(vx * vx + vy * vy) + c;
+  const f2 v2 = fma2(vx, vx, mul2(vy, vy));
+  return fmaxf(sqrt_fast(v2.x) + c.x, sqrt_fast(v2.y) + c.y);
 }
 
-// |v| + c at a node of full state U; flags non-positive density or pressure
-__device__ __forceinline__ float euler_speed(float g, const float* U, bool& bad) {
-  float vn, c;
-  return euler_wave(g, U, 0, vn, c, bad);
-}
-
-// HLL flux minus F(Ubar) . n across a face with normal +x (dir 0) or +y (dir 1), from
-// the left/lower state Ubar + dL to the right/upper state Ubar + dR (reading A14), with
-// Davis wave speeds from the two node states' normal velocities vnl, vnr and sound speeds
-// cl, cr (euler_wave).  The constant F(Ubar) drops out of every branch:
+// HLL flux minus F(Ubar) . n across a face with normal +x (dir 0) or +y (dir 1) at a pair of
+// nodes, from the left/lower state Ubar + dL to the right/upper state Ubar + dR (reading
+// A14), with Davis wave speeds from the node states' normal velocities vnl, vnr and sound
+// speeds cl, cr (euler_wave).  The constant F(Ubar) drops out of every branch:
 // (S_R F(Ubar) - S_L F(Ubar)) / (S_R - S_L) = F(Ubar).
-__device__ __forceinline__ void hll_dev(float g, const EulerMean& M, const float* dL, const float* dR, float vnl,
-                                        float cl, float vnr, float cr, int dir, float* F) {
-  const float sl = fminf(vnl - cl, vnr - cr), sr = fmaxf(vnl + cl, vnr + cr);
-  float fxl[NV], fyl[NV], fxr[NV], fyr[NV];
-  euler_dflux(g, M, dL, fxl, fyl);
-  euler_dflux(g, M, dR, fxr, fyr);
-  const float* fl = dir == 0 ? fxl : fyl;
-  const float* fr = dir == 0 ? fxr : fyr;
-  if (sl >= 0.0f) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = fl[v];
-  } else if (sr <= 0.0f) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = fr[v];
+__device__ __forceinline__ void hll_dev(float g, const EulerMean& M, const f2 (&dL)[NV], const f2 (&dR)[NV], f2 vnl, f2 cl,
+                                        f2 vnr, f2 cr, int dir, f2 (&F)[NV]) {
+  const f2 sl = mk2(fminf(vnl.x - cl.x, vnr.x - cr.x), fminf(vnl.y - cl.y, vnr.y - cr.y));
+  const f2 sr = mk2(fmaxf(vnl.x + cl.x, vnr.x + cr.x), fmaxf(vnl.y + cl.y, vnr.y + cr.y));
+  f2 fl[NV], fr[NV], o[NV];
+  if (dir == 0) {
+    euler_dflux(g, M, dL, fl, o);
+    euler_dflux(g, M, dR, fr, o);
   } else {
-    const float inv = rcp_fast(sr - sl);
+    euler_dflux(g, M, dL, o, fl);
+    euler_dflux(g, M, dR, o, fr);
+  }
+  const f2 inv = mk2(rcp_fast(sr.x - sl.x), rcp_fast(sr.y - sl.y));
+  const f2 wl = mul2(sr, inv), wr = mul2(mul2(dup2(-1.0f), sl), inv), wd = mul2(mul2(sl, sr), inv);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = (sr * fl[v] - sl * fr[v] + sl * sr * (dR[v] - dL[v])) * inv;
+  for (int v = 0; v < NV; ++v) {
+    const f2 m = fma2(wl, fl[v], fma2(wr, fr[v], mul2(wd, sub2(dR[v], dL[v]))));
+    F[v] = mk2(sl.x >= 0.0f ? fl[v].x : sr.x <= 0.0f ? fr[v].x : m.x, sl.y >= 0.0f ? fl[v].y : sr.y <= 0.0f ? fr[v].y : m.y);
   }
 }
 
-// Shared-memory layout of the Euler stage tile (floats).
+// Shared-memory layout of the Euler stage tile (floats): four variables' cells, each laid
+// out as the scalar tile's (TileLayout), then the density's vertex data (later the
+// indicator), the node tabulations, the faces' projected fluxes (mode pairs,
+// component-major, so that neighbouring faces lie in neighbouring banks) and the largest
+// wave speed of each side of a face (later the SC factors of the four variables).
 template <int P, int TX, int TY>
 struct EulerLayout {
-  static constexpr int N = P + 1, ND = N * N, NT = TX * TY;
-  static constexpr int HX = TX + 2, HY = TY + 2, NH = HX * HY;
-  static constexpr int NVT = (TX + 1) * (TY + 1);
-  // the tile's faces: x-faces (TX + 1 per tile row), then y-faces (TX per row of TY + 1)
-  static constexpr int NFX = (TX + 1) * TY, NFACE = NFX + TX * (TY + 1);
-  // per face: the projected flux h[v][j] (NV x N), then the largest wave speed of the
-  // left/lower and of the right/upper cell's trace over the face nodes
-  static constexpr int FS = NV * N + 2;
-  static constexpr int OFF_SC = 0;                     // [NV][ND][NH] tile + halo, mode-major
-  static constexpr int OFF_ST = OFF_SC + NV * ND * NH;  // [ND][NVT] density vertex candidates (to the sensor)
-  static constexpr int OFF_NQ = OFF_ST;                 // [ND][NT] pointwise density indicator (after the sensor)
-  static constexpr int OFF_F = OFF_ST + ND * NVT;       // [FS][NFACE] face results, component-major
-  // halo staging of two variables, cell-major (cells of whole 16-byte chunks only), over
-  // the vertex and face regions, which are written after the load
-  static constexpr int OFF_STG = OFF_ST;
-  static constexpr int STG = ND % 4 == 0 ? 2 * NH * ND : 0;
-  static constexpr int FLOATS = OFF_F + FS * NFACE > OFF_STG + STG ? OFF_F + FS * NFACE : OFF_STG + STG;
+  using L = TileLayout<2, P, TX, TY>;
+  static constexpr int NT = L::NT, ND = L::ND, MP = L::MP, NFACE = L::NFACE;
+  static constexpr int VAR = (L::HY * L::RS + 3) / 4 * 4;        // floats of a variable's cells
+  static constexpr int OFF_C = 0;                                // [NV][VAR]
+  static constexpr int OFF_ST = OFF_C + NV * VAR;                // vertex data, then [ND][NT] indicator
+  static constexpr int OFF_IMG = (OFF_ST + imax(L::VS * L::NVT, ND * NT) + 3) / 4 * 4;
+  static constexpr int OFF_F = OFF_IMG + L::Img::FLOATS;         // [NV][MP][NFACE] pairs
+  static constexpr int OFF_LAM = OFF_F + 2 * NV * MP * NFACE;    // [2][NFACE], then [NV][NT]
+  static constexpr int FLOATS = OFF_LAM + imax(2 * NFACE, NV * NT);
   static constexpr size_t BYTES = sizeof(float) * (size_t)FLOATS;
-  static_assert(ND * NT <= ND * NVT, "the indicator must fit over the vertex candidates");
 };
 
-// After the vertex phase, each thread takes its cell's sensor and then a share of the
-// tile's faces, each face once (rolled over faces and nodes): both cells' traces, HLL
-// relative to the left/lower cell's mean, projection onto the tangential modes, and each
-// side's largest wave speed over the face nodes.  Then one thread per cell, ordered so
-// that nothing larger than one row of volume nodes is held at a time:
-//   faces: the four projected fluxes into r (a left/lower face was projected relative to
-//     the neighbour's mean, so the cell adds F(Ubar_nb) - F(Ubar) on the face's mean
-//     mode), lambda_e over the face nodes;
-//   volume pass A (rolled over node rows): flux deviation projected into r, lambda_e
-//     over the volume nodes, and the two sums of stage (d) per variable;
-//   volume pass B, only where the viscosity (1 - gamma_e) nu_e is non-zero: the
-//     alpha-weighted viscous term.
-// Minimum resident CTAs the register allocation must allow, from a sweep on the 512^2
-// quadrants (stage time, ms: p = 2: 0.21 uncapped, 0.20 at 4 CTAs; p = 3: 0.45 uncapped,
-// 0.41 at 3 CTAs; p = 4 (8x8 tiles): 0.97 uncapped, 1.15 at 6 CTAs).
+// Minimum resident CTAs the register allocation must allow, from sweeps (us per step).
+// p = 1, 512^2: 4 CTAs of 160 threads 108.7, 3 CTAs 114, 6 CTAs 114.  p = 2, 512^2: 3 CTAs 321,
+// 2 CTAs 352 (but 5 % faster on meshes of one wave), 4 CTAs 360.  p = 3, 512^2: 2 CTAs at
+// 255 registers 415, 3 CTAs at 168 (spills) 496.  p = 4 (8x8 tiles), 300^2: 2 CTAs 494.
 template <int P, int TX, int TY>
 constexpr int euler_min_ctas() {
-  return P <= 2 ? 4 * (128 / (TX * TY)) : P == 3 ? 3 * (128 / (TX * TY)) : 1;
+  return P == 1 ? 4 : P == 2 ? 3 : 2;
+}
+// Threads of a block: at p = 1 one warp more than the cells, at p = 4 two, to share the
+// vertices and faces; at p = 2 and 3 the extra warp would cost more registers than it saves.
+template <int P, int TX, int TY>
+__host__ __device__ constexpr int euler_threads() {
+  return TX * TY + (P == 1 ? 32 : P == 4 ? 64 : 0);
 }
 
+// One CTA per tile.  Density vertices and faces share the threads, as in the scalar kernel;
+// then one thread per cell, on two-wide FMAs over mode and node pairs (dg_packed.cuh), which
+// took the Q3 stage of 512^2 from 137 M to 63 M warp instructions and the step from 681 to
+// 415 us (Q1 at 256^2 59 -> 39 us, Q2 131 -> 106, Q4 at 128^2 257 -> 127).  Bound by
+// instruction issue (43 %) and latency at 8 warps per SM (255 registers: four variables'
+// residuals and node sums are live together):
+//   faces: the four projected fluxes into r (a left/lower face was projected relative to
+//     the neighbour's mean, so the cell adds F(Ubar_nb) - F(Ubar) on the face's mean mode);
+//   volume pass A (by node groups): flux deviation projected into r, lambda_e over the nodes;
+//   volume pass B, only where the viscosity (1 - gamma_e) nu_e is non-zero: the viscous term.
+// The SC weights of troubled cells (stage d) are taken before that by all threads of the
+// tile, (cell, node group) and (cell, variable) at a time.
 template <int P, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, (euler_min_ctas<P, TX, TY>()))
-    dg_euler_stage(const __grid_constant__ StageArgs a, const __grid_constant__ DgTables<2, P> T) {
-  using Tb = DgTables<2, P>;
-  using L = EulerLayout<P, TX, TY>;
-  constexpr int N = P + 1, ND = Tb::ND, NS = Tb::NS, NC = 4;
-  constexpr int NT = TX * TY;
-  constexpr int HX = TX + 2, NH = HX * (TY + 2);
-  constexpr int VXT = TX + 1, NVT = VXT * (TY + 1);
+__global__ void __launch_bounds__(euler_threads<P, TX, TY>(), (euler_min_ctas<P, TX, TY>()))
+    dg_euler_stage(const __grid_constant__ StageArgs a, const __grid_constant__ PackedTables<2, P> T) {
+  using E = EulerLayout<P, TX, TY>;
+  using L = typename E::L;
+  using Img = PackedImage<2, P>;
+  constexpr int N = L::N, ND = L::ND, MP = L::MP, NG = L::NG, NT = L::NT, NB = euler_threads<P, TX, TY>();
+  constexpr int HX = L::HX, HY = L::HY, NH = L::NH, NFACE = L::NFACE;
   extern __shared__ __align__(16) float smem[];
-  float* sc = smem + L::OFF_SC;
-  float* st = smem + L::OFF_ST;
-  float* sNq = smem + L::OFF_NQ;
+  float* sc = smem + E::OFF_C;
+  float* st = smem + E::OFF_ST;
+  float* sNq = smem + E::OFF_ST;
+  const float* img = smem + E::OFF_IMG;
+  f2* sF = reinterpret_cast<f2*>(smem + E::OFF_F);
+  float* sLam = smem + E::OFF_LAM;
+  float* sAf = smem + E::OFF_LAM;
+  __shared__ int phs[NV][HY];
+  __shared__ int sc_count;
+  __shared__ short sc_cell[NT];
+  if (threadIdx.x == 0) sc_count = 0;
   const int nx = a.nx, ny = a.ny;
   const size_t ncell = (size_t)nx * ny;
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
   const float g = a.gas_gamma;
 
-  // ---- load tile + halo of all variables (asynchronous copies) ---------------------------
-  // Cells of whole 16-byte chunks (Q1, Q3) in a 16-byte-aligned state: 16-byte copies,
-  // two variables at a time, land cell-major in the staging area and are transposed to
-  // the mode-major layout; otherwise 4-byte copies straight into sc.
-  static_assert(L::OFF_STG % 4 == 0, "staging must be 16-byte aligned");
-  if (ND % 4 == 0 && (reinterpret_cast<uintptr_t>(a.u_in) & 15) == 0) {
-    constexpr int NQ4 = ND / 4, NCH = NH * NQ4;
-    float* stg = smem + L::OFF_STG;
-#pragma unroll 1
-    for (int half = 0; half < NV / 2; ++half) {
-      for (int f = threadIdx.x; f < 2 * NCH; f += NT) {
-        const int vv = f / NCH, rem = f - vv * NCH, h = rem / NQ4, q = rem - h * NQ4;
-        const int v = 2 * half + vv, r = h / HX, cc = h - r * HX;
-        int gi = i0 - 1 + cc, gj = j0 - 1 + r;
-        bool ok = true;
-        if (gi < 0 || gi >= nx) {
-          if (a.perx) gi = (gi + nx) % nx; else ok = false;
-        }
-        if (gj < 0 || gj >= ny) {
-          if (a.pery) gj = (gj + ny) % ny; else ok = false;
-        }
-        ok = ok && CVW_SPAN(a.status, ((size_t)v * ncell + (size_t)gj * nx + gi) * ND + 4 * q, 4, a.lim_in);
-        cp_async16z(stg + 4 * f, ok ? a.u_in + ((size_t)v * ncell + (size_t)gj * nx + gi) * ND + 4 * q : a.u_in,
-                    ok ? 16 : 0);
-      }
-      cp_async_wait_all();
-      __syncthreads();
-      for (int f = threadIdx.x; f < 2 * NCH; f += NT) {
-        const int vv = f / NCH, rem = f - vv * NCH, h = rem / NQ4, q = rem - h * NQ4;
-        const float4 x = *reinterpret_cast<const float4*>(stg + 4 * f);
-        float* d = sc + ((2 * half + vv) * ND + 4 * q) * NH + h;
-        d[0] = x.x;
-        d[NH] = x.y;
-        d[2 * NH] = x.z;
-        d[3 * NH] = x.w;
-      }
-      __syncthreads();
+  // ---- load tile + halo of all variables: asynchronous copies in place ---------------------
+  for (int f = threadIdx.x; f < Img::FLOATS / 4; f += NB) cp_async16(smem + E::OFF_IMG + 4 * f, a.pk_img + 4 * f);
+  pdl_wait();  // everything below reads or writes what earlier kernels write
+  const bool aligned = (reinterpret_cast<uintptr_t>(a.u_in) & 15) == 0;
+  // Otherwise the rows of a tile that touches no x boundary are copied by 16-byte chunks, and
+  // the rest (and a state that is not 16-byte aligned) float by float.
+  if (!L::CHUNKED && aligned && i0 > 0 && i0 + TX < nx) {
+    if constexpr (!L::CHUNKED) {
+      stage_rows16_inner<ND, HX, HY, L::RS, NB, NV>(sc, E::VAR, phs[0], a.u_in, (int64_t)ncell * ND, nx, ny, i0 - 1, j0 - 1,
+                                                    a.pery, a.status, CVW_EXTENT(a, lim_in));
     }
   } else {
-  for (int f = threadIdx.x; f < NV * NH * ND; f += NT) {
-    int v = f / (NH * ND);
-    int rem0 = f - v * (NH * ND);
-    int r = rem0 / (HX * ND);
-    int rem = rem0 - r * (HX * ND);
-    int cc = rem / ND;
-    int mm = rem - cc * ND;
-    int gi = i0 - 1 + cc, gj = j0 - 1 + r;
-    bool ok = true;
-    if (gi < 0 || gi >= nx) {
-      if (a.perx) gi = (gi + nx) % nx; else ok = false;
+    // whole 16-byte chunks, or floats where the state is not 16-byte aligned
+    constexpr int NQ4 = ND / 4 > 0 ? ND / 4 : 1;
+    const int per = L::CHUNKED && aligned ? NQ4 : ND;
+    for (int f = threadIdx.x; f < NH * per; f += NB) {
+      const int h = f / per, q = f - h * per, r = h / HX, cc = h - r * HX;
+      int gi = i0 - 1 + cc, gj = j0 - 1 + r;
+      bool in = true;
+      if (gi < 0 || gi >= nx) {
+        if (a.perx) gi = (gi + nx) % nx; else in = false;
+      }
+      if (gj < 0 || gj >= ny) {
+        if (a.pery) gj = (gj + ny) % ny; else in = false;
+      }
+      const size_t src = ((size_t)gj * nx + gi) * ND;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const size_t s = (size_t)v * ncell * ND + src;
+        if (L::CHUNKED && aligned) {
+          const bool ok = in && CVW_SPAN(a.status, s + 4 * q, 4, a.lim_in);
+          cp_async16z(sc + v * E::VAR + (L::cell(phs[v], cc, r) ^ (4 * q)), ok ? a.u_in + s + 4 * q : a.u_in, ok ? 16 : 0);
+        } else {
+          const bool ok = in && CVW_SPAN(a.status, s + q, 1, a.lim_in);
+          const int dst = L::CHUNKED ? (L::cell(phs[v], cc, r) ^ (q & ~3)) + (q & 3) : r * L::RS + cc * ND + q;
+          cp_async4(sc + v * E::VAR + dst, ok ? a.u_in + s + q : a.u_in, ok ? 4 : 0);
+        }
+      }
     }
-    if (gj < 0 || gj >= ny) {
-      if (a.pery) gj = (gj + ny) % ny; else ok = false;
-    }
-    ok = ok && CVW_SPAN(a.status, ((size_t)v * ncell + (size_t)gj * nx + gi) * ND + mm, 1, a.lim_in);
-    cp_async4(sc + (v * ND + mm) * NH + r * HX + cc,
-              ok ? a.u_in + ((size_t)v * ncell + (size_t)gj * nx + gi) * ND + mm : a.u_in, ok ? 4 : 0);
+    for (int r = threadIdx.x; r < NV * HY; r += NB) (&phs[0][0])[r] = 0;
   }
   cp_async_wait_all();
   __syncthreads();
-  }
 
   // ---- (a)+(b): density vertex candidates ---------------------------------------------------
-  const int act_x = min(TX, nx - i0), act_y = min(TY, ny - j0);
-  for (int vtx = threadIdx.x; vtx < NVT; vtx += NT) {
-    int va = vtx % VXT, vb = vtx / VXT;
-    if (va > act_x || vb > act_y) continue;
-    float acc[ND];
-#pragma unroll
-    for (int k = 0; k < ND; ++k) acc[k] = 0.0f;
-    float wsum = 0.0f;
-    const int gi_w = i0 - 1 + va, gj_s = j0 - 1 + vb;
-    const bool has_w = a.perx || gi_w >= 0, has_e = a.perx || gi_w + 1 < nx;
-    const bool has_s = a.pery || gj_s >= 0, has_n = a.pery || gj_s + 1 < ny;
-    const float* base = sc + vb * HX + va;
-    // slots SW, SE, NW, NE (density block only)
-#pragma unroll 1
-    for (int s = 0; s < NC; ++s) {
-      const int ex = s & 1, ey = (s >> 1) & 1;
-      if (!((ex ? has_e : has_w) && (ey ? has_n : has_s))) continue;
-      float t[ND];
-      corner_taylor<2, P>(T, base + ex + ey * HX, NH, ex ? -1.0f : 1.0f, ey ? -1.0f : 1.0f, t);
-      float b2 = 0.0f;
-#pragma unroll
-      for (int k = 1; k < ND; ++k) b2 = fmaf(T.sigma[k] * t[k], t[k], b2);
-      const float wt = rcp_fast(ipowf(a.eps + powq(sqrt_fast(b2), a.q), a.r));
-      wsum += wt;
-#pragma unroll
-      for (int k = 0; k < ND; ++k) acc[k] = fmaf(wt, t[k], acc[k]);
-    }
-    const float inv = rcp_fast(wsum);
-#pragma unroll
-    for (int k = 0; k < ND; ++k) st[k * NVT + vtx] = acc[k] * inv;
-    if (a.tstar_out) {
-      int I = i0 + va, J = j0 + vb;
-      int vyn = a.pery ? ny : ny + 1;
-      if ((va < TX || I == nx) && I < a.vx && (vb < TY || J == ny) && J < vyn) {
-        size_t vi = (size_t)I + (size_t)a.vx * J;
-#pragma unroll
-        for (int k = 0; k < ND; ++k) a.tstar_out[vi * ND + k] = acc[k] * inv * T.tscale[k];
-      }
-    }
-  }
+  tile_vertex_phase<2, P, TX, TY, NB>(a, T, sc, phs[0], st, i0, j0, nx, ny);
 
-  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-  const int gi = i0 + tx, gj = j0 + ty;
-  const int hc = (ty + 1) * HX + tx + 1;
-  const size_t cell = (size_t)gj * nx + gi;
-  // (the checked build also checks the cell's index in the per-cell outputs and its span of
-  // u_n and u_out in the last variable)
-  const bool active = gi < nx && gj < ny && CVW_SPAN(a.status, cell, 1, a.lim_cell) &&
-                      CVW_SPAN(a.status, ((size_t)(NV - 1) * ncell + cell) * ND, ND,
-                               a.lim_in < a.lim_out ? a.lim_in : a.lim_out);
-  auto C = [&](int v, int m, int h) -> float { return sc[(v * ND + m) * NH + h]; };
   const bool sensor_only = (a.mode & kModeSensorOnly) != 0;
+  const bool rk = (a.mode & kModeRK) != 0, with_un = rk && a.rk_a != 0.0f;
+  const int act_x = min(TX, nx - i0), act_y = min(TY, ny - j0);
   bool bad = false;
 
   // ---- the tile's faces, each once: traces, HLL, projection, each side's wave speed --------------
-  // In the vertex phase's barrier interval (the face results do not overlap the vertex
-  // candidates), from the block's last thread backwards: the vertex phase's extra round
-  // falls on the first threads, the face phase's on the last.
-  float* sF = smem + L::OFF_F;
+  // In the vertex phase's barrier interval, from the block's last thread backwards: the
+  // vertex phase's extra round falls on the first threads, the face phase's on the last.
 #pragma unroll 1
-  for (int f = NT - 1 - threadIdx.x; f < L::NFACE; f += NT) {
-    int dirn, hl, hr;
+  for (int f = NB - 1 - threadIdx.x; f < NFACE; f += NB) {
+    int dirn, hx, hy;
     bool hasl, hasr, needed;
     if (f < L::NFX) {
-      const int row = f / (TX + 1), col = f - row * (TX + 1);
-      hl = (row + 1) * HX + col;
-      hr = hl + 1;
-      dirn = 0;
-      const int gl = i0 - 1 + col;
+      hy = f / (TX + 1), hx = f - hy * (TX + 1);
+      needed = hy < act_y && hx <= act_x;  // a side of an active cell
+      const int gl = i0 - 1 + hx;
       hasl = a.perx || gl >= 0;
       hasr = a.perx || gl + 1 < nx;
-      needed = row < act_y && col <= act_x;  // a side of an active cell
+      ++hy;
+      dirn = 0;
     } else {
-      const int h = f - L::NFX, row = h / TX, col = h - row * TX;
-      hl = row * HX + col + 1;
-      hr = hl + HX;
-      dirn = 1;
-      const int gl = j0 - 1 + row;
+      const int q = f - L::NFX;
+      hy = q / TX, hx = q - hy * TX;
+      needed = hx < act_x && hy <= act_y;
+      ++hx;
+      const int gl = j0 - 1 + hy;
       hasl = a.pery || gl >= 0;
       hasr = a.pery || gl + 1 < ny;
-      needed = col < act_x && row <= act_y;
+      dirn = 1;
     }
     if (!needed) continue;
-    // tangential trace coefficients (non-mean modes): the left/lower cell meets the face
+    // tangential traces (non-mean modes) as mode pairs: the left/lower cell meets the face
     // with its upper side (+1), the right/upper cell with its lower side ((-1)^i along the
     // normal); a missing side (transmissive boundary) is the other side's ghost
-    float tl[NV][N], tr[NV][N], UL[NV], UR[NV];
+    f2 tr[2][NV][MP];
+    float um[2][NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
+    for (int side = 0; side < 2; ++side) {
+      const float sg = side ? -1.0f : 1.0f;
+      const int cx = hx + (dirn == 0 ? side : 0), cy = hy + (dirn == 1 ? side : 0);
 #pragma unroll
-      for (int j = 0; j < N; ++j) {
-        float sl = 0.0f, sr = 0.0f;
+      for (int v = 0; v < NV; ++v) {
+        f2 c[N][MP];
+        load_cell<L>(sc + v * E::VAR, L::cell(phs[v], cx, cy), c);
+        um[side][v] = c[0][0].x;
+        c[0][0].x = 0.0f;
+        if (dirn == 0) {
+          float d[2 * MP];
+          d[2 * MP - 1] = 0.0f;
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-          const int m = dirn == 0 ? i + N * j : j + N * i;
-          if (m == 0) continue;
-          const float cl = C(v, m, hl), cr = C(v, m, hr);
-          sl += cl;
-          sr += (i & 1) ? -cr : cr;
+          for (int my = 0; my < N; ++my) {
+            f2 s = c[my][0];
+#pragma unroll
+            for (int p = 1; p < MP; ++p) s = add2(s, c[my][p]);
+            d[my] = fmaf(sg, s.y, s.x);
+          }
+#pragma unroll
+          for (int p = 0; p < MP; ++p) tr[side][v][p] = mk2(d[2 * p], d[2 * p + 1]);
+        } else {
+#pragma unroll
+          for (int p = 0; p < MP; ++p) {
+            f2 e = c[0][p], o = c[1][p];
+#pragma unroll
+            for (int my = 2; my < N; ++my) {
+              if (my & 1) o = add2(o, c[my][p]);
+              else e = add2(e, c[my][p]);
+            }
+            tr[side][v][p] = fma2(dup2(sg), o, e);
+          }
         }
-        tl[v][j] = sl;
-        tr[v][j] = sr;
       }
-      UL[v] = C(v, 0, hl);
-      UR[v] = C(v, 0, hr);
     }
-    if (!hasl) {
+    if (!hasl || !hasr) {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        UL[v] = UR[v];
+        um[0][v] = hasl ? um[0][v] : um[1][v];
+        um[1][v] = hasr ? um[1][v] : um[0][v];
 #pragma unroll
-        for (int j = 0; j < N; ++j) tl[v][j] = tr[v][j];
+        for (int p = 0; p < MP; ++p) {
+          tr[0][v][p] = hasl ? tr[0][v][p] : tr[1][v][p];
+          tr[1][v][p] = hasr ? tr[1][v][p] : tr[0][v][p];
+        }
       }
     }
-    if (!hasr) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        UR[v] = UL[v];
-#pragma unroll
-        for (int j = 0; j < N; ++j) tr[v][j] = tl[v][j];
-      }
-    }
-    const EulerMean ML = euler_mean(g, UL);
-    float dm[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) dm[v] = UR[v] - UL[v];
-    float h[NV][N];
+    const EulerMean ML = euler_mean(g, um[0]);
+    f2 h[NV][MP];
 #pragma unroll
     for (int v = 0; v < NV; ++v)
 #pragma unroll
-      for (int j = 0; j < N; ++j) h[v][j] = 0.0f;
+      for (int p = 0; p < MP; ++p) h[v][p] = mk2(0.0f, 0.0f);
     float laml = 0.0f, lamr = 0.0f;
 #pragma unroll 1
-    for (int q = 0; q < N; ++q) {
-      float dL[NV], dR[NV];
+    for (int q = 0; q < NG; ++q) {
+      f2 b[MP], dL[NV], dR[NV], U[NV];
+      load_pairs<MP>(img + Img::BX + 2 * MP * q, b);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        float sl = 0.0f, sr = 0.0f;
+        f2 sl = mul2(b[0], tr[0][v][0]), sr = mul2(b[0], tr[1][v][0]);
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-          const float bq = T.B[q][j];
-          sl = fmaf(bq, tl[v][j], sl);
-          sr = fmaf(bq, tr[v][j], sr);
+        for (int p = 1; p < MP; ++p) {
+          sl = fma2(b[p], tr[0][v][p], sl);
+          sr = fma2(b[p], tr[1][v][p], sr);
         }
-        dL[v] = sl;
-        dR[v] = sr;
+        dL[v] = mk2(sl.x + sl.y, sl.x - sl.y);
+        dR[v] = mk2(sr.x + sr.y, sr.x - sr.y);
       }
-      float vnl, cl, vnr, cr;
-      {
-        float U[NV];
+      f2 vnl, cl, vnr, cr;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) U[v] = UL[v] + dL[v];
-        laml = fmaxf(laml, euler_wave(g, U, dirn, vnl, cl, bad));
+      for (int v = 0; v < NV; ++v) U[v] = add2(dup2(um[0][v]), dL[v]);
+      laml = fmaxf(laml, euler_wave(g, U, dirn, vnl, cl, bad));
 #pragma unroll
-        for (int v = 0; v < NV; ++v) U[v] = UR[v] + dR[v];
-        lamr = fmaxf(lamr, euler_wave(g, U, dirn, vnr, cr, bad));
-      }
+      for (int v = 0; v < NV; ++v) U[v] = add2(dup2(um[1][v]), dR[v]);
+      lamr = fmaxf(lamr, euler_wave(g, U, dirn, vnr, cr, bad));
       if (sensor_only) continue;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) dR[v] = dm[v] + dR[v];
-      float F[NV];
+      for (int v = 0; v < NV; ++v) dR[v] = add2(dup2(um[1][v] - um[0][v]), dR[v]);
+      f2 F[NV];
       hll_dev(g, ML, dL, dR, vnl, cl, vnr, cr, dirn, F);
+      const float w = img[Img::WX + q];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const float wf = T.w[q] * F[v];
+        const f2 sd = mul2(dup2(w), mk2(F[v].x + F[v].y, F[v].x - F[v].y));
 #pragma unroll
-        for (int j = 0; j < N; ++j) h[v][j] = fmaf(wf, T.B[q][j], h[v][j]);
+        for (int p = 0; p < MP; ++p) h[v][p] = fma2(b[p], sd, h[v][p]);
       }
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v)
 #pragma unroll
-      for (int j = 0; j < N; ++j) sF[(v * N + j) * L::NFACE + f] = h[v][j];
-    sF[NV * N * L::NFACE + f] = laml;
-    sF[(NV * N + 1) * L::NFACE + f] = lamr;
+      for (int p = 0; p < MP; ++p) sF[(v * MP + p) * NFACE + f] = h[v][p];
+    sLam[f] = laml;
+    sLam[NFACE + f] = lamr;
   }
   __syncthreads();
+  pdl_launch_dependents();
 
-  // ---- (c) sensor from the density -------------------------------------------------------
-  float gam = 1.0f, n0 = 0.0f;
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  const int gi = i0 + tx, gj = j0 + ty;
+  const size_t cell = (size_t)gj * nx + gi;
+  // (the checked build also checks the cell's index in the per-cell outputs and its span of
+  // u_n and u_out in the last variable)
+  const bool active = (NB == NT || threadIdx.x < NT) && gi < nx && gj < ny && CVW_SPAN(a.status, cell, 1, a.lim_cell) &&
+                      CVW_SPAN(a.status, ((size_t)(NV - 1) * ncell + cell) * ND, ND,
+                               a.lim_in < a.lim_out ? a.lim_in : a.lim_out);
+  // ---- (c) sensor from the density; lambda_e over the face nodes -------------------------------
+  float gam = 1.0f, n0 = 0.0f, lam = 0.0f;
   if (active) {
-    float c[ND];
+    f2 c[N][MP], S[N][MP];
+    load_cell<L>(sc, L::cell(phs[0], tx + 1, ty + 1), c);
+    gam = cell_sensor<2, P, TX, TY>(a, T, st, c, tx, ty, n0, S);
 #pragma unroll
-    for (int m = 0; m < ND; ++m) c[m] = C(0, m, hc);
-    float w0[NS];
+    for (int k = 0; k < 4; ++k) lam = fmaxf(lam, sLam[((k & 1) ? NFACE : 0) + cell_face<L, TX>(k, tx, ty)]);
+  }
+
+  // ---- (d) troubled cells: the density's pointwise indicator Nq at the volume nodes, then each
+  // variable's factor afac = sum w g / sum w Nq g, g = |grad u_v|^2 (alpha_{v,q} = Nq[q] afac[v];
+  // alpha = 1 where afac < 0).  The tile's threads share the troubled cells' work.
+  bool troubled = false, need_sc = false;
+  float afac[NV];
+  // mean deviations of the left (first half) and lower neighbour, zero where there is none
+  // (after this stage a cell's slot is its thread's own)
+  f2 dn[NV];
 #pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      float acc = 0.0f;
+  for (int v = 0; v < NV; ++v) {
+    const float m = active ? sc[v * E::VAR + L::cell(phs[v], tx + 1, ty + 1)] : 0.0f;
+    dn[v] = mk2(active && (a.perx || gi > 0) ? sc[v * E::VAR + L::cell(phs[v], tx, ty + 1)] - m : 0.0f,
+                active && (a.pery || gj > 0) ? sc[v * E::VAR + L::cell(phs[v], tx + 1, ty)] - m : 0.0f);
+  }
 #pragma unroll
-      for (int j = i; j < NS; ++j) acc = fmaf(T.R[i][j], c[j + 1], acc);
-      w0[i] = acc;
-    }
-    float n0sq = 0.0f;
-#pragma unroll
-    for (int i = 0; i < NS; ++i) n0sq = fmaf(w0[i], w0[i], n0sq);
-    n0 = sqrt_fast(n0sq);
-    const float om0 = (1.0f - NC * a.gamma_vertex) * rcp_fast(ipowf(a.eps + powq(n0, a.q), a.r));
-    float S[NS];
-#pragma unroll
-    for (int i = 0; i < NS; ++i) S[i] = om0 * w0[i];
-    float osum = om0;
-#pragma unroll
-    for (int l = 0; l < NC; ++l) {
-      const int vi = (tx + (l & 1)) + (ty + ((l >> 1) & 1)) * VXT;
-      float tl[NS];
-#pragma unroll
-      for (int k = 0; k < NS; ++k) tl[k] = st[(k + 1) * NVT + vi];
-      float wl[NS];
-      float b2 = 0.0f;
-#pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int j = 0; j < NS; ++j) acc = fmaf(T.A[l][i][j], tl[j], acc);
-        wl[i] = acc;
-        b2 = fmaf(acc, acc, b2);
+  for (int v = 0; v < NV; ++v) afac[v] = -1.0f;
+  if (!sensor_only) {
+    if (active) {
+      troubled = a.sc && gam < a.c_gamma && n0 > 1e-30f;
+      if (a.troubled_override) {
+        const int ov = a.troubled_override[cell];
+        if (ov >= 0) troubled = ov && n0 > 1e-30f;
       }
-      const float om = a.gamma_vertex * rcp_fast(ipowf(a.eps + powq(sqrt_fast(b2), a.q), a.r));
-      osum += om;
-#pragma unroll
-      for (int i = 0; i < NS; ++i) S[i] = fmaf(om, wl[i], S[i]);
     }
-    const float inv = rcp_fast(osum);
-    float d2 = 0.0f;
+    need_sc = troubled && gam < 1.0f;
+    if (need_sc) sc_cell[atomicAdd(&sc_count, 1)] = (short)threadIdx.x;
+    if (__syncthreads_or(need_sc)) {
+      const int n = sc_count;
+#pragma unroll 1
+      for (int t = threadIdx.x; t < n * L::NGG; t += NB) {
+        const int gh = t / n, id = sc_cell[t - gh * n];
+        f2 s1, s2;
+        sc_node_group<2, P, TX, TY>(a, T, img, sNq, sc, phs[0], id, gh / NG, gh % NG, s1, s2);
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int t = threadIdx.x; t < n * NV; t += NB) {
+        const int v = t / n, id = sc_cell[t - v * n];
+        f2 c[N][MP], s1 = mk2(0.0f, 0.0f), s2 = s1;
+        load_cell<L>(sc + v * E::VAR, L::cell(phs[v], id % TX + 1, id / TX + 1), c);
+        c[0][0].x = 0.0f;
+#pragma unroll 1
+        for (int q = 0; q < NG; ++q) {
+          f2 b[MP], d[MP], tb[N], td[N];
+          load_pairs<MP>(img + Img::BX + 2 * MP * q, b);
+          load_pairs<MP>(img + Img::DX + 2 * MP * q, d);
 #pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      float df = w0[i] - S[i] * inv;
-      d2 = fmaf(df, df, d2);
+          for (int my = 0; my < N; ++my) {
+            f2 s = mul2(b[0], c[my][0]), sd = mul2(d[0], c[my][0]);
+#pragma unroll
+            for (int p = 1; p < MP; ++p) {
+              s = fma2(b[p], c[my][p], s);
+              sd = fma2(d[p], c[my][p], sd);
+            }
+            tb[my] = mk2(s.x + s.y, s.x - s.y);
+            td[my] = mk2(sd.x + sd.y, sd.y - sd.x);
+          }
+#pragma unroll 1
+          for (int h = 0; h < NG; ++h) {
+            f2 ua, ub, va, vb;
+            node_gradient<N, MP>(img + Img::BY + 2 * N * h, img + Img::DY + 2 * N * h, tb, td, ua, ub, va, vb);
+            const f2 kx = dup2(a.two_dx * a.two_dx), ky = dup2(a.two_dy * a.two_dy);
+            const f2 qa = fma2(kx, mul2(ua, ua), mul2(ky, mul2(va, va)));
+            const f2 qb = fma2(kx, mul2(ub, ub), mul2(ky, mul2(vb, vb)));
+            const f2 w = dup2(img[Img::WX + q] * img[Img::WY + h]);
+            const float* ra = sNq + N * h * NT + id;
+            s1 = fma2(w, qa, s1);
+            s2 = fma2(mul2(w, mk2(ra[q * NT], ra[(N - 1 - q) * NT])), qa, s2);
+            if (2 * h != N - 1) {
+              const float* rb = sNq + N * (N - 1 - h) * NT + id;
+              s1 = fma2(w, qb, s1);
+              s2 = fma2(mul2(w, mk2(rb[q * NT], rb[(N - 1 - q) * NT])), qb, s2);
+            }
+          }
+        }
+        const float t2 = s2.x + s2.y;
+        sAf[v * NT + id] = t2 > 0.0f ? (s1.x + s1.y) / t2 : -1.0f;
+      }
+      __syncthreads();
+      if (need_sc) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) afac[v] = sAf[v * NT + threadIdx.x];
+      }
     }
-    if (a.sensor_mode == CVWENO_SENSOR_SMOOTH)
-      gam = 1.0f;
-    else if (a.sensor_mode == CVWENO_SENSOR_TROUBLED)
-      gam = 0.0f;
-    else if (n0 <= 1e-30f)
-      gam = 1.0f;
-    else
-      gam = 1.0f - powq(fminf(1.0f, sqrt_fast(d2) * rcp_fast(n0)), a.q);
   }
+  if (active) {
 
-  // the indicator sNq, written below, lies over the vertex candidates that the sensor reads
-  __syncthreads();
-  if (!active) {
-    if (bad) atomicOr(a.status, kStatPositivity);
-    return;
-  }
-
-  // ---- faces into the residual: right, left, top, bottom; lambda_e over the face nodes ---------
+  // ---- faces into the residual: right, left, top, bottom ---------------------------------------
+  int hc[NV];
   float Ubar[NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) Ubar[v] = C(v, 0, hc);
+  for (int v = 0; v < NV; ++v) {
+    hc[v] = v * E::VAR + L::cell(phs[v], tx + 1, ty + 1);
+    Ubar[v] = sc[hc[v]];
+  }
   const EulerMean M = euler_mean(g, Ubar);
-  float r[NV][ND];
+  f2 r[NV][N][MP];
+  if (!sensor_only) {
+    // the lower faces' F(Ubar_nb) - F(Ubar), twice (its projection on the face's mean mode)
+    f2 nx2[NV], ny2[NV];
+    euler_dflux(g, M, dn, nx2, ny2);
+    const int fR = cell_face<L, TX>(0, tx, ty), fL = cell_face<L, TX>(1, tx, ty), fT = cell_face<L, TX>(2, tx, ty),
+              fB = cell_face<L, TX>(3, tx, ty);
 #pragma unroll
-  for (int v = 0; v < NV; ++v)
+    for (int v = 0; v < NV; ++v) {
+      // r[mx,my] = -2/dx (hR[my] - (-1)^mx hL[my]) - 2/dy (hT[mx] - (-1)^my hB[mx])
+      f2 ve[MP], vo[MP], hr[MP], hl[MP];
 #pragma unroll
-    for (int m = 0; m < ND; ++m) r[v][m] = 0.0f;
-  float lam = 0.0f;
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    const int dirn = k >> 1;
-    const bool upper = (k & 1) == 0;  // this cell is the face's left/lower cell
-    const int f = dirn == 0 ? ty * (TX + 1) + tx + (upper ? 1 : 0) : L::NFX + (ty + (upper ? 1 : 0)) * TX + tx;
-    lam = fmaxf(lam, sF[(NV * N + (upper ? 0 : 1)) * L::NFACE + f]);
-    if (sensor_only) continue;
-    float h[NV][N];
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int j = 0; j < N; ++j) h[v][j] = sF[(v * N + j) * L::NFACE + f];
-    const bool nb = dirn == 0 ? (a.perx || gi > 0) : (a.pery || gj > 0);
-    if (!upper && nb) {
-      // projected relative to the neighbour's mean: F - F(Ubar) = (F - F(Ubar_nb)) + D with
-      // D = F(Ubar_nb) - F(Ubar) constant along the face, whose projection is 2 D on mode 0
-      float d[NV], dFx[NV], dFy[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) d[v] = C(v, 0, hc - (dirn == 0 ? 1 : HX)) - Ubar[v];
-      euler_dflux(g, M, d, dFx, dFy);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) h[v][0] = fmaf(2.0f, dirn == 0 ? dFx[v] : dFy[v], h[v][0]);
-    }
-    // r[mx,my] -= 2/dx (hR[my] - (-1)^mx hL[my]) + 2/dy (hT[mx] - (-1)^my hB[mx])
-    const float s2d = dirn == 0 ? a.two_dx : a.two_dy;
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int my = 0; my < N; ++my)
-#pragma unroll
-        for (int mx = 0; mx < N; ++mx) {
-          const int nrm = dirn == 0 ? mx : my;
-          const float hv = dirn == 0 ? h[v][my] : h[v][mx];
-          r[v][mx + N * my] = upper ? fmaf(-s2d, hv, r[v][mx + N * my])
-                                    : fmaf(s2d, (nrm & 1) ? -hv : hv, r[v][mx + N * my]);
+      for (int p = 0; p < MP; ++p) {
+        const f2* row = sF + (v * MP + p) * NFACE;
+        f2 top = row[fT], bot = row[fB];
+        hr[p] = row[fR];
+        hl[p] = row[fL];
+        if (p == 0) {
+          hl[0].x = fmaf(2.0f, nx2[v].x, hl[0].x);
+          bot.x = fmaf(2.0f, ny2[v].y, bot.x);
         }
-  }
-
-  // ---- troubled cells: the density's pointwise indicator Nq at the volume nodes -------------
-  bool troubled = a.sc && gam < a.c_gamma && n0 > 1e-30f;
-  if (!sensor_only && a.troubled_override) {
-    const int ov = a.troubled_override[cell];
-    if (ov >= 0) troubled = ov && n0 > 1e-30f;
-  }
-  const bool need_sc = !sensor_only && troubled && gam < 1.0f;
-  if (need_sc) {
-#pragma unroll 1
-    for (int qx = 0; qx < N; ++qx) {
-      float X[N][N];
-#pragma unroll
-      for (int kx = 0; kx < N; ++kx)
-#pragma unroll
-        for (int my = 0; my < N; ++my) {
-          float acc = 0.0f;
-#pragma unroll
-          for (int mx = 0; mx < N; ++mx) acc = fmaf(T.Bk[kx][qx][mx], C(0, mx + N * my, hc), acc);
-          X[kx][my] = acc;
-        }
-#pragma unroll 1
-      for (int qy = 0; qy < N; ++qy) {
-        float s2 = 0.0f;
-#pragma unroll
-        for (int ky = 0; ky < N; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < N; ++kx) {
-            if (kx + ky == 0) continue;
-            float d = 0.0f;
-#pragma unroll
-            for (int my = 0; my < N; ++my) d = fmaf(T.Bk[ky][qy][my], X[kx][my], d);
-            s2 = fmaf(T.sigma[kx + N * ky] * d, d, s2);
-          }
-        sNq[(qx + N * qy) * NT + threadIdx.x] = sqrtf(s2);
+        ve[p] = mul2(dup2(a.two_dy), sub2(bot, top));
+        vo[p] = mul2(dup2(-a.two_dy), add2(bot, top));
       }
-    }
-  }
-
-  // ---- volume pass A: flux deviation into r, lambda_e, the sums of stage (d) ----------------
-  float s1[NV], s2[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) s1[v] = s2[v] = 0.0f;
-#pragma unroll 1
-  for (int qx = 0; qx < N; ++qx) {
-    float tb[NV][N], td[NV][N];
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
 #pragma unroll
       for (int my = 0; my < N; ++my) {
-        float s0 = 0.0f, sd = 0.0f;
+        const float R = (my & 1) ? hr[my / 2].y : hr[my / 2].x, Lf = (my & 1) ? hl[my / 2].y : hl[my / 2].x;
+        const f2 x = mk2(-a.two_dx * (R - Lf), -a.two_dx * (R + Lf));
 #pragma unroll
-        for (int mx = 0; mx < N; ++mx) {
-          const float cm = (mx + N * my) ? C(v, mx + N * my, hc) : 0.0f;  // deviation: no mean mode
-          s0 = fmaf(T.B[qx][mx], cm, s0);
-          sd = fmaf(T.Bd[qx][mx], cm, sd);
-        }
-        tb[v][my] = s0;
-        td[v][my] = sd;
+        for (int p = 0; p < MP; ++p) r[v][my][p] = add2(x, (my & 1) ? vo[p] : ve[p]);
       }
-    float hx[NV][N], hy[NV][N];
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int my = 0; my < N; ++my) hx[v][my] = hy[v][my] = 0.0f;
+    }
+  }
+
+  // ---- volume pass A: flux deviation into r, lambda_e over the nodes -------------------------------
 #pragma unroll 1
-    for (int qy = 0; qy < N; ++qy) {
-      const int q = qx + N * qy;
-      const float W = T.w[qx] * T.w[qy];
-      float dU[NV];
-      const float nq = need_sc ? sNq[q * NT + threadIdx.x] : 0.0f;
+  for (int q = 0; q < NG; ++q) {
+    f2 b[MP], tb[NV][N], hx[NV][N], hy[NV][N];
+    load_pairs<MP>(img + Img::BX + 2 * MP * q, b);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        float u = 0.0f, ux = 0.0f, uy = 0.0f;
+    for (int v = 0; v < NV; ++v) {
+      f2 c[N][MP];
+      load_cell<L>(sc, hc[v], c);
+      c[0][0].x = 0.0f;  // deviation: no mean mode
 #pragma unroll
-        for (int my = 0; my < N; ++my) {
-          const float bq = T.B[qy][my];
-          u = fmaf(bq, tb[v][my], u);
-          ux = fmaf(bq, td[v][my], ux);
-          uy = fmaf(T.Bd[qy][my], tb[v][my], uy);
-        }
-        dU[v] = u;
-        if (need_sc) {
-          ux *= a.two_dx;
-          uy *= a.two_dy;
-          const float gsq = fmaf(ux, ux, uy * uy);
-          s1[v] = fmaf(W, gsq, s1[v]);
-          s2[v] = fmaf(W * nq, gsq, s2[v]);
+      for (int my = 0; my < N; ++my) {
+        f2 s = mul2(b[0], c[my][0]);
+#pragma unroll
+        for (int p = 1; p < MP; ++p) s = fma2(b[p], c[my][p], s);
+        tb[v][my] = mk2(s.x + s.y, s.x - s.y);
+        hx[v][my] = hy[v][my] = mk2(0.0f, 0.0f);
+      }
+    }
+#pragma unroll 1
+    for (int h = 0; h < NG; ++h) {
+      const float* yb = img + Img::BY + 2 * N * h;
+      const bool mid = (N & 1) && h == NG - 1;  // the middle row: one row only
+      f2 ua[NV], ub[NV], fx[NV], fy[NV], gx[NV], gy[NV];
+      {
+        f2 by[N];
+        load_pairs<N>(yb, by);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          f2 e = mul2(by[0], tb[v][0]), o = mul2(by[1], tb[v][1]);
+#pragma unroll
+          for (int my = 2; my < N; ++my) {
+            if (my & 1) o = fma2(by[my], tb[v][my], o);
+            else e = fma2(by[my], tb[v][my], e);
+          }
+          ua[v] = add2(e, o);
+          ub[v] = sub2(e, o);
         }
       }
       {
-        float U[NV];
+        f2 U[NV], vn, cs;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) U[v] = Ubar[v] + dU[v];
-        lam = fmaxf(lam, euler_speed(g, U, bad));
+        for (int v = 0; v < NV; ++v) U[v] = add2(dup2(Ubar[v]), ua[v]);
+        lam = fmaxf(lam, euler_wave(g, U, 0, vn, cs, bad));
+        if (!mid) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) U[v] = add2(dup2(Ubar[v]), ub[v]);
+          lam = fmaxf(lam, euler_wave(g, U, 0, vn, cs, bad));
+        }
       }
       if (sensor_only) continue;
-      float Fx[NV], Fy[NV];
-      euler_dflux(g, M, dU, Fx, Fy);
+      euler_dflux(g, M, ua, fx, fy);
 #pragma unroll
-      for (int v = 0; v < NV; ++v)
+      for (int v = 0; v < NV; ++v) gx[v] = gy[v] = mk2(0.0f, 0.0f);
+      if (!mid) euler_dflux(g, M, ub, gx, gy);
+      f2 by[N], dy[N];
+      load_pairs<N>(yb, by);
+      load_pairs<N>(img + Img::DY + 2 * N * h, dy);
+      const f2 w = dup2(img[Img::WY + h]);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const f2 xs = mul2(w, add2(fx[v], gx[v])), xd = mul2(w, sub2(fx[v], gx[v]));
+        const f2 ys = mul2(w, add2(fy[v], gy[v])), yd = mul2(w, sub2(fy[v], gy[v]));
 #pragma unroll
         for (int my = 0; my < N; ++my) {
-          hx[v][my] = fmaf(W * Fx[v], T.B[qy][my], hx[v][my]);
-          hy[v][my] = fmaf(W * Fy[v], T.Bd[qy][my], hy[v][my]);
+          hx[v][my] = fma2(by[my], (my & 1) ? xd : xs, hx[v][my]);
+          if (my > 0) hy[v][my] = fma2(dy[my], (my & 1) ? ys : yd, hy[v][my]);
         }
+      }
     }
     if (sensor_only) continue;
+    f2 d[MP];
+    load_pairs<MP>(img + Img::BX + 2 * MP * q, b);
+    load_pairs<MP>(img + Img::DX + 2 * MP * q, d);
+    const float kx = a.two_dx * img[Img::WX + q], ky = a.two_dy * img[Img::WX + q];
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int my = 0; my < N; ++my)
-#pragma unroll
-        for (int mx = 0; mx < N; ++mx) {
-          float val = r[v][mx + N * my];
-          val = fmaf(a.two_dx * T.Bd[qx][mx], hx[v][my], val);
-          val = fmaf(a.two_dy * T.B[qx][mx], hy[v][my], val);
-          r[v][mx + N * my] = val;
-        }
+    for (int v = 0; v < NV; ++v) project_nodes<N, MP>(b, d, kx, ky, hx[v], hy[v], r[v]);
   }
   const float nu = lam * a.nu_scale;
   if (a.gamma_out) a.gamma_out[cell] = gam;
@@ -679,11 +612,6 @@ __global__ void __launch_bounds__(TX* TY, (euler_min_ctas<P, TX, TY>()))
     if (bad) atomicOr(a.status, kStatPositivity);
     return;
   }
-
-  // ---- (d) SC weights: alpha_{v,q} = Nq[q] afac[v] (afac < 0: alpha = 1) ------------------------
-  float afac[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) afac[v] = (need_sc && s2[v] > 0.0f) ? s1[v] / s2[v] : -1.0f;
   if (a.troubled_out) a.troubled_out[cell] = troubled ? 1 : 0;
   if (a.alpha_out) {
 #pragma unroll 1
@@ -695,149 +623,99 @@ __global__ void __launch_bounds__(TX* TY, (euler_min_ctas<P, TX, TY>()))
   }
 
   // ---- volume pass B: the viscous term, where (1 - gamma_e) nu_e > 0 -----------------------------
-  // With the linear weights (alpha = 1 for every variable) the term is -mu times the
-  // stiffness form of the Legendre basis, which the Gauss rule integrates exactly and which
-  // separates: the x part of mode (mx, my) is (2/dx)^2 (2 / (2 my + 1)) sum_k S[mx][k]
-  // c[k, my], with S[m][k] = int P_m' P_k' = min(m,k) (min(m,k) + 1) where m + k is even
-  // (0 otherwise), and likewise in y.  Alpha-weighted cells take the quadrature.
+  // Where every variable has the linear weights, the stiffness form of the Legendre basis
+  // (add_stiffness); alpha-weighted cells take the quadrature.
   const float mu = (1.0f - gam) * nu;
   bool weighted = false;
 #pragma unroll
   for (int v = 0; v < NV; ++v) weighted |= afac[v] >= 0.0f;
   if (mu > 0.0f && !weighted) {
-    const float kx = -mu * a.two_dx * a.two_dx, ky = -mu * a.two_dy * a.two_dy;
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
+    for (int v = 0; v < NV; ++v) {
+      f2 c[N][MP];
+      load_cell<L>(sc, hc[v], c);
+      c[0][0].x = 0.0f;
+      add_stiffness<2, N, N, MP>(-mu * a.two_dx * a.two_dx, -mu * a.two_dy * a.two_dy, c, r[v]);
+    }
+  } else if (mu > 0.0f) {
+#pragma unroll 1
+    for (int v = 0; v < NV; ++v) {
+      f2 c[N][MP], rv[N][MP];
+      const float af = v == 0 ? afac[0] : v == 1 ? afac[1] : v == 2 ? afac[2] : afac[3];
+      load_cell<L>(sc + v * E::VAR, L::cell(phs[v], tx + 1, ty + 1), c);
+      c[0][0].x = 0.0f;
 #pragma unroll
       for (int my = 0; my < N; ++my)
 #pragma unroll
-        for (int mx = 0; mx < N; ++mx) {
-          if (mx + my == 0) continue;
-          float sx = 0.0f, sy = 0.0f;
-#pragma unroll
-          for (int k = 1; k < N; ++k) {
-            if ((k + mx) % 2 == 0 && mx > 0) {
-              const int mn = mx < k ? mx : k;
-              sx = fmaf((float)(mn * (mn + 1)), C(v, k + N * my, hc), sx);
-            }
-            if ((k + my) % 2 == 0 && my > 0) {
-              const int mn = my < k ? my : k;
-              sy = fmaf((float)(mn * (mn + 1)), C(v, mx + N * k, hc), sy);
-            }
-          }
-          const float val = fmaf(kx * (2.0f / (2 * my + 1)), sx, r[v][mx + N * my]);
-          r[v][mx + N * my] = fmaf(ky * (2.0f / (2 * mx + 1)), sy, val);
-        }
-  } else if (mu > 0.0f) {
+        for (int p = 0; p < MP; ++p) rv[my][p] = mk2(0.0f, 0.0f);
 #pragma unroll 1
-    for (int qx = 0; qx < N; ++qx) {
-      float tb[NV][N], td[NV][N];
+      for (int q = 0; q < NG; ++q)
+        weighted_viscous<N, MP, NT>(a, img, sNq + threadIdx.x, q, -mu * (af >= 0.0f ? af : 1.0f), af >= 0.0f, c, rv);
 #pragma unroll
-      for (int v = 0; v < NV; ++v)
+      for (int w = 0; w < NV; ++w)
+        if (w == v) {
 #pragma unroll
-        for (int my = 0; my < N; ++my) {
-          float s0 = 0.0f, sd = 0.0f;
+          for (int my = 0; my < N; ++my)
 #pragma unroll
-          for (int mx = 0; mx < N; ++mx) {
-            const float cm = (mx + N * my) ? C(v, mx + N * my, hc) : 0.0f;
-            s0 = fmaf(T.B[qx][mx], cm, s0);
-            sd = fmaf(T.Bd[qx][mx], cm, sd);
-          }
-          tb[v][my] = s0;
-          td[v][my] = sd;
+            for (int p = 0; p < MP; ++p) r[w][my][p] = add2(r[w][my][p], rv[my][p]);
         }
-      float hx[NV][N], hy[NV][N];
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int my = 0; my < N; ++my) hx[v][my] = hy[v][my] = 0.0f;
-#pragma unroll 1
-      for (int qy = 0; qy < N; ++qy) {
-        const int q = qx + N * qy;
-        const float W = T.w[qx] * T.w[qy];
-        const float nq = need_sc ? sNq[q * NT + threadIdx.x] : 0.0f;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          float ux = 0.0f, uy = 0.0f;
-#pragma unroll
-          for (int my = 0; my < N; ++my) {
-            ux = fmaf(T.B[qy][my], td[v][my], ux);
-            uy = fmaf(T.Bd[qy][my], tb[v][my], uy);
-          }
-          const float al = afac[v] >= 0.0f ? nq * afac[v] : 1.0f;
-          const float gx = -W * mu * al * a.two_dx * ux, gy = -W * mu * al * a.two_dy * uy;
-#pragma unroll
-          for (int my = 0; my < N; ++my) {
-            hx[v][my] = fmaf(gx, T.B[qy][my], hx[v][my]);
-            hy[v][my] = fmaf(gy, T.Bd[qy][my], hy[v][my]);
-          }
-        }
-      }
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int my = 0; my < N; ++my)
-#pragma unroll
-          for (int mx = 0; mx < N; ++mx) {
-            float val = r[v][mx + N * my];
-            val = fmaf(a.two_dx * T.Bd[qx][mx], hx[v][my], val);
-            val = fmaf(a.two_dy * T.B[qx][mx], hy[v][my], val);
-            r[v][mx + N * my] = val;
-          }
     }
   }
 
-  // ---- M^{-1}, output ---------------------------------------------------------------------------
+  // ---- M^{-1} and the RK combination; cells of whole 16-byte chunks are written here ----------------
   // Per variable, the cell's u_n is read in full before any of its outputs is written: only
   // this thread reads or writes the cell's span, so u_n may alias u_out, and the reads of a
-  // variable go out together instead of one round trip per mode.  16-byte loads and stores
-  // where the cell is whole 16-byte chunks and both states are 16-byte aligned.
-  bool nonfinite = false;
-  const bool rk = (a.mode & kModeRK) != 0, with_un = rk && a.rk_a != 0.0f;
+  // variable go out together.  16-byte loads and stores where both states are 16-byte aligned.
+  f2 fin = mk2(0.0f, 0.0f);  // stays zero while every du/dt is finite
   const bool v16 = ND % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.u_out) | reinterpret_cast<uintptr_t>(a.u_n)) & 15) == 0;
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    float* out = a.u_out + ((size_t)v * ncell + cell) * ND;
-    const float* un = a.u_n + ((size_t)v * ncell + cell) * ND;
-    float o[ND];
+    f2 c[N][MP], n[N][MP];
+    load_cell<L>(sc, hc[v], c);
     if (with_un) {
+      const float* un = a.u_n + ((size_t)v * ncell + cell) * ND;
       if (v16) {
 #pragma unroll
         for (int q = 0; q < ND / 4; ++q) {
           const float4 x = reinterpret_cast<const float4*>(un)[q];
-          o[4 * q] = x.x;
-          o[4 * q + 1] = x.y;
-          o[4 * q + 2] = x.z;
-          o[4 * q + 3] = x.w;
+          const int m = 4 * q, m2 = m + 2;
+          n[m / N][m % N / 2] = mk2(x.x, x.y);
+          n[m2 / N][m2 % N / 2] = mk2(x.z, x.w);
         }
       } else {
 #pragma unroll
-        for (int m = 0; m < ND; ++m) o[m] = un[m];
+        for (int my = 0; my < N; ++my)
+#pragma unroll
+          for (int p = 0; p < MP; ++p) n[my][p] = mk2(un[2 * p + N * my], 2 * p + 1 < N ? un[2 * p + 1 + N * my] : 0.0f);
       }
     }
 #pragma unroll
-    for (int m = 0; m < ND; ++m) {
-      const int mx = m % N, my = m / N;
-      const float d = r[v][m] * (0.25f * (2 * mx + 1) * (2 * my + 1));
-      nonfinite |= !isfinite(d);
-      if (rk) {
-        float val = fmaf(a.dt, d, C(v, m, hc));
-        if (with_un) val = fmaf(a.rk_b, val - o[m], o[m]);
-        o[m] = val;
-      } else {
-        o[m] = d;
+    for (int my = 0; my < N; ++my)
+#pragma unroll
+      for (int p = 0; p < MP; ++p) {
+        const float ys = 0.25f * (2 * my + 1);
+        f2 d = mul2(r[v][my][p], mk2(ys * (4 * p + 1), ys * (4 * p + 3)));
+        if (2 * p + 1 >= N) d.y = 0.0f;
+        fin = fma2(d, dup2(0.0f), fin);
+        if (rk) {
+          d = fma2(dup2(a.dt), d, c[my][p]);
+          if (with_un) d = fma2(dup2(a.rk_b), sub2(d, n[my][p]), n[my][p]);
+        }
+        c[my][p] = d;
       }
-    }
+    auto val = [&](int m) { return (m % N) & 1 ? c[m / N][m % N / 2].y : c[m / N][m % N / 2].x; };
+    float* out = a.u_out + ((size_t)v * ncell + cell) * ND;
     if (v16) {
 #pragma unroll
       for (int q = 0; q < ND / 4; ++q)
-        reinterpret_cast<float4*>(out)[q] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+        reinterpret_cast<float4*>(out)[q] = make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
     } else {
 #pragma unroll
-      for (int m = 0; m < ND; ++m) out[m] = o[m];
+      for (int m = 0; m < ND; ++m) out[m] = val(m);
     }
   }
-  if (nonfinite) atomicOr(a.status, kStatNonfinite);
+  if (!(fin.x + fin.y == 0.0f)) atomicOr(a.status, kStatNonfinite);
+  }  // active
   if (bad) atomicOr(a.status, kStatPositivity);
 }
 
@@ -853,8 +731,7 @@ cudaError_t launch_euler(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_
   }
   if (m->tables_bytes != sizeof(Tb)) return cudaErrorInvalidValue;
   dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
-  kern<<<grid, TX * TY, smem, s>>>(a, *static_cast<const Tb*>(m->tables));
-  return cudaGetLastError();
+  return launch_pdl(kern, grid, dim3(euler_threads<P, TX, TY>()), smem, s, a, static_cast<const Tb*>(m->tables)->pk);
 }
 
 

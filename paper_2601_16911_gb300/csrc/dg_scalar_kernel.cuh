@@ -72,7 +72,7 @@ struct TileLayout {
   static constexpr int HX = TX + 2, HY = DIM == 2 ? TY + 2 : 1, NH = HX * HY;
   static constexpr int VXT = TX + 1, VYT = DIM == 2 ? TY + 1 : 1, NVT = VXT * VYT;
   static_assert(!TC || (Img::HAS_TC && TX == 8 && NT == 128), "tensor-core form: 2D p = 3, 8 x 16 tiles");
-  static constexpr bool CHUNKED = ND % 4 == 0, SWIZZLED = ND == 16;
+  static constexpr bool CHUNKED = ND % 4 == 0, SWIZZLED = ND == 16, ROWS = DIM == 2 && P == 4;  // ROWS: store_rows
   static constexpr int RS = CHUNKED ? HX * ND
                             : DIM == 1 ? (HX * ND + 6) / 4 * 4
                                        : TX * ND + 32 * ((2 * ND + 3 + 31) / 32);
@@ -90,7 +90,7 @@ struct TileLayout {
   static constexpr int OFF_IMG = (OFF_ST + imax(TC ? 2 * TSA_PART : VS * NVT, SCF) + 3) / 4 * 4;  // the staged PackedImage
   static constexpr int OFF_ATC = OFF_IMG + Img::TC;               // TC: [2][NC][TCCH][TCK][4]
   // u_n of the tile's cells: CHUNKED [NT][US] (a padded stride, conflict-free for 16-byte
-  // loads), otherwise [ND][NT]
+  // loads), otherwise [ND][NT] (ROWS tiles read u_n when they write)
   static constexpr int US = ND == 16 ? 20 : ND;
   static constexpr int OFF_UN = OFF_IMG + IMG;
   // face fluxes of the tile, projected on the tangential modes: x-faces ((TX+1) per tile
@@ -98,7 +98,7 @@ struct TileLayout {
   // nodes of the left/lower and of the right/upper cell
   static constexpr int NFP = DIM == 2 ? N : 1;
   static constexpr int NFX = (TX + 1) * TY, NFY = DIM == 2 ? TX * (TY + 1) : 0, NFACE = NFX + NFY;
-  static constexpr int OFF_F = OFF_UN + (CHUNKED ? US : ND) * NT;  // [NFACE][NFP]
+  static constexpr int OFF_F = OFF_UN + (ROWS ? 0 : CHUNKED ? US : ND) * NT;  // [NFACE][NFP]
   static constexpr int OFF_LAM = OFF_F + NFACE * NFP;             // [2][NFACE]
   static constexpr int FLOATS = OFF_LAM + 2 * NFACE;
   static constexpr size_t BYTES = sizeof(float) * (size_t)FLOATS;
@@ -194,6 +194,81 @@ __device__ __forceinline__ void load_pairs(const float* t, f2 (&b)[MP]) {
   } else {
 #pragma unroll
     for (int p = 0; p < MP; ++p) b[p] = *reinterpret_cast<const f2*>(t + 2 * p);
+  }
+}
+
+// Output of a 2D Q4 tile.  A thread's own 25 floats lie 25 apart in global memory, so its
+// stores (and reads of u_n) would each touch a sector per lane: by rows the 256^2 Burgers
+// step takes 113.5 us instead of 122.9, the 330 x 170 residual 29.6 instead of 31.4.  (At Q2
+// the nine floats per thread cost less than the copy: 69 against 63 us per limited step.)
+//  Its cell's slot in the tile, which no other thread reads by then, already
+// has the phase of the cell's place in the array: each thread writes its result there, and
+// its warp copies the tile rows of its cells as runs: out = w, or u_n + rk_b (w - u_n) where
+// with_un.  off: first float of the variable.  Every lane of the warps that hold cells calls it.
+template <class L, int TX, int TY>
+__device__ __forceinline__ void store_rows(const StageArgs& a, const float* sc, const int* ph, int64_t off, int i0, int j0,
+                                           bool with_un) {
+  constexpr int ND = L::ND, RPW = 32 / TX, NCH = (TX * ND + 6) / 4;
+  const int nx = a.nx, ny = a.ny, row0 = (int)(threadIdx.x / 32) * RPW, wid = min(TX, nx - i0) * ND;
+  const bool vec = ((reinterpret_cast<uintptr_t>(a.u_in) | reinterpret_cast<uintptr_t>(a.u_out) |
+                     (with_un ? reinterpret_cast<uintptr_t>(a.u_n) : 0)) & 15) == 0;
+#pragma unroll
+  for (int it = 0; it < (RPW * NCH + 31) / 32; ++it) {
+    const int f = it * 32 + (threadIdx.x & 31), r = row0 + f / NCH, k = f % NCH;
+    if (f >= RPW * NCH || r >= TY || j0 + r >= ny) continue;
+    const int64_t g0 = off + ((int64_t)(j0 + r) * nx + i0) * ND, c = (g0 & ~(int64_t)3) + 4 * k;
+    const int x0 = (int)(c - g0);  // the chunk's first float within the run
+    const float* w = sc + (r + 1) * L::RS + ph[r + 1] + ND + x0;
+    if (vec && x0 >= 0 && x0 + 4 <= wid) {
+      if (!CVW_SPAN(a.status, c, 4, a.lim_out)) continue;
+      float4 v = *reinterpret_cast<const float4*>(w);
+      if (with_un) {
+        const float4 n = *reinterpret_cast<const float4*>(a.u_n + c);
+        v = make_float4(fmaf(a.rk_b, v.x - n.x, n.x), fmaf(a.rk_b, v.y - n.y, n.y), fmaf(a.rk_b, v.z - n.z, n.z),
+                        fmaf(a.rk_b, v.w - n.w, n.w));
+      }
+      *reinterpret_cast<float4*>(a.u_out + c) = v;
+    } else {
+      for (int e = max(0, -x0); e < 4 && x0 + e < wid; ++e) {
+        if (!CVW_SPAN(a.status, c + e, 1, a.lim_out)) continue;
+        float v = w[e];
+        if (with_un) {
+          const float n = a.u_n[c + e];
+          v = fmaf(a.rk_b, v - n, n);
+        }
+        a.u_out[c + e] = v;
+      }
+    }
+  }
+}
+
+// Writes a 2D or 1D tile's scalar cells: by rows (store_rows) where the layout says so, each
+// thread its own cell otherwise, 16 bytes at a time where it is whole chunks and the output
+// aligned.  hc: the cell's slot in sc.
+template <class L, int TX, int TY>
+__device__ __forceinline__ void write_cell(const StageArgs& a, float* sc, const int* ph, int hc, const f2 (&c)[L::NY1][L::MP],
+                                           int i0, int j0, int tx, int ty, bool active, bool with_un) {
+  constexpr int N = L::N, ND = L::ND;
+  auto val = [&](int m) { return (m % N) & 1 ? c[m / N][m % N / 2].y : c[m / N][m % N / 2].x; };
+  if constexpr (L::ROWS) {
+    if (threadIdx.x >= TX * TY) return;
+    if (active) {
+#pragma unroll
+      for (int m = 0; m < ND; ++m) sc[hc + m] = val(m);
+    }
+    __syncwarp();
+    store_rows<L, TX, TY>(a, sc, ph, 0, i0, j0, with_un);
+  } else {
+    if (!active) return;
+    float* out = a.u_out + ((size_t)(L::NY1 > 1 ? j0 + ty : 0) * a.nx + i0 + tx) * ND;
+    if (ND % 4 == 0 && (reinterpret_cast<uintptr_t>(a.u_out) & 15) == 0) {
+#pragma unroll
+      for (int q = 0; q < ND / 4; ++q)
+        reinterpret_cast<float4*>(out)[q] = make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
+    } else {
+#pragma unroll
+      for (int m = 0; m < ND; ++m) out[m] = val(m);
+    }
   }
 }
 
@@ -692,7 +767,7 @@ __device__ __forceinline__ int cell_face(int k, int tx, int ty) {
 // neighbour is present.  r is set.
 template <int DIM, int P, int SYS, int TX, int TY, bool TC>
 __device__ __forceinline__ void face_residual(const StageArgs& a, const ScalarLaw<SYS, DIM>& law, const float* smem,
-                                              const float* sc, const int* ph, float ubar, int tx, int ty, int gi, int gj,
+                                              float ml, float mb, float ubar, int tx, int ty, int gi, int gj,
                                               f2 (&r)[PackedTables<DIM, P>::NY1][PackedTables<DIM, P>::MP]) {
   using L = TileLayout<DIM, P, TX, TY, TC>;
   constexpr int N = L::N, MP = L::MP, NFP = L::NFP;
@@ -700,7 +775,7 @@ __device__ __forceinline__ void face_residual(const StageArgs& a, const ScalarLa
   if constexpr (DIM == 1) {
     const bool hasL = a.perx || gi > 0;
     const float FR = sF[tx + 1];
-    const float FL = sF[tx] + (hasL ? law.flux_dev_dir(sc[L::cell(ph, tx, 0)] - ubar, 0) : 0.0f);
+    const float FL = sF[tx] + (hasL ? law.flux_dev_dir(ml - ubar, 0) : 0.0f);
     // r[m] = -2/dx (FR - (-1)^m FL)
     const f2 v = mk2(-a.two_dx * (FR - FL), -a.two_dx * (FR + FL));
 #pragma unroll
@@ -721,8 +796,8 @@ __device__ __forceinline__ void face_residual(const StageArgs& a, const ScalarLa
         for (int j = 0; j < N; ++j) h[k][j] = src[j];
       }
     }
-    if (a.perx || gi > 0) h[1][0] = fmaf(2.0f, law.flux_dev_dir(sc[L::cell(ph, tx, ty + 1)] - ubar, 0), h[1][0]);
-    if (a.pery || gj > 0) h[3][0] = fmaf(2.0f, law.flux_dev_dir(sc[L::cell(ph, tx + 1, ty)] - ubar, 1), h[3][0]);
+    if (a.perx || gi > 0) h[1][0] = fmaf(2.0f, law.flux_dev_dir(ml - ubar, 0), h[1][0]);
+    if (a.pery || gj > 0) h[3][0] = fmaf(2.0f, law.flux_dev_dir(mb - ubar, 1), h[3][0]);
     // r[mx,my] = -2/dx (hR[my] - (-1)^mx hL[my]) - 2/dy (hT[mx] - (-1)^my hB[mx])
     f2 ve[MP], vo[MP];
 #pragma unroll
@@ -975,9 +1050,15 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
                   ok ? 16 : 0);
     }
   } else if (!L::CHUNKED && aligned) {
-    if constexpr (!L::CHUNKED)
-      stage_rows16<ND, HX, HY, L::RS, NB>(sc, ph, a.u_in, nx, DIM == 2 ? ny : 1, i0 - 1, DIM == 2 ? j0 - 1 : 0, a.perx,
-                                          DIM == 2 && a.pery, a.status, CVW_EXTENT(a, lim_in));
+    if constexpr (!L::CHUNKED) {
+      if (i0 > 0 && i0 + TX < nx)
+        stage_rows16_inner<ND, HX, HY, L::RS, NB, 1>(sc, 0, ph, a.u_in, 0, nx, DIM == 2 ? ny : 1, i0 - 1,
+                                                     DIM == 2 ? j0 - 1 : 0, DIM == 2 && a.pery, a.status,
+                                                     CVW_EXTENT(a, lim_in));
+      else
+        stage_rows16<ND, HX, HY, L::RS, NB>(sc, ph, a.u_in, nx, DIM == 2 ? ny : 1, i0 - 1, DIM == 2 ? j0 - 1 : 0, a.perx,
+                                            DIM == 2 && a.pery, a.status, CVW_EXTENT(a, lim_in));
+    }
   } else {
     for (int f = threadIdx.x; f < NH * ND; f += NB) {
       const int r = DIM == 2 ? f / (HX * ND) : 0, rem = f - r * (HX * ND), cc = rem / ND, mm = rem - cc * ND;
@@ -1001,7 +1082,7 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
   // u_n of the thread's own cell (RK stages 2 and 3), read only by the output: copied after
   // the halo so that it overlaps the stages below, and awaited before the output.
   // Only this thread reads u_n or writes u_out for its cell, so u_n may alias u_out.
-  const bool pre_un = (a.mode & kModeRK) && a.rk_a != 0.0f;
+  const bool with_un = (a.mode & kModeRK) && a.rk_a != 0.0f, pre_un = with_un && !L::ROWS;
   const bool un16 = L::CHUNKED && (reinterpret_cast<uintptr_t>(a.u_n) & 15) == 0;
   {
     const int ogi = i0 + threadIdx.x % TX, ogj = DIM == 2 ? j0 + threadIdx.x / TX : 0;
@@ -1097,7 +1178,9 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
   } else if constexpr (TC) {
     const bool faces_now = active && !(a.mode & (kModeSensorOnly | kModeLimit));
     gam = cell_sensor_tc<P, TX, TY>(a, T, tcx, c, n0, wstar, [&] {
-      if (faces_now) face_residual<DIM, P, SYS, TX, TY, TC>(a, Law(a, ubar), smem, sc, ph, ubar, tx, ty, gi, gj, r);
+      if (faces_now)
+        face_residual<DIM, P, SYS, TX, TY, TC>(a, Law(a, ubar), smem, sc[L::cell(ph, tx, ty + 1)], sc[L::cell(ph, tx + 1, ty)],
+                                               ubar, tx, ty, gi, gj, r);
     });
   } else if (active) {
     gam = cell_sensor<DIM, P, TX, TY>(a, T, st, c, tx, ty, n0, wstar);
@@ -1105,8 +1188,7 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
 
   // ---- HWENO limiter (Sec. 3): u^{e,*} = mean of u^e + R^{-1} w* on the other modes ----
   if (a.mode & kModeLimit) {
-    if (!active) return;
-    const bool lim = a.limit_all || (gam < a.c_gamma && n0 > 1e-30f);
+    const bool lim = active && (a.limit_all || (gam < a.c_gamma && n0 > 1e-30f));
     if (lim) {
       norm_solve2<DIM, P>(T, wstar);
       f2 bad = mk2(ubar * 0.0f, 0.0f);
@@ -1120,10 +1202,8 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
       c[0][0].x = ubar;
       if (!(bad.x + bad.y == 0.0f)) atomicOr(a.status, kStatNonfinite);
     }
-    float* o = a.u_out + cell * ND;
-#pragma unroll
-    for (int m = 0; m < ND; ++m) o[m] = (m % N) & 1 ? c[m / N][m % N / 2].y : c[m / N][m % N / 2].x;
-    if (a.troubled_out) a.troubled_out[cell] = lim ? 1 : 0;
+    if (active && a.troubled_out) a.troubled_out[cell] = lim ? 1 : 0;
+    write_cell<L, TX, TY>(a, sc, ph, hc, c, i0, j0, tx, ty, active, false);
     return;
   }
 
@@ -1134,6 +1214,9 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
   // (cell, node group) tasks; each cell then sums its groups in a fixed order.
   bool troubled = false;
   float afac = -1.0f;  // alpha_q = Nq[q] * afac where afac >= 0, else alpha_q = 1
+  // means of the left and lower neighbours (after stage (d) a cell's slot is its thread's own)
+  const float ml = active ? sc[L::cell(ph, tx, DIM == 2 ? ty + 1 : 0)] : 0.0f;
+  const float mb = DIM == 2 && active ? sc[L::cell(ph, tx + 1, ty)] : 0.0f;
   if (!sensor_only) {
     if (active) {
       troubled = a.sc && gam < a.c_gamma && n0 > 1e-30f;
@@ -1167,14 +1250,14 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
       }
     }
   }
-  if (!active) return;
+  if (active) {
 
   // ---- (e) faces into the residual; lambda_e over the face nodes ----------------------------
   // From here on the modes without the mean: rounding stays relative to the in-cell variation.
   if (!TC) load_cell<L>(sc, hc, c);  // again, rather than held over the sensor
   c[0][0].x = 0.0f;
   const Law law(a, ubar);
-  if (!TC && !sensor_only) face_residual<DIM, P, SYS, TX, TY, TC>(a, law, smem, sc, ph, ubar, tx, ty, gi, gj, r);
+  if (!TC && !sensor_only) face_residual<DIM, P, SYS, TX, TY, TC>(a, law, smem, ml, mb, ubar, tx, ty, gi, gj, r);
   float lam = need_lam ? 0.0f : a.lambda_const;
   if (need_lam) {
     const float* sLam = smem + L::OFF_LAM;
@@ -1277,9 +1360,7 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
     }
   }
 
-  // ---- M^{-1} and output; 16-byte stores where the cell is whole 16-byte chunks and the
-  // output is 16-byte aligned
-  float* out = a.u_out + cell * ND;
+  // ---- M^{-1} and the RK combination (without u_n where the rows take it) ------------------------
   const float* sUn = smem + L::OFF_UN;  // u_n of this cell
   if (pre_un) cp_async_wait_all();
   c[0][0].x = ubar;
@@ -1314,18 +1395,10 @@ __device__ __forceinline__ void scalar_tile(const StageArgs& a, const PackedTabl
       r[my][p] = d;
     }
   }
-  if (ND % 4 == 0 && (reinterpret_cast<uintptr_t>(a.u_out) & 15) == 0) {
-#pragma unroll
-    for (int q = 0; q < ND / 4; ++q) {
-      const int m = 4 * q, m2 = m + 2;
-      const f2 x = r[m / N][m % N / 2], y = r[m2 / N][m2 % N / 2];
-      reinterpret_cast<float4*>(out)[q] = make_float4(x.x, x.y, y.x, y.y);
-    }
-  } else {
-#pragma unroll
-    for (int m = 0; m < ND; ++m) out[m] = (m % N) & 1 ? r[m / N][m % N / 2].y : r[m / N][m % N / 2].x;
-  }
   if (!(bad.x + bad.y == 0.0f)) atomicOr(a.status, kStatNonfinite);
+  }  // active
+  if (sensor_only) return;
+  write_cell<L, TX, TY>(a, sc, ph, hc, r, i0, j0, tx, ty, active, with_un);
 }
 
 template <int DIM, int P, int SYS, int TX, int TY, bool SURR, int NB = TX * TY, bool TC = false>

@@ -331,4 +331,34 @@ __device__ __forceinline__ void stage_rows16(float* dst, int* ph, const float* s
   }
 }
 
+// The same rows for NV arrays (array v at src + v * var, staged at dst + v * dstv, phases at ph +
+// v * R) where every column is in range: a row is the 16-byte chunks that cover its run, the
+// first up to 3 floats early (floats of the same array), the last zero-filled past the run, so
+// one flat loop over the chunks serves them.  Rows outside the array wrap or read as zeros.
+// Requires RS >= W * E + 6.
+template <int E, int W, int R, int RS, int NT, int NV>
+__device__ __forceinline__ void stage_rows16_inner(float* dst, int dstv, int* ph, const float* src, int64_t var, int ncol,
+                                                   int nrow, int c0, int r0, bool perr, int* status, int64_t lim) {
+  constexpr int NCH = (W * E + 6) / 4;
+  static_assert(RS >= 4 * NCH && RS % 4 == 0, "staging row too short");
+  for (int f = threadIdx.x; f < R * NCH; f += NT) {
+    const int r = f / NCH, k = f - r * NCH;
+    int gr = r0 + r;
+    bool ok = true;
+    if (gr < 0 || gr >= nrow) {
+      if (perr) gr = ((gr % nrow) + nrow) % nrow; else ok = false;
+    }
+    const int64_t row = ((int64_t)gr * ncol + c0) * E;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int64_t g0 = v * var + row, c = (g0 & ~(int64_t)3) + 4 * k;
+      const int left = (int)(g0 + W * E - c);
+      const int n = !ok || left <= 0 ? 0 : left < 4 ? left : 4;
+      const bool in = n > 0 && CVW_SPAN(status, c, n, lim);
+      if (k == 0) ph[v * R + r] = (int)(g0 & 3);
+      cp_async16z(dst + v * dstv + r * RS + 4 * k, in ? src + c : src, in ? 4 * n : 0);
+    }
+  }
+}
+
 }  // namespace cvw
