@@ -12,8 +12,8 @@
 #include <new>
 #include <vector>
 
-#include "cvweno_internal.cuh"
 #include "mlp_mma.cuh"
+#include "stage_common.cuh"
 
 using namespace cvw;
 
@@ -23,8 +23,9 @@ inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 inline cvweno_status cuda_status(cudaError_t e) { return e == cudaSuccess ? CVWENO_OK : CVWENO_ERR_CUDA; }
 
 constexpr int kGradThreads = 256;
-constexpr int kSub = 64;            // samples per shared-memory sub-batch
+constexpr int kSub = 32;            // samples per shared-memory sub-batch
 constexpr int kMaxGradBlocks = 304; // 2 x 152 SMs
+constexpr int kGradStride = (kMlpParams + 3) / 4 * 4;  // floats of one block's partial gradient
 constexpr float kLam = 0.1f, kTau = 0.05f;
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
@@ -41,189 +42,263 @@ __device__ __forceinline__ float gelu_acc(float x, float& dgelu) {
 __device__ __forceinline__ float sigm(float x) { return 1.0f / (1.0f + expf(-x)); }
 __device__ __forceinline__ float softplus(float x) { return fmaxf(x, 0.0f) + log1pf(expf(-fabsf(x))); }
 
-// Shared-memory layout of the gradient kernel (floats).
+// Shared-memory layout of the gradient kernel (floats).  Rows of 64 are padded to 68, so that
+// 16-byte loads of eight consecutive rows cover all banks.
+constexpr int kRow = 68;
 struct GradLayout {
-  static constexpr int W = 0;                        // kMlpParams: W rounded to bf16, biases FP32
-  static constexpr int X = (kMlpParams + 3) / 4 * 4; // [kSub][12]
-  static constexpr int Z1 = X + kSub * kMlpIn;       // [kSub][64] z1, then dz1
-  static constexpr int A1 = Z1 + kSub * 64;          // [kSub][64]
-  static constexpr int Z2 = A1 + kSub * 64;          // [kSub][64] z2, then dz2
-  static constexpr int A2 = Z2 + kSub * 64;          // [kSub][64]
-  static constexpr int DO = A2 + kSub * 64;          // [kSub][2] outputs, then their gradient
-  static constexpr int LS = DO + kSub * 2;           // [kSub] per-sample loss
-  static constexpr int FLOATS = LS + kSub;
+  static constexpr int W1 = 0;                     // [64][12], rounded to bf16
+  static constexpr int W2 = W1 + 64 * kMlpIn;      // [j][k], rounded to bf16
+  static constexpr int W2T = W2 + 64 * kRow;       // [k][j]
+  static constexpr int W3 = W2T + 64 * kRow;       // [2][64]
+  static constexpr int B = W3 + 128;               // b1 [64], b2 [64], b3 [2]
+  static constexpr int X = B + 132;                // [kSub][12]
+  static constexpr int G1 = X + kSub * kMlpIn;     // [kSub][kRow] GELU'(z1), then dz1
+  static constexpr int A1 = G1 + kSub * kRow;
+  static constexpr int G2 = A1 + kSub * kRow;      // GELU'(z2), then dz2
+  static constexpr int A2 = G2 + kSub * kRow;
+  static constexpr int DO = A2 + kSub * kRow;      // [kSub][2] gradient of the outputs
+  static constexpr int FLOATS = DO + kSub * 2;
 };
+
+// acc[s][o] += sum over K of v[row s][k] w[row o][k], in pairs over k: two samples by four outputs
+// (rows o, o + 16, ...) per thread, 16-byte loads of both.
+template <int K>
+__device__ __forceinline__ void dot_tile(const float* v, int vstride, const float* w, int wstride, f2 (&acc)[2][4]) {
+#pragma unroll 4
+  for (int k = 0; k < K; k += 4) {
+    float4 x[2], y[4];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) x[t] = *reinterpret_cast<const float4*>(v + t * vstride + k);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) y[o] = *reinterpret_cast<const float4*>(w + 16 * o * wstride + k);
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        acc[t][o] = fma2(mk2(x[t].x, x[t].y), mk2(y[o].x, y[o].y), acc[t][o]);
+        acc[t][o] = fma2(mk2(x[t].z, x[t].w), mk2(y[o].z, y[o].w), acc[t][o]);
+      }
+  }
+}
 
 // Forward and backward over samples [begin, end) of this block's share of the batch;
 // writes the block's summed gradient (already divided by the batch size n) and loss.
-__global__ void __launch_bounds__(kGradThreads)
+// Sub-batches of 32 samples live in shared memory; every product is a register-tiled one on
+// two-wide FMAs (2 samples x 4 outputs per thread forward and back, 4 x 4 of dW2 over the
+// samples), so a shared-memory load feeds several FMAs.  32 samples rather than 64 give a
+// minibatch of 4,096 128 blocks.  Bound by FP32 issue (tanhf and the products).
+// Minibatch 4,096: 20 us (one output per thread and step, W2 rows 64 floats apart: every
+// load of a warp hit one bank: 65 us).
+__global__ void __launch_bounds__(kGradThreads, 2)
     mlp_grad_kernel(const float* __restrict__ params, const float* __restrict__ X, const float* __restrict__ y,
                     int64_t n, int64_t per_block, float* __restrict__ gpart, float* __restrict__ lpart) {
   extern __shared__ __align__(16) float sm[];
   using L = GradLayout;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < kMlpParams; i += kGradThreads) {
-    const bool is_w = i < kMlpOffB1 || (i >= kMlpOffW2 && i < kMlpOffB2) || (i >= kMlpOffW3 && i < kMlpOffB3);
-    sm[L::W + i] = is_w ? bf16r(params[i]) : params[i];
+  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int i = tid; i < 64 * kMlpIn; i += kGradThreads) sm[L::W1 + i] = bf16r(params[kMlpOffW1 + i]);
+  for (int i = tid; i < 64 * 64; i += kGradThreads) {
+    const float w = bf16r(params[kMlpOffW2 + i]);
+    sm[L::W2 + (i >> 6) * kRow + (i & 63)] = w;
+    sm[L::W2T + (i & 63) * kRow + (i >> 6)] = w;
   }
-  const float* W1 = sm + L::W + kMlpOffW1;
-  const float* B1 = sm + L::W + kMlpOffB1;
-  const float* W2 = sm + L::W + kMlpOffW2;
-  const float* B2 = sm + L::W + kMlpOffB2;
-  const float* W3 = sm + L::W + kMlpOffW3;
-  const float* B3 = sm + L::W + kMlpOffB3;
+  if (tid < 128) {
+    sm[L::W3 + tid] = bf16r(params[kMlpOffW3 + tid]);
+    sm[L::B + tid] = tid < 64 ? params[kMlpOffB1 + tid] : params[kMlpOffB2 + tid - 64];
+  }
+  if (tid < 2) sm[L::B + 128 + tid] = params[kMlpOffB3 + tid];
   float* xs = sm + L::X;
-  float* z1 = sm + L::Z1;
-  float* a1 = sm + L::A1;
-  float* z2 = sm + L::Z2;
-  float* a2 = sm + L::A2;
-  float* dout = sm + L::DO;
-  float* ls = sm + L::LS;
-  // gradient accumulators of the parameters this thread owns: i = tid + 256 k
-  constexpr int KOWN = (kMlpParams + kGradThreads - 1) / kGradThreads;
-  float acc[KOWN];
+  float *g1 = sm + L::G1, *a1 = sm + L::A1, *g2 = sm + L::G2, *a2 = sm + L::A2, *dout = sm + L::DO;
+  // this thread's sums: dW2 rows 4 ty .. + 3, columns 4 tx .. + 3; dW1 row tid / 4, columns
+  // 3 (tid % 4) .. + 2; one of db1, db2, dW3; db3 on the first two
+  f2 w2acc[4][2];
+  float w1acc[3] = {0.0f, 0.0f, 0.0f}, bacc = 0.0f, b3acc = 0.0f, lsum = 0.0f;
 #pragma unroll
-  for (int k = 0; k < KOWN; ++k) acc[k] = 0.0f;
-  float lsum = 0.0f;  // thread 0 only
+  for (int o = 0; o < 4; ++o) w2acc[o][0] = w2acc[o][1] = mk2(0.0f, 0.0f);
   const int64_t begin = (int64_t)blockIdx.x * per_block;
   const int64_t end = begin + per_block < n ? begin + per_block : n;
   const float inv_n = 1.0f / (float)n;
-  __syncthreads();
   for (int64_t s0 = begin; s0 < end; s0 += kSub) {
     const int nb = (int)(end - s0 < kSub ? end - s0 : kSub);
-    for (int i = tid; i < kSub * kMlpIn; i += kGradThreads) {
-      const int b = i / kMlpIn;
-      xs[i] = b < nb ? bf16r(X[(s0 + b) * kMlpIn + (i - b * kMlpIn)]) : 0.0f;
-    }
+    for (int i = tid; i < kSub * kMlpIn; i += kGradThreads)
+      xs[i] = i / kMlpIn < nb ? bf16r(X[s0 * kMlpIn + i]) : 0.0f;
     __syncthreads();
-    // layer 1
-    for (int i = tid; i < kSub * 64; i += kGradThreads) {
-      const int b = i >> 6, j = i & 63;
-      float z = B1[j];
+    // layers 1 and 2: samples 2 ty, 2 ty + 1, outputs tx + 16 o
+    auto layer = [&](const f2 (&acc)[2][4], const float* bias, float* a, float* g) {
 #pragma unroll
-      for (int k = 0; k < kMlpIn; ++k) z = fmaf(W1[j * kMlpIn + k], xs[b * kMlpIn + k], z);
-      float dg;
-      a1[i] = gelu_acc(z, dg);
-      z1[i] = dg;  // keep GELU'(z1) for the backward pass
-    }
-    __syncthreads();
-    // layer 2
-    for (int i = tid; i < kSub * 64; i += kGradThreads) {
-      const int b = i >> 6, j = i & 63;
-      float z = B2[j];
-#pragma unroll 16
-      for (int k = 0; k < 64; ++k) z = fmaf(W2[j * 64 + k], a1[b * 64 + k], z);
-      float dg;
-      a2[i] = gelu_acc(z, dg);
-      z2[i] = dg;
-    }
-    __syncthreads();
-    // outputs, loss (S5) and the output gradient
-    if (tid < kSub) {
-      const int b = tid;
-      float o[2];
+      for (int t = 0; t < 2; ++t)
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        float z = B3[r];
-        for (int k = 0; k < 64; ++k) z = fmaf(W3[r * 64 + k], a2[b * 64 + k], z);
-        o[r] = z;
+        for (int o = 0; o < 4; ++o) {
+          const int j = tx + 16 * o, at = (2 * ty + t) * kRow + j;
+          float dg;
+          a[at] = gelu_acc(bias[j] + (acc[t][o].x + acc[t][o].y), dg);
+          g[at] = dg;  // kept for the backward pass
+        }
+    };
+    f2 acc[2][4];
+    auto zero = [&] {
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[t][o] = mk2(0.0f, 0.0f);
+    };
+    zero();
+    dot_tile<kMlpIn>(xs + 2 * ty * kMlpIn, kMlpIn, sm + L::W1 + tx * kMlpIn, kMlpIn, acc);
+    layer(acc, sm + L::B, a1, g1);
+    __syncthreads();
+    zero();
+    dot_tile<64>(a1 + 2 * ty * kRow, kRow, sm + L::W2 + tx * kRow, kRow, acc);
+    layer(acc, sm + L::B + 64, a2, g2);
+    __syncthreads();
+    // outputs, loss (S5) and the output gradient: eight lanes per sample, eight inputs each
+    {
+      const int b = tid / 8, l = tid % 8;
+      float o0 = 0.0f, o1 = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float v = a2[b * kRow + l + 8 * k];
+        o0 = fmaf(sm[L::W3 + l + 8 * k], v, o0);
+        o1 = fmaf(sm[L::W3 + 64 + l + 8 * k], v, o1);
       }
-      float l = 0.0f, d0 = 0.0f, d1 = 0.0f;
-      if (b < nb) {
-        const float yy = y[s0 + b];
-        const float gh = sigm(o[0]);
-        const float t = fabsf(gh - yy) < kTau ? 1.0f : 0.0f;
-        l = (gh - yy) * (gh - yy) + kLam * (softplus(o[1]) - t * o[1]);
-        d0 = 2.0f * (gh - yy) * gh * (1.0f - gh) * inv_n;
-        d1 = kLam * (sigm(o[1]) - t) * inv_n;
+#pragma unroll
+      for (int d = 1; d < 8; d *= 2) {
+        o0 += __shfl_xor_sync(0xffffffffu, o0, d, 8);
+        o1 += __shfl_xor_sync(0xffffffffu, o1, d, 8);
       }
-      dout[2 * b] = d0;
-      dout[2 * b + 1] = d1;
-      ls[b] = l;
+      o0 += sm[L::B + 128];
+      o1 += sm[L::B + 129];
+      if (l == 0) {
+        float d0 = 0.0f, d1 = 0.0f;
+        if (b < nb) {
+          const float yy = y[s0 + b];
+          const float gh = sigm(o0);
+          const float t = fabsf(gh - yy) < kTau ? 1.0f : 0.0f;
+          lsum += (gh - yy) * (gh - yy) + kLam * (softplus(o1) - t * o1);
+          d0 = 2.0f * (gh - yy) * gh * (1.0f - gh) * inv_n;
+          d1 = kLam * (sigm(o1) - t) * inv_n;
+        }
+        dout[2 * b] = d0;
+        dout[2 * b + 1] = d1;
+      }
     }
     __syncthreads();
-    if (tid == 0)
-      for (int b = 0; b < nb; ++b) lsum += ls[b];  // fixed order
     // dz2 = (dout W3) * GELU'(z2), in place of GELU'(z2)
-    for (int i = tid; i < kSub * 64; i += kGradThreads) {
-      const int b = i >> 6, j = i & 63;
-      z2[i] *= fmaf(dout[2 * b], W3[j], dout[2 * b + 1] * W3[64 + j]);
-    }
-    __syncthreads();
-    // dz1 = (dz2 W2) * GELU'(z1)
-    for (int i = tid; i < kSub * 64; i += kGradThreads) {
-      const int b = i >> 6, j = i & 63;
-      float s = 0.0f;
-#pragma unroll 16
-      for (int k = 0; k < 64; ++k) s = fmaf(z2[b * 64 + k], W2[k * 64 + j], s);
-      z1[i] *= s;
-    }
-    __syncthreads();
-    // parameter gradients of this sub-batch, summed over its samples in order
 #pragma unroll
-    for (int k = 0; k < KOWN; ++k) {
-      const int p = tid + kGradThreads * k;
-      if (p >= kMlpParams) continue;
-      float g = 0.0f;
-      if (p < kMlpOffB1) {
-        const int j = p / kMlpIn, c = p - j * kMlpIn;
-        for (int b = 0; b < nb; ++b) g = fmaf(z1[b * 64 + j], xs[b * kMlpIn + c], g);
-      } else if (p < kMlpOffW2) {
-        const int j = p - kMlpOffB1;
-        for (int b = 0; b < nb; ++b) g += z1[b * 64 + j];
-      } else if (p < kMlpOffB2) {
-        const int j = (p - kMlpOffW2) >> 6, c = (p - kMlpOffW2) & 63;
-        for (int b = 0; b < nb; ++b) g = fmaf(z2[b * 64 + j], a1[b * 64 + c], g);
-      } else if (p < kMlpOffW3) {
-        const int j = p - kMlpOffB2;
-        for (int b = 0; b < nb; ++b) g += z2[b * 64 + j];
-      } else if (p < kMlpOffB3) {
-        const int r = (p - kMlpOffW3) >> 6, c = (p - kMlpOffW3) & 63;
-        for (int b = 0; b < nb; ++b) g = fmaf(dout[2 * b + r], a2[b * 64 + c], g);
-      } else {
-        const int r = p - kMlpOffB3;
-        for (int b = 0; b < nb; ++b) g += dout[2 * b + r];
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        const int b = 2 * ty + t, j = tx + 16 * o;
+        g2[b * kRow + j] *= fmaf(dout[2 * b], sm[L::W3 + j], dout[2 * b + 1] * sm[L::W3 + 64 + j]);
       }
-      acc[k] += g;
+    __syncthreads();
+    // dz1 = (dz2 W2) * GELU'(z1), in place of GELU'(z1)
+    zero();
+    dot_tile<64>(g2 + 2 * ty * kRow, kRow, sm + L::W2T + tx * kRow, kRow, acc);
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) g1[(2 * ty + t) * kRow + tx + 16 * o] *= acc[t][o].x + acc[t][o].y;
+    __syncthreads();
+    // parameter gradients of this sub-batch, summed over its samples in order (samples past
+    // nb have dout = 0, hence zero dz)
+#pragma unroll 4
+    for (int b = 0; b < kSub; ++b) {
+      const float4 d = *reinterpret_cast<const float4*>(g2 + b * kRow + 4 * ty);
+      const float4 v = *reinterpret_cast<const float4*>(a1 + b * kRow + 4 * tx);
+      const f2 lo = mk2(v.x, v.y), hi = mk2(v.z, v.w);
+      w2acc[0][0] = fma2(dup2(d.x), lo, w2acc[0][0]);
+      w2acc[0][1] = fma2(dup2(d.x), hi, w2acc[0][1]);
+      w2acc[1][0] = fma2(dup2(d.y), lo, w2acc[1][0]);
+      w2acc[1][1] = fma2(dup2(d.y), hi, w2acc[1][1]);
+      w2acc[2][0] = fma2(dup2(d.z), lo, w2acc[2][0]);
+      w2acc[2][1] = fma2(dup2(d.z), hi, w2acc[2][1]);
+      w2acc[3][0] = fma2(dup2(d.w), lo, w2acc[3][0]);
+      w2acc[3][1] = fma2(dup2(d.w), hi, w2acc[3][1]);
+      const float e = g1[b * kRow + tid / 4];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) w1acc[c] = fmaf(e, xs[b * kMlpIn + 3 * (tid % 4) + c], w1acc[c]);
+      if (tid < 64)
+        bacc += g1[b * kRow + tid];
+      else if (tid < 128)
+        bacc += g2[b * kRow + tid - 64];
+      else
+        bacc = fmaf(dout[2 * b + (tid - 128) / 64], a2[b * kRow + tid % 64], bacc);
+      if (tid < 2) b3acc += dout[2 * b + tid];
     }
     __syncthreads();
   }
+  float* gp = gpart + (size_t)blockIdx.x * kGradStride;
 #pragma unroll
-  for (int k = 0; k < KOWN; ++k) {
-    const int p = tid + kGradThreads * k;
-    if (p < kMlpParams) gpart[(size_t)blockIdx.x * kMlpParams + p] = acc[k];
+  for (int o = 0; o < 4; ++o)
+    *reinterpret_cast<float4*>(gp + kMlpOffW2 + (4 * ty + o) * 64 + 4 * tx) =
+        make_float4(w2acc[o][0].x, w2acc[o][0].y, w2acc[o][1].x, w2acc[o][1].y);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) gp[kMlpOffW1 + 3 * tid + c] = w1acc[c];
+  gp[tid < 64 ? kMlpOffB1 + tid : tid < 128 ? kMlpOffB2 + tid - 64 : kMlpOffW3 + tid - 128] = bacc;
+  if (tid < 2) gp[kMlpOffB3 + tid] = b3acc;
+  // loss: the samples' lanes, in order
+  if (tid % 8 == 0) dout[tid / 8] = lsum;
+  __syncthreads();
+  if (tid == 0) {
+    float s = 0.0f;
+    for (int b = 0; b < kSub; ++b) s += dout[b];
+    lpart[blockIdx.x] = s * inv_n;
   }
-  if (tid == 0) lpart[blockIdx.x] = lsum * inv_n;
 }
 
-// grad[p] = sum over blocks, in block order; loss likewise (block 0's thread 0).
-__global__ void mlp_reduce_kernel(const float* __restrict__ gpart, const float* __restrict__ lpart, int nblk,
-                                  float* __restrict__ grad, float* __restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+// Moments and learning rate of one Adam step with bias correction (c1 = 1 - beta1^t,
+// c2 = 1 - beta2^t from the host).
+struct AdamArgs {
+  float *params, *m, *v;
+  float lr, b1, b2, c1, c2, eps;
+};
+__device__ __forceinline__ void adam_update(const AdamArgs& a, int p, float g) {
+  const float mm = fmaf(a.b1, a.m[p], (1.0f - a.b1) * g);
+  const float vv = fmaf(a.b2, a.v[p], (1.0f - a.b2) * g * g);
+  a.m[p] = mm;
+  a.v[p] = vv;
+  a.params[p] -= a.lr * (mm / a.c1) / (sqrtf(vv / a.c2) + a.eps);
+}
+
+// grad[p] = sum over the blocks' partial gradients, and with ADAM the parameter's step: 32
+// parameters per block, eight slices of the partials each summed in block order, then the
+// slices in order.  loss likewise (block 0).
+constexpr int kRedParams = 32, kRedSlices = 8;
+template <bool ADAM>
+__global__ void __launch_bounds__(kRedParams* kRedSlices)
+    mlp_reduce_kernel(const float* __restrict__ gpart, const float* __restrict__ lpart, int nblk, float* __restrict__ grad,
+                      float* __restrict__ loss, AdamArgs a) {
+  __shared__ float part[kRedSlices][kRedParams];
+  const int c = threadIdx.x % kRedParams, sl = threadIdx.x / kRedParams, p = blockIdx.x * kRedParams + c;
+  pdl_wait();
+  pdl_launch_dependents();
+  float s = 0.0f;
   if (p < kMlpParams) {
-    float s = 0.0f;
-    for (int b = 0; b < nblk; ++b) s += gpart[(size_t)b * kMlpParams + p];
-    grad[p] = s;
+#pragma unroll 8
+    for (int b = sl; b < nblk; b += kRedSlices) s += gpart[(size_t)b * kGradStride + p];
   }
-  if (p == 0) {
-    float s = 0.0f;
-    for (int b = 0; b < nblk; ++b) s += lpart[b];
-    *loss = s;
+  part[sl][c] = s;
+  __syncthreads();
+  if (sl == 0 && p < kMlpParams) {
+    s = part[0][c];
+#pragma unroll
+    for (int k = 1; k < kRedSlices; ++k) s += part[k][c];
+    grad[p] = s;
+    if (ADAM) adam_update(a, p, s);
+  }
+  if (blockIdx.x == 0 && sl == 1) {
+    float l = 0.0f;
+    for (int b = c; b < nblk; b += 32) l += lpart[b];
+#pragma unroll
+    for (int d = 16; d > 0; d /= 2) l += __shfl_down_sync(0xffffffffu, l, d);
+    if (c == 0) *loss = l;
   }
 }
 
-// Adam with bias correction (c1 = 1 - beta1^t, c2 = 1 - beta2^t from the host).
-__global__ void mlp_adam_kernel(float* __restrict__ params, float* __restrict__ m, float* __restrict__ v,
-                                const float* __restrict__ grad, float lr, float b1, float b2, float c1, float c2,
-                                float eps) {
+__global__ void mlp_adam_kernel(const float* __restrict__ grad, AdamArgs a) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= kMlpParams) return;
-  const float g = grad[p];
-  const float mm = fmaf(b1, m[p], (1.0f - b1) * g);
-  const float vv = fmaf(b2, v[p], (1.0f - b2) * g * g);
-  m[p] = mm;
-  v[p] = vv;
-  params[p] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+  if (p < kMlpParams) adam_update(a, p, grad[p]);
 }
 
 }  // namespace
@@ -299,7 +374,7 @@ struct cvweno_mlp_s {
   float* d_v = nullptr;
   float* d_grad = nullptr;
   float* d_loss = nullptr;
-  float* d_gpart = nullptr;   // [kMaxGradBlocks][kMlpParams]
+  float* d_gpart = nullptr;   // [kMaxGradBlocks][kGradStride]
   float* d_lpart = nullptr;
   MlpPacked* d_packed = nullptr;
   unsigned int* d_fallbacks = nullptr;
@@ -328,24 +403,32 @@ cudaError_t repack(cvweno_mlp n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t enqueue_grad(cvweno_mlp n, const float* X, const float* y, int64_t count, cudaStream_t s) {
+// Arguments of the network's next Adam step.
+AdamArgs next_adam(cvweno_mlp n, float lr) {
+  const double b1 = 0.9, b2 = 0.999;
+  n->step += 1;
+  return AdamArgs{n->d_params, n->d_m, n->d_v, lr, (float)b1, (float)b2, (float)(1.0 - pow(b1, (double)n->step)),
+                  (float)(1.0 - pow(b2, (double)n->step)), 1e-8f};
+}
+
+// Gradient of the batch into d_grad, and with adam the step too.  Both kernels are launched
+// with programmatic stream serialisation (they wait before they touch anything).
+cudaError_t enqueue_grad(cvweno_mlp n, const float* X, const float* y, int64_t count, const AdamArgs* adam, cudaStream_t s) {
   int64_t nblk = (count + kSub - 1) / kSub;
   if (nblk > kMaxGradBlocks) nblk = kMaxGradBlocks;
   const int64_t per_block = ((count + nblk - 1) / nblk + kSub - 1) / kSub * kSub;
   nblk = (count + per_block - 1) / per_block;
   const size_t smem = sizeof(float) * GradLayout::FLOATS;
-  mlp_grad_kernel<<<(int)nblk, kGradThreads, smem, s>>>(n->d_params, X, y, count, per_block, n->d_gpart, n->d_lpart);
-  mlp_reduce_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(n->d_gpart, n->d_lpart, (int)nblk, n->d_grad,
-                                                              n->d_loss);
-  return cudaGetLastError();
+  cudaError_t e = launch_pdl(mlp_grad_kernel, dim3((unsigned)nblk), dim3(kGradThreads), smem, s, n->d_params, X, y, count,
+                             per_block, n->d_gpart, n->d_lpart);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((kMlpParams + kRedParams - 1) / kRedParams), block(kRedParams * kRedSlices);
+  return launch_pdl(adam ? mlp_reduce_kernel<true> : mlp_reduce_kernel<false>, grid, block, 0, s, n->d_gpart, n->d_lpart,
+                    (int)nblk, n->d_grad, n->d_loss, adam ? *adam : AdamArgs{});
 }
 
 cudaError_t enqueue_adam(cvweno_mlp n, float lr, cudaStream_t s) {
-  const double b1 = 0.9, b2 = 0.999;
-  n->step += 1;
-  const float c1 = (float)(1.0 - pow(b1, (double)n->step)), c2 = (float)(1.0 - pow(b2, (double)n->step));
-  mlp_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(n->d_params, n->d_m, n->d_v, n->d_grad, lr, (float)b1,
-                                                            (float)b2, c1, c2, 1e-8f);
+  mlp_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(n->d_grad, next_adam(n, lr));
   return cudaGetLastError();
 }
 
@@ -365,7 +448,7 @@ cvweno_status cvweno_mlp_create(const float* params, cvweno_mlp* out) {
   if (e == cudaSuccess) e = cudaMalloc(&n->d_v, pb);
   if (e == cudaSuccess) e = cudaMalloc(&n->d_grad, pb);
   if (e == cudaSuccess) e = cudaMalloc(&n->d_loss, sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&n->d_gpart, pb * kMaxGradBlocks);
+  if (e == cudaSuccess) e = cudaMalloc(&n->d_gpart, sizeof(float) * kGradStride * kMaxGradBlocks);
   if (e == cudaSuccess) e = cudaMalloc(&n->d_lpart, sizeof(float) * kMaxGradBlocks);
   if (e == cudaSuccess) e = cudaMalloc(&n->d_packed, sizeof(MlpPacked));
   if (e == cudaSuccess) e = cudaMalloc(&n->d_fallbacks, sizeof(unsigned int));
@@ -404,7 +487,7 @@ cvweno_status cvweno_mlp_loss_grad(cvweno_mlp n, const float* X, const float* y,
                                    float* grad, void* stream) {
   if (!n || !X || !y || count < 1) return CVWENO_ERR_ARG;
   cudaStream_t s = S(stream);
-  cudaError_t e = enqueue_grad(n, X, y, count, s);
+  cudaError_t e = enqueue_grad(n, X, y, count, nullptr, s);
   if (e == cudaSuccess && loss) e = cudaMemcpyAsync(n->h_loss, n->d_loss, sizeof(float), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && grad)
     e = cudaMemcpyAsync(grad, n->d_grad, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost, s);
@@ -430,8 +513,8 @@ cvweno_status cvweno_mlp_train(cvweno_mlp n, const float* X, const float* y, int
   for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep)
     for (int64_t b0 = 0; b0 < count && e == cudaSuccess; b0 += batch) {
       const int64_t nb = count - b0 < batch ? count - b0 : batch;
-      e = enqueue_grad(n, X + b0 * kMlpIn, y + b0, nb, s);
-      if (e == cudaSuccess) e = enqueue_adam(n, lr, s);
+      const AdamArgs adam = next_adam(n, lr);
+      e = enqueue_grad(n, X + b0 * kMlpIn, y + b0, nb, &adam, s);
     }
   if (e == cudaSuccess) e = repack(n, s);
   if (e == cudaSuccess && last_loss)

@@ -620,14 +620,14 @@ class Mlp:
     def params(self):
         buf = (ctypes.c_float * NPARAM_MLP)()
         _check(load().cvweno_mlp_get_params(self._h, buf), "cvweno_mlp_get_params")
-        return [buf[i] for i in range(NPARAM_MLP)]
+        return buf[:]
 
     def loss_grad(self, X, y, stream=None):
         loss = ctypes.c_float()
         grad = (ctypes.c_float * NPARAM_MLP)()
         _check(load().cvweno_mlp_loss_grad(self._h, _ptr(X), _ptr(y), int(X.shape[0]), ctypes.byref(loss), grad,
                                            _stream(stream)), "cvweno_mlp_loss_grad")
-        return loss.value, [grad[i] for i in range(NPARAM_MLP)]
+        return loss.value, grad[:]
 
     def adam_step(self, lr: float, stream=None):
         _check(load().cvweno_mlp_adam_step(self._h, float(lr), _stream(stream)), "cvweno_mlp_adam_step")
