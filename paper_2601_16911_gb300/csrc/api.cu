@@ -13,6 +13,7 @@ namespace {
 
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 304;  // 2 x 152 SMs
+constexpr int kRedOut = 4 * kRedBlocks;  // d_red: partials of up to four variables, then results [8], slots [2]
 constexpr int kProjN = 12;       // projection rule points per direction
 
 inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
@@ -22,9 +23,24 @@ inline cvweno_status cuda_status(cudaError_t e) { return e == cudaSuccess ? CVWE
 // ---- analytic initial data --------------------------------------------------------------
 
 struct ProjTables {
-  float x[kProjN], w[kProjN];
-  float P[kProjN][kMaxP + 1];  // Legendre values at the projection nodes
+  float x[kProjN];
+  float wP[kProjN][kMaxP + 1];  // weight times Legendre value at the projection nodes
 };
+
+// The projection rule and its Legendre values (FP64), built once per process.
+struct ProjRule {
+  double x[kProjN], w[kProjN], P[kProjN][kMaxP + 1];
+  bool ok;
+  ProjRule() {
+    static_assert(kProjN <= kMaxGaussRule, "projection rule larger than the Gauss rule builder");
+    ok = gauss_rule(kProjN, x, w);
+    for (int q = 0; ok && q < kProjN; ++q) legendre_values(x[q], kMaxP, P[q]);
+  }
+};
+const ProjRule& proj_rule() {
+  static const ProjRule rule;
+  return rule;
+}
 
 struct ProjArgs {
   float* u;
@@ -96,36 +112,200 @@ __device__ void ic_eval(const ProjArgs& a, float x, float y, float* U) {
   }
 }
 
-// one thread per cell: c_m = (2mx+1)(2my+1)/4 sum_q w w P_mx P_my u0   (2D)
-__global__ void project_kernel(const __grid_constant__ ProjArgs a, const __grid_constant__ ProjTables T) {
+// L2 projection c_m = (2mx+1)(2my+1)/4 sum_ab w_a w_b P_mx(a) P_my(b) u0(x_a, y_b) (2D), by sum
+// factorisation: each row b of nodes is contracted over x first.  Four lanes per cell take
+// three rows each and add their sums by shuffles, so that a small mesh still fills warps and a
+// cell's chain is a quarter as long.
+constexpr int kProjLanes = 4, kProjRows = kProjN / kProjLanes, kProjThreads = 128;
+
+template <int DIM, int N, int NVAR>
+__global__ void __launch_bounds__(kProjThreads) project_kernel(const __grid_constant__ ProjArgs a,
+                                                               const __grid_constant__ ProjTables T) {
+  constexpr int NY1 = DIM == 2 ? N : 1, ND = N * NY1, R = DIM == 2 ? kProjRows : 1;
   const int64_t ncell = (int64_t)a.nx * a.ny;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ncell; e += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x % kProjLanes;
+  // whole warps stay in the loop (the shuffles are warp-wide); cells past the end are clamped
+  for (int64_t e0 = (blockIdx.x * (int64_t)kProjThreads + (threadIdx.x & ~31)) / kProjLanes; e0 < ncell;
+       e0 += (int64_t)gridDim.x * kProjThreads / kProjLanes) {
+    const int64_t mine = e0 + (threadIdx.x & 31) / kProjLanes, e = mine < ncell ? mine : ncell - 1;
     const int i = (int)(e % a.nx), j = (int)(e / a.nx);
-    const double xc = a.x0 + (i + 0.5) * a.dx, yc = a.dim == 2 ? a.y0 + (j + 0.5) * a.dy : 0.0;
-    float acc[4][25];
-    for (int v = 0; v < 4; ++v)
-      for (int m = 0; m < 25; ++m) acc[v][m] = 0.0f;
-    const int npy = a.dim == 2 ? kProjN : 1;
-    for (int qb = 0; qb < npy; ++qb)
-      for (int qa = 0; qa < kProjN; ++qa) {
-        float x = (float)(xc + 0.5 * a.dx * T.x[qa]);
-        float y = a.dim == 2 ? (float)(yc + 0.5 * a.dy * T.x[qb]) : 0.0f;
-        float W = T.w[qa] * (a.dim == 2 ? T.w[qb] : 1.0f);
+    const double xc = a.x0 + (i + 0.5) * a.dx, yc = DIM == 2 ? a.y0 + (j + 0.5) * a.dy : 0.0;
+    auto node_x = [&](int q) { return (float)(xc + 0.5 * a.dx * T.x[q]); };
+    auto node_y = [&](int q) { return DIM == 2 ? (float)(yc + 0.5 * a.dy * T.x[q]) : 0.0f; };
+    // row k of this lane is b = lane + 4 k (1D: the one row, on lane 0)
+    float s[R][NVAR][N];
+#pragma unroll
+    for (int k = 0; k < R; ++k)
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v)
+#pragma unroll
+        for (int m = 0; m < N; ++m) s[k][v][m] = 0.0f;
+    float y[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) y[k] = node_y(lane + kProjLanes * k);
+#pragma unroll 1
+    for (int q = 0; q < kProjN; ++q) {
+      const float x = node_x(q);
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
         float U[4];
-        ic_eval(a, x, y, U);
-        for (int m = 0; m < a.nd; ++m) {
-          int mx = m % a.n, my = m / a.n;
-          float ph = T.P[qa][mx] * (a.dim == 2 ? T.P[qb][my] : 1.0f);
-          for (int v = 0; v < a.nvar; ++v) acc[v][m] = fmaf(W * ph, U[v], acc[v][m]);
-        }
+        ic_eval(a, x, y[k], U);
+#pragma unroll
+        for (int v = 0; v < NVAR; ++v)
+#pragma unroll
+          for (int m = 0; m < N; ++m) s[k][v][m] = fmaf(T.wP[q][m], U[v], s[k][v][m]);
       }
-    for (int v = 0; v < a.nvar; ++v)
-      for (int m = 0; m < a.nd; ++m) {
-        int mx = m % a.n, my = m / a.n;
-        float s = a.dim == 2 ? 0.25f * (2 * mx + 1) * (2 * my + 1) : 0.5f * (2 * mx + 1);
-        a.u[((size_t)v * ncell + e) * a.nd + m] = acc[v][m] * s;
+    }
+    // over the lane's rows, then over the lanes
+    float c[NVAR][ND];
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v)
+#pragma unroll
+      for (int m = 0; m < ND; ++m) {
+        float acc;
+        if constexpr (DIM == 2) {
+          acc = 0.0f;
+#pragma unroll
+          for (int k = 0; k < R; ++k) acc = fmaf(T.wP[lane + kProjLanes * k][m / N], s[k][v][m % N], acc);
+#pragma unroll
+          for (int d = 1; d < kProjLanes; d *= 2) acc += __shfl_xor_sync(0xffffffffu, acc, d, kProjLanes);
+        } else {
+          acc = s[0][v][m];
+        }
+        c[v][m] = acc * (DIM == 2 ? 0.25f * (2 * (m % N) + 1) * (2 * (m / N) + 1) : 0.5f * (2 * m + 1));
+      }
+    if (mine >= ncell) continue;
+    // lane l writes modes l, l + 4, ...
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v)
+#pragma unroll
+      for (int m0 = 0; m0 < ND; m0 += kProjLanes) {
+        float o = c[v][m0];
+#pragma unroll
+        for (int l = 1; l < kProjLanes; ++l)
+          if (m0 + l < ND && lane == l) o = c[v][m0 + l < ND ? m0 + l : m0];
+        if (m0 + lane < ND) a.u[((size_t)v * ncell + e) * ND + m0 + lane] = o;
       }
   }
+}
+
+// A 2D Fourier datum in closed form.  About the cell's centre, sin(A_c + B_c + d_a + d_b) with
+// offsets d the same in every cell, so the rule's sums over x and y separate: per mode a cell
+// needs the sine and cosine of its two centre phases, and the projections of sin and cos of the
+// offsets (host, FP64).  The centre phases are formed in turns, as the product of i + 1/2 with a
+// two-float ratio, and reduced before they are rounded.  Bound by the stores and by FP32 issue:
+// 512^2 Q3 with four modes: 9.8 us (2.63 ms with 144 full evaluations and a dense projection per
+// cell, 0.104 ms with one-dimensional phases at the nodes).
+struct FourierArgs {
+  float* u;
+  int nx, ny, modes;
+  float rx[15][2], ry[15][2];                  // turns per cell in x and y (two-float)
+  float cx[15][kMaxP + 1], sx[15][kMaxP + 1];  // (2m+1)/2 sum_a w_a P_m(a) (cos, sin)(d_a)
+  float cy[15][kMaxP + 1], sy[15][kMaxP + 1];  // likewise in y
+  float amp_cos[15], amp_sin[15];              // amplitude times cosine and sine of the phase
+};
+constexpr int kFourierThreads = 128;
+
+// sin and cos of 2 pi (i + 1/2) r, r = r[0] + r[1]
+__device__ __forceinline__ void turn_sincos(int i, const float (&r)[2], float& s, float& c) {
+  const float h = (float)i + 0.5f, p = h * r[0];
+  const float lo = fmaf(h, r[1], fmaf(h, r[0], -p));
+  sincospif(2.0f * ((p - rintf(p)) + lo), &s, &c);
+}
+
+template <int N>
+__global__ void __launch_bounds__(kFourierThreads) project_fourier_kernel(const __grid_constant__ FourierArgs a) {
+  constexpr int ND = N * N;
+  const int64_t ncell = (int64_t)a.nx * a.ny;
+  for (int64_t e = blockIdx.x * (int64_t)kFourierThreads + threadIdx.x; e < ncell; e += (int64_t)gridDim.x * kFourierThreads) {
+    const int i = (int)(e % a.nx), j = (int)(e / a.nx);
+    float c[ND];
+#pragma unroll
+    for (int m = 0; m < ND; ++m) c[m] = 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < a.modes; ++k) {
+      float sa, ca, sb0, cb0;
+      turn_sincos(i, a.rx[k], sa, ca);
+      turn_sincos(j, a.ry[k], sb0, cb0);
+      const float sb = fmaf(sb0, a.amp_cos[k], cb0 * a.amp_sin[k]), cb = fmaf(cb0, a.amp_cos[k], -sb0 * a.amp_sin[k]);
+      float S[N], C[N];  // x projections of sin and cos of A
+#pragma unroll
+      for (int m = 0; m < N; ++m) {
+        S[m] = fmaf(sa, a.cx[k][m], ca * a.sx[k][m]);
+        C[m] = fmaf(ca, a.cx[k][m], -sa * a.sx[k][m]);
+      }
+#pragma unroll
+      for (int my = 0; my < N; ++my) {
+        const float s = fmaf(sb, a.cy[k][my], cb * a.sy[k][my]), t = fmaf(cb, a.cy[k][my], -sb * a.sy[k][my]);
+#pragma unroll
+        for (int m = 0; m < N; ++m) c[m + N * my] = fmaf(S[m], t, fmaf(C[m], s, c[m + N * my]));
+      }
+    }
+    float* o = a.u + e * ND;
+    if (ND % 4 == 0 && (reinterpret_cast<uintptr_t>(a.u) & 15) == 0) {
+#pragma unroll
+      for (int q = 0; q < ND / 4; ++q)
+        reinterpret_cast<float4*>(o)[q] = make_float4(c[4 * q], c[4 * q + 1], c[4 * q + 2], c[4 * q + 3]);
+    } else {
+#pragma unroll
+      for (int m = 0; m < ND; ++m) o[m] = c[m];
+    }
+  }
+}
+
+cudaError_t launch_project_fourier(cvweno_mesh m, const float* prm, const ProjRule& R, float* u, cudaStream_t s) {
+  FourierArgs a;
+  memset(&a, 0, sizeof(a));
+  a.u = u;
+  a.nx = m->nx;
+  a.ny = m->ny;
+  a.modes = (int)prm[0] < 0 ? 0 : (int)prm[0] < 15 ? (int)prm[0] : 15;
+  auto direction = [&](double k, int n, float (&r)[2], float* c, float* sn) {
+    const double turns = k / n;  // per cell
+    r[0] = (float)turns;
+    r[1] = (float)(turns - (double)r[0]);
+    double cs[kMaxP + 1] = {0.0}, ss[kMaxP + 1] = {0.0};
+    for (int q = 0; q < kProjN; ++q) {
+      const double d = M_PI * turns * R.x[q], cd = R.w[q] * cos(d), sd = R.w[q] * sin(d);
+      for (int mm = 0; mm <= m->p; ++mm) {
+        cs[mm] += 0.5 * (2 * mm + 1) * R.P[q][mm] * cd;
+        ss[mm] += 0.5 * (2 * mm + 1) * R.P[q][mm] * sd;
+      }
+    }
+    for (int mm = 0; mm <= m->p; ++mm) c[mm] = (float)cs[mm], sn[mm] = (float)ss[mm];
+  };
+  for (int k = 0; k < a.modes; ++k) {
+    const float* md = prm + 1 + 4 * k;
+    direction(md[1], m->nx, a.rx[k], a.cx[k], a.sx[k]);
+    direction(md[2], m->ny, a.ry[k], a.cy[k], a.sy[k]);
+    a.amp_cos[k] = (float)(md[0] * cos((double)md[3]));
+    a.amp_sin[k] = (float)(md[0] * sin((double)md[3]));
+  }
+  int64_t blocks = (m->ncell + kFourierThreads - 1) / kFourierThreads;
+  if (blocks > 65535) blocks = 65535;
+  switch (m->p) {
+    case 1: project_fourier_kernel<2><<<(int)blocks, kFourierThreads, 0, s>>>(a); break;
+    case 2: project_fourier_kernel<3><<<(int)blocks, kFourierThreads, 0, s>>>(a); break;
+    case 3: project_fourier_kernel<4><<<(int)blocks, kFourierThreads, 0, s>>>(a); break;
+    case 4: project_fourier_kernel<5><<<(int)blocks, kFourierThreads, 0, s>>>(a); break;
+    default: return cudaErrorNotSupported;
+  }
+  return cudaGetLastError();
+}
+
+template <int DIM, int N>
+cudaError_t launch_project(const ProjArgs& a, const ProjTables& T, cudaStream_t s) {
+  const int64_t ncell = (int64_t)a.nx * a.ny;
+  int64_t blocks = (ncell * kProjLanes + kProjThreads - 1) / kProjThreads;
+  if (blocks > 65535) blocks = 65535;
+  if constexpr (DIM == 2) {
+    if (a.nvar == 4) {
+      project_kernel<DIM, N, 4><<<(int)blocks, kProjThreads, 0, s>>>(a, T);
+      return cudaGetLastError();
+    }
+  }
+  project_kernel<DIM, N, 1><<<(int)blocks, kProjThreads, 0, s>>>(a, T);
+  return cudaGetLastError();
 }
 
 // CG: interpolation at the GLL nodes of the periodic lattice (reading A25)
@@ -165,19 +345,42 @@ __global__ void sum_cg_partial(const float* __restrict__ u, int nnx, int nny, in
   if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
 }
 
-// partial[b] = sum over a grid-stride slice of x[i * stride] (FP64), fixed order per block
-__global__ void sum_mode0_partial(const float* __restrict__ x, int64_t n, int stride, double* __restrict__ partial) {
-  __shared__ double sh[kRedThreads];
+// DG conservation totals in one launch: block (b, v) sums mode 0 of a grid-stride slice of
+// variable v (FP64) into partial[v][b]; the last block to finish adds each variable's partials
+// in a fixed order into out[v] and leaves the counter zero for the next call.
+__global__ void __launch_bounds__(kRedThreads) sum_mode0_kernel(const float* __restrict__ u, int64_t n, int stride,
+                                                                double* __restrict__ partial, double* __restrict__ out,
+                                                                unsigned* done) {
+  __shared__ double sh[kRedThreads / 32];
+  __shared__ bool last;
+  const int nb = gridDim.x, nvar = gridDim.y, v = blockIdx.y, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  auto warp_sum = [](double x) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) x += __shfl_down_sync(0xffffffffu, x, d);
+    return x;
+  };
   double acc = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    acc += (double)x[i * stride];
-  sh[threadIdx.x] = acc;
+  for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < n; i += (int64_t)nb * kRedThreads)
+    acc += (double)u[((int64_t)v * n + i) * stride];
+  acc = warp_sum(acc);
+  if (lane == 0) sh[warp] = acc;
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kRedThreads / 32; ++w) acc += sh[w];
+    partial[v * kRedBlocks + blockIdx.x] = acc;
+    __threadfence();
+    last = atomicAdd(done, 1u) == (unsigned)(nb * nvar) - 1;
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (warp < nvar) {  // one warp per variable
+    acc = 0.0;
+    for (int b = lane; b < nb; b += 32) acc += __ldcg(partial + warp * kRedBlocks + b);
+    acc = warp_sum(acc);
+    if (lane == 0) out[warp] = acc;
+  }
+  if (threadIdx.x == 0) *done = 0;
 }
 
 __global__ void max_partial(const float* __restrict__ x, int64_t n, double* __restrict__ partial) {
@@ -257,11 +460,9 @@ cudaError_t launch(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t s) {
   return e;
 }
 
-cvweno_status read_status(cvweno_mesh m, cudaStream_t s) {
-  cudaError_t e = cudaMemcpyAsync(m->h_status, m->d_status, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return CVWENO_ERR_CUDA;
-  int st = *m->h_status;
+// Clears a raised status word that has been read, and its code.
+cvweno_status take_status(cvweno_mesh m, int st, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
   if (st) {
     e = cudaMemsetAsync(m->d_status, 0, sizeof(int), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -274,8 +475,15 @@ cvweno_status read_status(cvweno_mesh m, cudaStream_t s) {
   return CVWENO_OK;
 }
 
+cvweno_status read_status(cvweno_mesh m, cudaStream_t s) {
+  cudaError_t e = cudaMemcpyAsync(m->h_status, m->d_status, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return CVWENO_ERR_CUDA;
+  return take_status(m, *m->h_status, s);
+}
+
 cvweno_status rk_stage(cvweno_mesh m, const float* in, const float* un, float* out, float ra, float rb, float dt,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool limit_pos = false) {
   NvtxRange range("rk_stage");
   StageArgs a = base_args(m);
   a.u_in = in;
@@ -284,6 +492,7 @@ cvweno_status rk_stage(cvweno_mesh m, const float* in, const float* un, float* o
   a.rk_a = ra;
   a.rk_b = rb;
   a.dt = dt;
+  a.limit_pos = limit_pos;
   a.mode = kModeRK;
   return cuda_status(launch(m, a, s));
 }
@@ -335,11 +544,16 @@ cvweno_status enqueue_steps_one_launch(cvweno_mesh m, float* u, float dt, int ns
 cvweno_status enqueue_step(cvweno_mesh m, float* u, float dt, cudaStream_t s) {
   if (steps_in_one_launch(m)) return enqueue_steps_one_launch(m, u, dt, 1, s);
   if (m->desc.params.positivity) {
-    // every stage result is limited in place (reading P3): the limiter is cell-local
-    if (m->timing) {
-      m->tcount = 0;
-      kernel_mark(m, s);
+    // every stage result is limited (reading P3): the limiter is cell-local, so the stage
+    // kernel applies it before it writes; with timing on it is a launch of its own
+    if (!m->timing) {
+      cvweno_status st = rk_stage(m, u, u, m->d_u1, 0.0f, 1.0f, dt, s, true);
+      if (st == CVWENO_OK) st = rk_stage(m, m->d_u1, u, m->d_u2, 0.75f, 0.25f, dt, s, true);
+      if (st == CVWENO_OK) st = rk_stage(m, m->d_u2, u, u, 1.0f / 3.0f, 2.0f / 3.0f, dt, s, true);
+      return st;
     }
+    m->tcount = 0;
+    kernel_mark(m, s);
     cvweno_status st = rk_stage(m, u, u, m->d_u1, 0.0f, 1.0f, dt, s);
     if (st == CVWENO_OK) st = positivity_stage(m, m->d_u1, s);
     if (st == CVWENO_OK) st = rk_stage(m, m->d_u1, u, m->d_u2, 0.75f, 0.25f, dt, s);
@@ -536,7 +750,8 @@ cvweno_status cvweno_mesh_create(const cvweno_mesh_desc* d, cvweno_mesh* out) {
       if (e == cudaSuccess) e = cudaMemcpy(m->d_cg_ml, ml, sizeof(ml), cudaMemcpyHostToDevice);
     }
   }
-  if (e == cudaSuccess) e = cudaMalloc(&m->d_red, sizeof(double) * (kRedBlocks + 8));
+  if (e == cudaSuccess) e = cudaMalloc(&m->d_red, sizeof(double) * (kRedOut + 10));
+  if (e == cudaSuccess) e = cudaMemset(m->d_red, 0, sizeof(double) * (kRedOut + 10));
   if (e == cudaSuccess) e = cudaMalloc(&m->d_status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(m->d_status, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost(&m->h_status, sizeof(int));
@@ -599,17 +814,14 @@ cvweno_status cvweno_project(cvweno_mesh m, int ic_type, const double* ic_params
   a.gas_gamma = m->desc.params.gas_gamma;
   for (int i = 0; i < 64; ++i) a.prm[i] = (float)ic_params[i];
   // Gauss nodes/weights of the 12-point projection rule and Legendre values there.
+  const ProjRule& R = proj_rule();
+  if (!R.ok) return CVWENO_ERR_ARG;
+  if (m->kind != CVWENO_CG && m->dim == 2 && ic_type == CVWENO_IC_FOURIER)
+    return cuda_status(launch_project_fourier(m, a.prm, R, u, S(stream)));
   ProjTables T;
-  {
-    static_assert(kProjN <= kMaxGaussRule, "projection rule larger than the Gauss rule builder");
-    double x[kProjN], w[kProjN], pv[kMaxP + 1];
-    if (!gauss_rule(kProjN, x, w)) return CVWENO_ERR_ARG;
-    for (int q = 0; q < kProjN; ++q) {
-      T.x[q] = (float)x[q];
-      T.w[q] = (float)w[q];
-      legendre_values(x[q], kMaxP, pv);
-      for (int mm = 0; mm <= kMaxP; ++mm) T.P[q][mm] = (float)pv[mm];
-    }
+  for (int q = 0; q < kProjN; ++q) {
+    T.x[q] = (float)R.x[q];
+    for (int mm = 0; mm <= kMaxP; ++mm) T.wP[q][mm] = (float)(R.w[q] * R.P[q][mm]);
   }
   if (m->kind == CVWENO_CG) {
     int blocks = (int)((m->nnode + 255) / 256);
@@ -617,10 +829,18 @@ cvweno_status cvweno_project(cvweno_mesh m, int ic_type, const double* ic_params
     project_cg_kernel<<<blocks, 256, 0, S(stream)>>>(a, T, m->p, m->nnx, m->nny, m->d_cg_xg);
     return cuda_status(cudaGetLastError());
   }
-  int blocks = (int)((m->ncell + 127) / 128);
-  if (blocks > 65535) blocks = 65535;
-  project_kernel<<<blocks, 128, 0, S(stream)>>>(a, T);
-  return cuda_status(cudaGetLastError());
+  cudaError_t e = cudaErrorNotSupported;
+  switch (m->dim * 10 + m->p) {
+    case 11: e = launch_project<1, 2>(a, T, S(stream)); break;
+    case 12: e = launch_project<1, 3>(a, T, S(stream)); break;
+    case 13: e = launch_project<1, 4>(a, T, S(stream)); break;
+    case 14: e = launch_project<1, 5>(a, T, S(stream)); break;
+    case 21: e = launch_project<2, 2>(a, T, S(stream)); break;
+    case 22: e = launch_project<2, 3>(a, T, S(stream)); break;
+    case 23: e = launch_project<2, 4>(a, T, S(stream)); break;
+    case 24: e = launch_project<2, 5>(a, T, S(stream)); break;
+  }
+  return cuda_status(e);
 }
 
 cvweno_status cvweno_vertex_data(cvweno_mesh m, const float* u, float* tstar, void* stream) {
@@ -693,18 +913,36 @@ cvweno_status cvweno_max_wavespeed(cvweno_mesh m, const float* u, double* lam, v
   cudaStream_t s = S(stream);
   StageArgs a = base_args(m);
   a.u_in = u;
-  a.lambda_out = m->d_lambda;
-  a.mode = kModeSensorOnly;
-  cudaError_t e = launch(m, a, s);
-  if (e == cudaSuccess) {
-    max_partial<<<kRedBlocks, kRedThreads, 0, s>>>(m->d_lambda, m->ncell, m->d_red);
-    finish_reduce<<<1, kRedThreads, 0, s>>>(m->d_red, kRedBlocks, 1, m->d_red + kRedBlocks);
-    e = cudaGetLastError();
+  cudaError_t e;
+  double* out = m->d_red + kRedOut;
+  if (m->kind == CVWENO_CG || (m->desc.system != CVWENO_EULER && m->desc.params.lambda_const > 0.0)) {
+    // CG cells' polynomials come from the stage kernel; a constant speed needs no pass, but takes
+    // this way for the same answer on an empty status
+    a.lambda_out = m->d_lambda;
+    a.mode = kModeSensorOnly;
+    e = launch(m, a, s);
+    if (e == cudaSuccess) {
+      max_partial<<<kRedBlocks, kRedThreads, 0, s>>>(m->d_lambda, m->ncell, m->d_red);
+      finish_reduce<<<1, kRedThreads, 0, s>>>(m->d_red, kRedBlocks, 1, out);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_red, out, sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e != cudaSuccess) return CVWENO_ERR_CUDA;
+    cvweno_status st = read_status(m, s);  // synchronises
+    if (st != CVWENO_OK) return st;
+  } else {
+    // one pass over the cells, one copy of the maximum and the status word
+    unsigned* slots = reinterpret_cast<unsigned*>(out + 8);
+    const MaxSlots ms{slots, slots + 1, out, reinterpret_cast<int*>(out + 1)};
+    e = m->desc.system == CVWENO_EULER ? launch_wavespeed_euler(m, a, ms, s) : launch_wavespeed_scalar(m, a, ms, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_red, out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return CVWENO_ERR_CUDA;
+    int bits;
+    memcpy(&bits, m->h_red + 1, sizeof(bits));
+    cvweno_status st = take_status(m, bits, s);
+    if (st != CVWENO_OK) return st;
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_red, m->d_red + kRedBlocks, sizeof(double), cudaMemcpyDeviceToHost, s);
-  if (e != cudaSuccess) return CVWENO_ERR_CUDA;
-  cvweno_status st = read_status(m, s);  // synchronises
-  if (st != CVWENO_OK) return st;
   *lam = m->h_red[0];
   return CVWENO_OK;
 }
@@ -744,9 +982,9 @@ cvweno_status cvweno_mass_total(cvweno_mesh m, const float* u, double* totals, v
     // sum_j ML_j u_j with ML_j = ml1x(I mod p) ml1y(J mod p)
     sum_cg_partial<<<kRedBlocks, kRedThreads, 0, s>>>(u, m->nnx, m->nny, m->p, m->d_cg_ml, m->d_cg_ml + (kMaxP + 1),
                                                      m->d_red);
-    finish_reduce<<<1, kRedThreads, 0, s>>>(m->d_red, kRedBlocks, 0, m->d_red + kRedBlocks);
+    finish_reduce<<<1, kRedThreads, 0, s>>>(m->d_red, kRedBlocks, 0, m->d_red + kRedOut);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_red, m->d_red + kRedBlocks, sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_red, m->d_red + kRedOut, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return CVWENO_ERR_CUDA;
     totals[0] = m->h_red[0];
@@ -754,14 +992,13 @@ cvweno_status cvweno_mass_total(cvweno_mesh m, const float* u, double* totals, v
   }
   // int_{K_e} u_h = |K_e| * (Legendre mode 0)
   const double vol = m->dim == 2 ? m->dx * m->dy : m->dx;
-  for (int v = 0; v < m->nvar; ++v) {
-    const float* base = u + (size_t)v * m->ncell * m->nd;
-    sum_mode0_partial<<<kRedBlocks, kRedThreads, 0, s>>>(base, m->ncell, m->nd, m->d_red);
-    finish_reduce<<<1, kRedThreads, 0, s>>>(m->d_red, kRedBlocks, 0, m->d_red + kRedBlocks + v);
-  }
+  const int64_t nb = (m->ncell + kRedThreads - 1) / kRedThreads;
+  unsigned* slots = reinterpret_cast<unsigned*>(m->d_red + kRedOut + 8);
+  sum_mode0_kernel<<<dim3((unsigned)(nb < kRedBlocks ? nb : kRedBlocks), m->nvar), kRedThreads, 0, s>>>(
+      u, m->ncell, m->nd, m->d_red, m->d_red + kRedOut, slots + 2);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(m->h_red, m->d_red + kRedBlocks, sizeof(double) * m->nvar, cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(m->h_red, m->d_red + kRedOut, sizeof(double) * m->nvar, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return CVWENO_ERR_CUDA;
   for (int v = 0; v < m->nvar; ++v) totals[v] = m->h_red[v] * vol;

@@ -254,6 +254,7 @@ struct StageArgs {
   int r;
   int sc, sensor_mode;
   int limit_all;       // kModeLimit: limit every cell, not only gamma_e < c_gamma
+  int limit_pos;       // Euler RK stage: positivity limiter on the result
   // surrogate sensor (2D DG scalar): packed network weights (MlpPacked) or null, the
   // confidence below which the plain sensor decides, a fallback counter (may be null),
   // and the features output of kModeFeatures ([ncell][12])
@@ -280,6 +281,15 @@ struct StageArgs {
   int64_t lim_out;     // floats writable at u_out
   int64_t lim_cell;    // cells: the extent of the per-cell outputs and of rloc (in cells)
 #endif
+};
+
+// Where a maximum over the mesh is formed (device): the running maximum (bits of a
+// non-negative float) and the blocks done, both zero between calls, and the result.
+struct MaxSlots {
+  unsigned* best;
+  unsigned* done;
+  double* max;     // the maximum,
+  int* status;     // and the mesh's status word at that time
 };
 
 // Sets the extents of the checked build's bounds checks (nothing in the normal build).
@@ -388,6 +398,10 @@ cudaError_t launch_positivity(const cvweno_mesh_s* m, const StageArgs& a, float*
 cudaError_t launch_tab_image(int dim, int p, const void* t, float* dst, cudaStream_t s);
 // dg_scalar_2d.cu: likewise PackedImage<dim, p> (packed_image_floats(dim, p) floats)
 cudaError_t launch_packed_image(int dim, int p, const void* t, float* dst, cudaStream_t s);
+// dg_euler.cu, dg_scalar_2d.cu: max over the cells of a.u_in of lambda_e at the volume and face
+// Gauss nodes (scalar: DG laws without a constant wave speed)
+cudaError_t launch_wavespeed_euler(const cvweno_mesh_s* m, const StageArgs& a, const MaxSlots& out, cudaStream_t s);
+cudaError_t launch_wavespeed_scalar(const cvweno_mesh_s* m, const StageArgs& a, const MaxSlots& out, cudaStream_t s);
 // cg_scalar.cu
 cudaError_t launch_stage_cg(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t s);
 // api.cu: the stage arguments common to every launch on mesh m (no state pointers, no RK)

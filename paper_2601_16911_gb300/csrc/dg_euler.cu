@@ -124,6 +124,121 @@ __device__ __forceinline__ void hll_dev(float g, const EulerMean& M, const f2 (&
   }
 }
 
+// Calls f(ua, ub, mid) for every pair of node rows of a cell with modes c: the volume nodes (x group
+// q, rows +eta_h (a) and -eta_h (b)) and the face nodes: the ends +-1 are one more x group and
+// one more row pair, whose Legendre values are all 1 (their corner combination is left out).
+// mid: the row pair is the one middle row.
+template <int N, int MP, class F>
+__device__ __forceinline__ void for_node_groups(const float* img, const f2 (&c)[NV][N][MP], F&& f) {
+  using Img = PackedImage<2, N - 1>;
+  constexpr int NG = Img::NG;
+#pragma unroll 1
+  for (int q = 0; q <= NG; ++q) {
+    f2 b[MP], tb[NV][N];
+    load_pairs<MP>(img + Img::BX + 2 * MP * (q < NG ? q : 0), b);
+    if (q == NG) {
+#pragma unroll
+      for (int p = 0; p < MP; ++p) b[p] = mk2(1.0f, 1.0f);
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+      for (int my = 0; my < N; ++my) {
+        f2 s = mul2(b[0], c[v][my][0]);
+#pragma unroll
+        for (int p = 1; p < MP; ++p) s = fma2(b[p], c[v][my][p], s);
+        tb[v][my] = mk2(s.x + s.y, s.x - s.y);
+      }
+#pragma unroll 1
+    for (int h = 0; h < (q < NG ? NG + 1 : NG); ++h) {
+      f2 by[N], ua[NV], ub[NV];
+      load_pairs<N>(img + Img::BY + 2 * N * (h < NG ? h : 0), by);
+      if (h == NG) {
+#pragma unroll
+        for (int my = 0; my < N; ++my) by[my] = mk2(1.0f, 1.0f);
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        f2 e = mul2(by[0], tb[v][0]), o = mul2(by[1], tb[v][1]);
+#pragma unroll
+        for (int my = 2; my < N; ++my) {
+          if (my & 1) o = fma2(by[my], tb[v][my], o);
+          else e = fma2(by[my], tb[v][my], e);
+        }
+        ua[v] = add2(e, o);
+        ub[v] = sub2(e, o);
+      }
+      f(ua, ub, (N & 1) && h == NG - 1);
+    }
+  }
+}
+
+// Positivity limiter of one cell (readings P1-P4; Zhang and Shu's scaling limiter): the density's
+// non-mean modes are scaled by th1 to keep rho >= eps_e at the volume and face Gauss nodes, then
+// all non-mean modes by th2 to keep p >= eps_e, the root of p(U_bar + t dU) = eps_e found by 40
+// bisection steps at the nodes that violate it.  False (and c unchanged) where the mean is not
+// admissible.
+template <int N, int MP>
+__device__ __forceinline__ bool limit_positivity(float g, const float* img, f2 (&c)[NV][N][MP], float& th1, float& th2) {
+  float Ub[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) Ub[v] = c[v][0][0].x;
+  auto pres = [&](const float (&U)[NV]) { return (g - 1.0f) * (U[3] - 0.5f * (U[1] * U[1] + U[2] * U[2]) / U[0]); };
+  const float pb = pres(Ub);
+  th1 = th2 = 1.0f;
+  if (!(Ub[0] > 0.0f && pb > 0.0f)) return false;
+  const float eps = 1e-3f * fminf(Ub[0], pb);
+  // the smallest density, and whether any node's pressure (with th1 = 1) is below eps
+  float rmin = Ub[0];
+  bool low = false;
+  for_node_groups<N, MP>(img, c, [&](const f2 (&ua)[NV], const f2 (&ub)[NV], bool mid) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k >= 2 && mid) continue;
+      const f2 (&u)[NV] = k < 2 ? ua : ub;
+      const float U[NV] = {k & 1 ? u[0].y : u[0].x, k & 1 ? u[1].y : u[1].x, k & 1 ? u[2].y : u[2].x, k & 1 ? u[3].y : u[3].x};
+      rmin = fminf(rmin, U[0]);
+      low |= !(pres(U) >= eps);
+    }
+  });
+  if (rmin < eps) th1 = fminf(1.0f, (Ub[0] - eps) / (Ub[0] - rmin));
+  // (the pressures are taken again where the density changed or a node was low)
+  if (low || th1 < 1.0f)
+    for_node_groups<N, MP>(img, c, [&](const f2 (&ua)[NV], const f2 (&ub)[NV], bool mid) {
+#pragma unroll 1
+      for (int k = 0; k < 4; ++k) {
+        if (k >= 2 && mid) continue;
+        float U[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) U[v] = k == 0 ? ua[v].x : k == 1 ? ua[v].y : k == 2 ? ub[v].x : ub[v].y;
+        U[0] = fmaf(th1, U[0] - Ub[0], Ub[0]);
+        if (!(pres(U) < eps)) continue;
+        float lo = 0.0f, hi = 1.0f;  // p(lo) >= eps > p(hi)
+#pragma unroll 1
+        for (int it = 0; it < 40; ++it) {
+          const float t = 0.5f * (lo + hi);
+          float Ut[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) Ut[v] = fmaf(t, U[v] - Ub[v], Ub[v]);
+          if (pres(Ut) >= eps) lo = t; else hi = t;
+        }
+        th2 = fminf(th2, lo);
+      }
+    });
+  if (th1 < 1.0f || th2 < 1.0f) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const f2 f = dup2((v == 0 ? th1 : 1.0f) * th2);
+#pragma unroll
+      for (int my = 0; my < N; ++my)
+#pragma unroll
+        for (int p = 0; p < MP; ++p) c[v][my][p] = mul2(c[v][my][p], f);
+      c[v][0][0].x = Ub[v];
+    }
+  }
+  return true;
+}
+
 // Shared-memory layout of the Euler stage tile (floats): four variables' cells, each laid
 // out as the scalar tile's (TileLayout), then the density's vertex data (later the
 // indicator), the node tabulations, the faces' projected fluxes (mode pairs,
@@ -170,7 +285,8 @@ __host__ __device__ constexpr int euler_threads() {
 //   volume pass B, only where the viscosity (1 - gamma_e) nu_e is non-zero: the viscous term.
 // The SC weights of troubled cells (stage d) are taken before that by all threads of the
 // tile, (cell, node group) and (cell, variable) at a time.
-template <int P, int TX, int TY>
+// POS: the positivity limiter on the stage's result, in registers, before it is written.
+template <int P, int TX, int TY, bool POS>
 __global__ void __launch_bounds__(euler_threads<P, TX, TY>(), (euler_min_ctas<P, TX, TY>()))
     dg_euler_stage(const __grid_constant__ StageArgs a, const __grid_constant__ PackedTables<2, P> T) {
   using E = EulerLayout<P, TX, TY>;
@@ -668,6 +784,18 @@ __global__ void __launch_bounds__(euler_threads<P, TX, TY>(), (euler_min_ctas<P,
   // variable go out together.  16-byte loads and stores where both states are 16-byte aligned.
   f2 fin = mk2(0.0f, 0.0f);  // stays zero while every du/dt is finite
   const bool v16 = ND % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.u_out) | reinterpret_cast<uintptr_t>(a.u_n)) & 15) == 0;
+  auto write_var = [&](int v) {
+    auto val = [&](int m) { return (m % N) & 1 ? r[v][m / N][m % N / 2].y : r[v][m / N][m % N / 2].x; };
+    float* out = a.u_out + ((size_t)v * ncell + cell) * ND;
+    if (v16) {
+#pragma unroll
+      for (int q = 0; q < ND / 4; ++q)
+        reinterpret_cast<float4*>(out)[q] = make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
+    } else {
+#pragma unroll
+      for (int m = 0; m < ND; ++m) out[m] = val(m);
+    }
+  };
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     f2 c[N][MP], n[N][MP];
@@ -701,30 +829,27 @@ __global__ void __launch_bounds__(euler_threads<P, TX, TY>(), (euler_min_ctas<P,
           d = fma2(dup2(a.dt), d, c[my][p]);
           if (with_un) d = fma2(dup2(a.rk_b), sub2(d, n[my][p]), n[my][p]);
         }
-        c[my][p] = d;
+        r[v][my][p] = d;
       }
-    auto val = [&](int m) { return (m % N) & 1 ? c[m / N][m % N / 2].y : c[m / N][m % N / 2].x; };
-    float* out = a.u_out + ((size_t)v * ncell + cell) * ND;
-    if (v16) {
+    if constexpr (!POS) write_var(v);
+  }
+  if constexpr (POS) {
+    float th1, th2;
+    bad |= !limit_positivity<N, MP>(g, img, r, th1, th2);
 #pragma unroll
-      for (int q = 0; q < ND / 4; ++q)
-        reinterpret_cast<float4*>(out)[q] = make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
-    } else {
-#pragma unroll
-      for (int m = 0; m < ND; ++m) out[m] = val(m);
-    }
+    for (int v = 0; v < NV; ++v) write_var(v);
   }
   if (!(fin.x + fin.y == 0.0f)) atomicOr(a.status, kStatNonfinite);
   }  // active
   if (bad) atomicOr(a.status, kStatPositivity);
 }
 
-template <int P, int TX, int TY>
+template <int P, int TX, int TY, bool POS>
 cudaError_t launch_euler(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t s) {
   using Tb = DgTables<2, P>;
   constexpr size_t smem = EulerLayout<P, TX, TY>::BYTES;
   static_assert(smem <= 220 * 1024, "tile too large for shared memory");
-  auto kern = dg_euler_stage<P, TX, TY>;
+  auto kern = dg_euler_stage<P, TX, TY, POS>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -735,111 +860,110 @@ cudaError_t launch_euler(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_
 }
 
 
-// ---- positivity limiter (readings P1-P4; Zhang and Shu's scaling limiter) --------------------
-// One thread per cell, cell-local (no neighbours, so it may run in place).  The cell's
-// coefficients of all four variables are staged in shared memory (mode-major per
-// thread); every volume and face Gauss node is evaluated from them, the density's
-// non-mean modes are scaled to keep rho >= eps_e, then all non-mean modes to keep
-// p >= eps_e, the root of p(U_bar + t dU) = eps_e found by 40 bisection steps.
+// Cell-local work outside the stage: one thread per cell, its coefficients in registers.
 template <int P>
-struct PosThreads {
-  static constexpr int value = P >= 4 ? 64 : 128;  // the staged coefficients stay under 48 KB
-};
+__device__ __forceinline__ void load_state(const StageArgs& a, const float* u, int64_t cell, int64_t ncell, f2 (&c)[NV][P + 1][(P + 2) / 2]) {
+  constexpr int N = P + 1, ND = N * N, MP = (N + 1) / 2;
+  const bool v16 = ND % 4 == 0 && (reinterpret_cast<uintptr_t>(u) & 15) == 0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const float* src = u + ((int64_t)v * ncell + cell) * ND;
+    if (v16) {
+#pragma unroll
+      for (int q = 0; q < ND / 4; ++q) {
+        const float4 x = reinterpret_cast<const float4*>(src)[q];
+        const int m = 4 * q, m2 = m + 2;
+        c[v][m / N][m % N / 2] = mk2(x.x, x.y);
+        c[v][m2 / N][m2 % N / 2] = mk2(x.z, x.w);
+      }
+    } else {
+#pragma unroll
+      for (int my = 0; my < N; ++my)
+#pragma unroll
+        for (int p = 0; p < MP; ++p) c[v][my][p] = mk2(src[2 * p + N * my], 2 * p + 1 < N ? src[2 * p + 1 + N * my] : 0.0f);
+    }
+  }
+}
+constexpr int kCellThreads = 128;
 
+// The node tabulations into shared memory (plain copies).
 template <int P>
-__global__ void __launch_bounds__(PosThreads<P>::value)
-    euler_positivity_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ DgTables<2, P> T,
-                            float* __restrict__ theta_out) {
-  constexpr int N = P + 1, ND = N * N, NTH = PosThreads<P>::value;
-  __shared__ float sc[NV * ND][NTH];
+__device__ __forceinline__ void load_image(const float* img, float* s) {
+  for (int f = threadIdx.x; f < PackedImage<2, P>::FLOATS; f += kCellThreads) s[f] = img[f];
+  __syncthreads();
+}
+
+// The positivity limiter on its own: u_in -> u_out (may be the same array), theta per cell.
+template <int P>
+__global__ void __launch_bounds__(kCellThreads)
+    euler_positivity_kernel(const __grid_constant__ StageArgs a, float* __restrict__ theta_out) {
+  constexpr int N = P + 1, ND = N * N, MP = (N + 1) / 2;
+  __shared__ __align__(16) float img[PackedImage<2, P>::FLOATS];
+  load_image<P>(a.pk_img, img);
   const int64_t ncell = (int64_t)a.nx * a.ny;
-  const int64_t cell = (int64_t)blockIdx.x * NTH + threadIdx.x;
+  const int64_t cell = (int64_t)blockIdx.x * kCellThreads + threadIdx.x;
   if (cell >= ncell) return;
   if (!CVW_SPAN(a.status, cell, 1, a.lim_cell) ||
       !CVW_SPAN(a.status, ((NV - 1) * ncell + cell) * ND, ND, a.lim_in < a.lim_out ? a.lim_in : a.lim_out))
     return;
-  const float g = a.gas_gamma;
-#pragma unroll 1
-  for (int k = 0; k < NV * ND; ++k) {
-    const int v = k / ND, m = k - v * ND;
-    sc[k][threadIdx.x] = a.u_in[((int64_t)v * ncell + cell) * ND + m];
-  }
-  float Ub[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) Ub[v] = sc[v * ND][threadIdx.x];
-  const float pb = (g - 1.0f) * (Ub[3] - 0.5f * (Ub[1] * Ub[1] + Ub[2] * Ub[2]) / Ub[0]);
-  float th1 = 1.0f, th2 = 1.0f;
-  const bool admissible = Ub[0] > 0.0f && pb > 0.0f;
-  if (admissible) {
-    const float eps = 1e-3f * fminf(Ub[0], pb);
-    // node q: volume (q < N^2: qx + N qy), then faces x = +1, x = -1, y = +1, y = -1
-    auto value = [&](int v, int q) -> float {
-      float s = 0.0f;
-#pragma unroll 1
-      for (int my = 0; my < N; ++my) {
-        float row = 0.0f;
-#pragma unroll
-        for (int mx = 0; mx < N; ++mx) {
-          float bx;
-          if (q < ND) bx = T.B[q % N][mx];
-          else if (q < ND + 2 * N) bx = (q < ND + N || !(mx & 1)) ? 1.0f : -1.0f;
-          else bx = T.B[(q - ND) % N][mx];
-          row = fmaf(bx, sc[v * ND + mx + N * my][threadIdx.x], row);
-        }
-        float by;
-        if (q < ND) by = T.B[q / N][my];
-        else if (q < ND + 2 * N) by = T.B[(q - ND) % N][my];
-        else by = (q < ND + 3 * N || !(my & 1)) ? 1.0f : -1.0f;
-        s = fmaf(by, row, s);
-      }
-      return s;
-    };
-    constexpr int NPT = ND + 4 * N;
-    float rmin = Ub[0];
-#pragma unroll 1
-    for (int q = 0; q < NPT; ++q) rmin = fminf(rmin, value(0, q));
-    if (rmin < eps) th1 = fminf(1.0f, (Ub[0] - eps) / (Ub[0] - rmin));
-    auto pres = [&](const float* U) {
-      return (g - 1.0f) * (U[3] - 0.5f * (U[1] * U[1] + U[2] * U[2]) / U[0]);
-    };
-#pragma unroll 1
-    for (int q = 0; q < NPT; ++q) {
-      float Uq[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Uq[v] = value(v, q);
-      Uq[0] = fmaf(th1, Uq[0] - Ub[0], Ub[0]);
-      if (!(pres(Uq) < eps)) continue;
-      float lo = 0.0f, hi = 1.0f;  // p(lo) >= eps > p(hi)
-#pragma unroll 1
-      for (int it = 0; it < 40; ++it) {
-        const float t = 0.5f * (lo + hi);
-        float Ut[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) Ut[v] = fmaf(t, Uq[v] - Ub[v], Ub[v]);
-        if (pres(Ut) >= eps) lo = t; else hi = t;
-      }
-      th2 = fminf(th2, lo);
-    }
-  } else {
-    atomicOr(a.status, kStatPositivity);
-  }
-#pragma unroll 1
-  for (int k = 0; k < NV * ND; ++k) {
-    const int v = k / ND, m = k - v * ND;
-    const float f = m == 0 ? 1.0f : (v == 0 ? th1 : 1.0f) * th2;
-    a.u_out[((int64_t)v * ncell + cell) * ND + m] = sc[k][threadIdx.x] * f;
-  }
+  f2 c[NV][N][MP];
+  load_state<P>(a, a.u_in, cell, ncell, c);
+  float th1, th2;
+  if (!limit_positivity<N, MP>(a.gas_gamma, img, c, th1, th2)) atomicOr(a.status, kStatPositivity);
   if (theta_out) theta_out[cell] = th1 * th2;
+  if (a.u_out == a.u_in && th1 == 1.0f && th2 == 1.0f) return;  // in place: nothing changed
+  const bool v16 = ND % 4 == 0 && (reinterpret_cast<uintptr_t>(a.u_out) & 15) == 0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    float* out = a.u_out + ((int64_t)v * ncell + cell) * ND;
+    auto val = [&](int m) { return (m % N) & 1 ? c[v][m / N][m % N / 2].y : c[v][m / N][m % N / 2].x; };
+    if (v16) {
+#pragma unroll
+      for (int q = 0; q < ND / 4; ++q)
+        reinterpret_cast<float4*>(out)[q] = make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
+    } else {
+#pragma unroll
+      for (int m = 0; m < ND; ++m) out[m] = val(m);
+    }
+  }
+}
+
+// max lambda_e = max(|v| + c) over every cell's volume and face Gauss nodes; non-positive density
+// or pressure at a node raises the status bit, as in the stage.
+template <int P>
+__global__ void __launch_bounds__(kCellThreads)
+    euler_wavespeed_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ MaxSlots out) {
+  constexpr int N = P + 1, ND = N * N, MP = (N + 1) / 2;
+  __shared__ __align__(16) float img[PackedImage<2, P>::FLOATS];
+  load_image<P>(a.pk_img, img);
+  const int64_t ncell = (int64_t)a.nx * a.ny;
+  float lam = 0.0f;
+  bool bad = false;
+  for (int64_t cell = (int64_t)blockIdx.x * kCellThreads + threadIdx.x; cell < ncell; cell += (int64_t)gridDim.x * kCellThreads) {
+    if (!CVW_SPAN(a.status, ((NV - 1) * ncell + cell) * ND, ND, a.lim_in)) continue;
+    f2 c[NV][N][MP];
+    load_state<P>(a, a.u_in, cell, ncell, c);
+    for_node_groups<N, MP>(img, c, [&](const f2 (&ua)[NV], const f2 (&ub)[NV], bool mid) {
+      f2 vn, cs;
+      lam = fmaxf(lam, euler_wave(a.gas_gamma, ua, 0, vn, cs, bad));
+      if (!mid) lam = fmaxf(lam, euler_wave(a.gas_gamma, ub, 0, vn, cs, bad));
+    });
+  }
+  if (bad) atomicOr(a.status, kStatPositivity);
+  finish_max(lam, a.status, out);
 }
 
 template <int P>
 cudaError_t launch_positivity_p(const cvweno_mesh_s* m, const StageArgs& a, float* theta, cudaStream_t s) {
-  using Tb = DgTables<2, P>;
-  if (m->tables_bytes != sizeof(Tb)) return cudaErrorInvalidValue;
   const int64_t ncell = (int64_t)a.nx * a.ny;
-  constexpr int nth = PosThreads<P>::value;
-  euler_positivity_kernel<P><<<(unsigned)((ncell + nth - 1) / nth), nth, 0, s>>>(a, *static_cast<const Tb*>(m->tables),
-                                                                                  theta);
+  euler_positivity_kernel<P><<<(unsigned)((ncell + kCellThreads - 1) / kCellThreads), kCellThreads, 0, s>>>(a, theta);
+  return cudaGetLastError();
+}
+
+template <int P>
+cudaError_t launch_wavespeed_p(const StageArgs& a, const MaxSlots& out, cudaStream_t s) {
+  const int64_t ncell = (int64_t)a.nx * a.ny, blocks = (ncell + kCellThreads - 1) / kCellThreads;
+  euler_wavespeed_kernel<P><<<(unsigned)(blocks < 1216 ? blocks : 1216), kCellThreads, 0, s>>>(a, out);
   return cudaGetLastError();
 }
 
@@ -847,11 +971,15 @@ cudaError_t launch_positivity_p(const cvweno_mesh_s* m, const StageArgs& a, floa
 
 cudaError_t launch_stage_euler(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t s) {
   if (m->dim != 2) return cudaErrorNotSupported;
-  switch (m->p) {
-    case 1: return launch_euler<1, 16, 8>(m, a, s);
-    case 2: return launch_euler<2, 16, 8>(m, a, s);
-    case 3: return launch_euler<3, 16, 8>(m, a, s);
-    case 4: return launch_euler<4, 8, 8>(m, a, s);
+  switch (m->p * 2 + (a.limit_pos ? 1 : 0)) {
+    case 2: return launch_euler<1, 16, 8, false>(m, a, s);
+    case 3: return launch_euler<1, 16, 8, true>(m, a, s);
+    case 4: return launch_euler<2, 16, 8, false>(m, a, s);
+    case 5: return launch_euler<2, 16, 8, true>(m, a, s);
+    case 6: return launch_euler<3, 16, 8, false>(m, a, s);
+    case 7: return launch_euler<3, 16, 8, true>(m, a, s);
+    case 8: return launch_euler<4, 8, 8, false>(m, a, s);
+    case 9: return launch_euler<4, 8, 8, true>(m, a, s);
     default: return cudaErrorNotSupported;
   }
 }
@@ -863,6 +991,16 @@ cudaError_t launch_positivity(const cvweno_mesh_s* m, const StageArgs& a, float*
     case 2: return launch_positivity_p<2>(m, a, theta, s);
     case 3: return launch_positivity_p<3>(m, a, theta, s);
     case 4: return launch_positivity_p<4>(m, a, theta, s);
+    default: return cudaErrorNotSupported;
+  }
+}
+
+cudaError_t launch_wavespeed_euler(const cvweno_mesh_s* m, const StageArgs& a, const MaxSlots& out, cudaStream_t s) {
+  switch (m->p) {
+    case 1: return launch_wavespeed_p<1>(a, out, s);
+    case 2: return launch_wavespeed_p<2>(a, out, s);
+    case 3: return launch_wavespeed_p<3>(a, out, s);
+    case 4: return launch_wavespeed_p<4>(a, out, s);
     default: return cudaErrorNotSupported;
   }
 }

@@ -58,6 +58,100 @@ cudaError_t launch_packed_image(int dim, int p, const void* t, float* dst, cudaS
   }
 }
 
+namespace {
+// max lambda_e over the volume and face Gauss nodes: one thread per cell, its coefficients in
+// registers; the ends +-1 are one more x group and one more row pair, whose Legendre values
+// are all 1 (their corner combination is left out).
+constexpr int kSpeedThreads = 128;
+template <int DIM, int P, int SYS>
+__global__ void __launch_bounds__(kSpeedThreads)
+    scalar_wavespeed_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ MaxSlots out) {
+  using Img = PackedImage<DIM, P>;
+  constexpr int N = Img::N, NY1 = Img::NY1, MP = Img::MP, NG = Img::NG, ND = N * NY1;
+  __shared__ __align__(16) float img[Img::FLOATS];
+  for (int f = threadIdx.x; f < Img::FLOATS; f += kSpeedThreads) img[f] = a.pk_img[f];
+  __syncthreads();
+  const int64_t ncell = (int64_t)a.nx * (DIM == 2 ? a.ny : 1);
+  float lam = 0.0f;
+  for (int64_t cell = (int64_t)blockIdx.x * kSpeedThreads + threadIdx.x; cell < ncell;
+       cell += (int64_t)gridDim.x * kSpeedThreads) {
+    if (!CVW_SPAN(a.status, cell * ND, ND, a.lim_in)) continue;
+    f2 c[NY1][MP];
+#pragma unroll
+    for (int my = 0; my < NY1; ++my)
+#pragma unroll
+      for (int p = 0; p < MP; ++p)
+        c[my][p] = mk2(a.u_in[cell * ND + 2 * p + N * my], 2 * p + 1 < N ? a.u_in[cell * ND + 2 * p + 1 + N * my] : 0.0f);
+    const float ubar = c[0][0].x;
+    c[0][0].x = 0.0f;
+    const ScalarLaw<SYS, DIM> law(a, ubar);
+    auto take = [&](f2 d) { lam = fmaxf(lam, fmaxf(law.speed(ubar + d.x), law.speed(ubar + d.y))); };
+#pragma unroll 1
+    for (int g = 0; g <= NG; ++g) {
+      f2 b[MP], tb[NY1];
+      load_pairs<MP>(img + Img::BX + 2 * MP * (g < NG ? g : 0), b);
+#pragma unroll
+      for (int my = 0; my < NY1; ++my) {
+        f2 s = g < NG ? mul2(b[0], c[my][0]) : c[my][0];
+#pragma unroll
+        for (int p = 1; p < MP; ++p) s = g < NG ? fma2(b[p], c[my][p], s) : add2(c[my][p], s);
+        tb[my] = mk2(s.x + s.y, s.x - s.y);
+      }
+      if constexpr (DIM == 1) {
+        take(tb[0]);
+      } else {
+#pragma unroll 1
+        for (int h = 0; h < (g < NG ? NG + 1 : NG); ++h) {
+          f2 by[N];
+          load_pairs<N>(img + Img::BY + 2 * N * (h < NG ? h : 0), by);
+          f2 e = h < NG ? mul2(by[0], tb[0]) : tb[0], o = h < NG ? mul2(by[1], tb[NY1 > 1 ? 1 : 0]) : tb[NY1 > 1 ? 1 : 0];
+#pragma unroll
+          for (int my = 2; my < NY1; ++my) {
+            if (my & 1) o = h < NG ? fma2(by[my], tb[my], o) : add2(tb[my], o);
+            else e = h < NG ? fma2(by[my], tb[my], e) : add2(tb[my], e);
+          }
+          take(add2(e, o));
+          take(sub2(e, o));
+        }
+      }
+    }
+  }
+  finish_max(lam, a.status, out);
+}
+
+template <int DIM, int P>
+cudaError_t launch_wavespeed_t(int system, const StageArgs& a, const MaxSlots& out, cudaStream_t s) {
+  const int64_t ncell = (int64_t)a.nx * (DIM == 2 ? a.ny : 1), n = (ncell + kSpeedThreads - 1) / kSpeedThreads;
+  const unsigned blocks = (unsigned)(n < 1216 ? n : 1216);  // 8 per SM
+  switch (system) {
+    case CVWENO_BURGERS: scalar_wavespeed_kernel<DIM, P, CVWENO_BURGERS><<<blocks, kSpeedThreads, 0, s>>>(a, out); break;
+    case CVWENO_LINADV: scalar_wavespeed_kernel<DIM, P, CVWENO_LINADV><<<blocks, kSpeedThreads, 0, s>>>(a, out); break;
+    case CVWENO_KPP:
+      if constexpr (DIM == 2) {
+        scalar_wavespeed_kernel<DIM, P, CVWENO_KPP><<<blocks, kSpeedThreads, 0, s>>>(a, out);
+        break;
+      }
+      return cudaErrorNotSupported;
+    default: return cudaErrorNotSupported;
+  }
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_wavespeed_scalar(const cvweno_mesh_s* m, const StageArgs& a, const MaxSlots& out, cudaStream_t s) {
+  switch (m->dim * 10 + m->p) {
+    case 11: return launch_wavespeed_t<1, 1>(m->desc.system, a, out, s);
+    case 12: return launch_wavespeed_t<1, 2>(m->desc.system, a, out, s);
+    case 13: return launch_wavespeed_t<1, 3>(m->desc.system, a, out, s);
+    case 14: return launch_wavespeed_t<1, 4>(m->desc.system, a, out, s);
+    case 21: return launch_wavespeed_t<2, 1>(m->desc.system, a, out, s);
+    case 22: return launch_wavespeed_t<2, 2>(m->desc.system, a, out, s);
+    case 23: return launch_wavespeed_t<2, 3>(m->desc.system, a, out, s);
+    case 24: return launch_wavespeed_t<2, 4>(m->desc.system, a, out, s);
+    default: return cudaErrorNotSupported;
+  }
+}
+
 }  // namespace cvw
 
 namespace cvw {

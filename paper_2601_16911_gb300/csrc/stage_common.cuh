@@ -361,4 +361,26 @@ __device__ __forceinline__ void stage_rows16_inner(float* dst, int dstv, int* ph
   }
 }
 
+// Ends a kernel that maximises x >= 0 over its threads (every thread calls it once): the block's
+// maximum goes into the slots; the last block publishes the result with the status word
+// and leaves the slots zero for the next call.
+__device__ __forceinline__ void finish_max(float x, int* status, const MaxSlots& out) {
+  __shared__ unsigned best;
+  if (threadIdx.x == 0) best = 0;
+  __syncthreads();
+  const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(x));
+  if ((threadIdx.x & 31) == 0) atomicMax(&best, w);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicMax(out.best, best);
+    __threadfence();
+    if (atomicAdd(out.done, 1u) == gridDim.x - 1) {
+      __threadfence();
+      *out.max = (double)__uint_as_float(atomicExch(out.best, 0u));
+      *out.status = atomicOr(status, 0);
+      *out.done = 0;
+    }
+  }
+}
+
 }  // namespace cvw
