@@ -60,14 +60,13 @@ cudaError_t launch_packed_image(int dim, int p, const void* t, float* dst, cudaS
 
 namespace {
 // max lambda_e over the volume and face Gauss nodes: one thread per cell, its coefficients in
-// registers; the ends +-1 are one more x group and one more row pair, whose Legendre values
-// are all 1 (their corner combination is left out).
+// registers.
 constexpr int kSpeedThreads = 128;
 template <int DIM, int P, int SYS>
 __global__ void __launch_bounds__(kSpeedThreads)
     scalar_wavespeed_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ MaxSlots out) {
   using Img = PackedImage<DIM, P>;
-  constexpr int N = Img::N, NY1 = Img::NY1, MP = Img::MP, NG = Img::NG, ND = N * NY1;
+  constexpr int N = Img::N, NY1 = Img::NY1, MP = Img::MP, ND = N * NY1;
   __shared__ __align__(16) float img[Img::FLOATS];
   for (int f = threadIdx.x; f < Img::FLOATS; f += kSpeedThreads) img[f] = a.pk_img[f];
   __syncthreads();
@@ -85,36 +84,7 @@ __global__ void __launch_bounds__(kSpeedThreads)
     const float ubar = c[0][0].x;
     c[0][0].x = 0.0f;
     const ScalarLaw<SYS, DIM> law(a, ubar);
-    auto take = [&](f2 d) { lam = fmaxf(lam, fmaxf(law.speed(ubar + d.x), law.speed(ubar + d.y))); };
-#pragma unroll 1
-    for (int g = 0; g <= NG; ++g) {
-      f2 b[MP], tb[NY1];
-      load_pairs<MP>(img + Img::BX + 2 * MP * (g < NG ? g : 0), b);
-#pragma unroll
-      for (int my = 0; my < NY1; ++my) {
-        f2 s = g < NG ? mul2(b[0], c[my][0]) : c[my][0];
-#pragma unroll
-        for (int p = 1; p < MP; ++p) s = g < NG ? fma2(b[p], c[my][p], s) : add2(c[my][p], s);
-        tb[my] = mk2(s.x + s.y, s.x - s.y);
-      }
-      if constexpr (DIM == 1) {
-        take(tb[0]);
-      } else {
-#pragma unroll 1
-        for (int h = 0; h < (g < NG ? NG + 1 : NG); ++h) {
-          f2 by[N];
-          load_pairs<N>(img + Img::BY + 2 * N * (h < NG ? h : 0), by);
-          f2 e = h < NG ? mul2(by[0], tb[0]) : tb[0], o = h < NG ? mul2(by[1], tb[NY1 > 1 ? 1 : 0]) : tb[NY1 > 1 ? 1 : 0];
-#pragma unroll
-          for (int my = 2; my < NY1; ++my) {
-            if (my & 1) o = h < NG ? fma2(by[my], tb[my], o) : add2(tb[my], o);
-            else e = h < NG ? fma2(by[my], tb[my], e) : add2(tb[my], e);
-          }
-          take(add2(e, o));
-          take(sub2(e, o));
-        }
-      }
-    }
+    lam = fmaxf(lam, cell_speed<DIM, P>(img, law, ubar, c));
   }
   finish_max(lam, a.status, out);
 }
