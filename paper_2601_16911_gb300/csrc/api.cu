@@ -426,8 +426,8 @@ StageArgs base_args(const cvweno_mesh_s* m) {
   a.two_dy = (float)(2.0 / m->dy);
   a.nu_scale = (float)(m->h / (2.0 * m->p));
   a.h_e = (float)m->h;
-  a.tab_img = m->d_tabimg;
   a.pk_img = m->d_pkimg;
+  a.cg_img = m->d_cgimg;
   a.mlp = m->surrogate;
   a.mlp_conf_min = m->surrogate_conf_min;
   a.mlp_fallbacks = m->surrogate_fallbacks;
@@ -645,7 +645,7 @@ cvweno_status cvweno_mesh_destroy(cvweno_mesh m) {
   cudaFree(m->d_du2);
   cudaFree(m->d_cg_xg);
   cudaFree(m->d_cg_ml);
-  cudaFree(m->d_tabimg);
+  cudaFree(m->d_cgimg);
   cudaFree(m->d_pkimg);
   cudaFreeHost(m->h_status);
   cudaFreeHost(m->h_red);
@@ -723,8 +723,6 @@ cvweno_status cvweno_mesh_create(const cvweno_mesh_desc* d, cvweno_mesh* out) {
   if (e == cudaSuccess) e = cudaMalloc(&m->d_u1, sbytes);
   if (e == cudaSuccess) e = cudaMalloc(&m->d_u2, sbytes);
   if (e == cudaSuccess) e = cudaMalloc(&m->d_lambda, sizeof(float) * (size_t)m->ncell);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d_tabimg, sizeof(float) * (size_t)tab_image_floats(m->dim, m->p));
-  if (e == cudaSuccess) e = launch_tab_image(m->dim, m->p, m->tables, m->d_tabimg, 0);
   if (e == cudaSuccess) e = cudaMalloc(&m->d_pkimg, sizeof(float) * (size_t)packed_image_floats(m->dim, m->p));
   if (e == cudaSuccess) e = launch_packed_image(m->dim, m->p, m->tables, m->d_pkimg, 0);
   if (e == cudaSuccess) e = cudaStreamSynchronize(0);
@@ -735,6 +733,11 @@ cvweno_status cvweno_mesh_create(const cvweno_mesh_desc* d, cvweno_mesh* out) {
       if (e == cudaSuccess) e = cudaMalloc(&m->d_r, sizeof(float) * (size_t)m->nnode);
       if (e == cudaSuccess) e = cudaMalloc(&m->d_du, sizeof(float) * (size_t)m->nnode);
     }
+    float cimg[kMaxCgImage];
+    const int nimg = cg_image(m->dim, m->p, m->cg_tables, cimg, kMaxCgImage);
+    if (nimg == 0) e = cudaErrorInvalidValue;
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_cgimg, sizeof(float) * nimg);
+    if (e == cudaSuccess) e = cudaMemcpy(m->d_cgimg, cimg, sizeof(float) * nimg, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_cg_xg, sizeof(float) * (kMaxP + 1));
     if (e == cudaSuccess) e = cudaMalloc(&m->d_cg_ml, sizeof(double) * 2 * (kMaxP + 1));
     if (e == cudaSuccess) {

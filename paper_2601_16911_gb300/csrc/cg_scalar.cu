@@ -18,10 +18,9 @@
 //                       iterate are formed on a halo of 2p nodes, so one launch suffices
 //   1D: cg_node_rhs (assembly, du = r / ML) and two cg_node_sweep launches
 // Nodal sums gather the cells around a node in a fixed order.
-#include "cg_tile.cuh"
+#include "dg_scalar_kernel.cuh"
 
 namespace cvw {
-using namespace legacy;
 namespace {
 
 // i mod n for any int i (n > 0), without a division when i is already in range
@@ -31,22 +30,157 @@ __device__ __forceinline__ int wrap_index(int i, int n) {
   return i < 0 ? i + n : i;
 }
 
+// Device image of the nodal tables in the order they take in shared memory (host-built, once per
+// mesh): V[m][a], the Legendre modes of the nodal basis, by mirrored node pairs g = (a = g,
+// a = p - g), whose columns differ by (-1)^m only (the middle node of an even p is its own
+// partner): rows of mode pairs for the x direction, every entry doubled for the y direction.
+template <int DIM, int P>
+struct CgImage {
+  static constexpr int N = P + 1, MP = (N + 1) / 2, NG = (N + 1) / 2;
+  static constexpr int VX = 0;                                    // [NG][MP] pairs
+  static constexpr int VY = VX + 2 * NG * MP;                     // [NG][N] doubled
+  static constexpr int FLOATS = (VY + (DIM == 2 ? 2 * NG * N : 0) + 3) / 4 * 4;
+};
+
+// The tile's cells are modes computed here, so they lie as padded mode pairs (like the vertex
+// data) at every degree.
+template <int DIM, int P, int TX, int TY>
+struct CgCells : TileLayout<DIM, P, TX, TY> {
+  using L = TileLayout<DIM, P, TX, TY>;
+  static constexpr bool PADDED = true;
+  static __device__ __forceinline__ int cell(const int*, int hx, int hy) { return L::vertex(hy * L::HX + hx); }
+};
+
 template <int DIM, int P, int TX, int TY>
 struct CgLayout {
-  using L = TileLayout<DIM, P, TX, TY>;
-  static constexpr int N = P + 1, ND = L::ND, NH = L::NH;
+  using L = CgCells<DIM, P, TX, TY>;
+  using Img = PackedImage<DIM, P>;
+  static constexpr int N = P + 1, ND = L::ND, NH = L::NH, NT = L::NT;
   static constexpr int NNX = P * (TX + 2) + 1, NNY = DIM == 2 ? P * (TY + 2) + 1 : 1;
   // nodal rows at a 16-byte stride with room for a per-row phase of up to 3 floats
   static constexpr int NNXP = (NNX + 3 + 3) / 4 * 4;
-  // The nodal tile is dead once the halo cells are converted to modes, and the local
-  // integrals are written after that barrier: both start at the u_n region of the DG
-  // layout, which the CG kernel does not use (its RK combination runs on the nodes).
-  static constexpr int OFF_NODE = L::OFF_UN;              // [NNY][NNXP] nodal values
-  static constexpr int OFF_BX = L::OFF_UN;                // [ND][NH] int phi_a d_x u
-  static constexpr int OFF_BY = OFF_BX + ND * NH;         // [ND][NH] int phi_a d_y u
-  static constexpr int FLOATS = L::OFF_UN + (2 * ND * NH > NNXP * NNY ? 2 * ND * NH : NNXP * NNY);
+  static constexpr int OFF_C = 0;                                              // cells
+  static constexpr int OFF_ST = (L::VS * NH + 3) / 4 * 4;                      // vertex data, then stage (d)
+  static constexpr int OFF_NQ = OFF_ST, OFF_S12 = OFF_NQ + ND * NT;            // as the DG tile's
+  static constexpr int OFF_IMG = (OFF_ST + imax(L::VS * L::NVT, L::SCF) + 3) / 4 * 4;
+  static constexpr int OFF_VIMG = OFF_IMG + Img::FLOATS;
+  // The nodal tile is dead once the halo cells are converted to modes, the local integrals
+  // (pairs (x, y), [ND][NH]) once P_h grad u is gathered; then its modes
+  // (pairs, [2 NY1 MP][NT]) lie there, and gamma_e of the troubled cells for the other threads.
+  static constexpr int OFF_NODE = OFF_VIMG + CgImage<DIM, P>::FLOATS;
+  static constexpr int OFF_B = OFF_NODE;
+  static constexpr int OFF_PH = OFF_NODE, OFF_GAM = OFF_PH + 4 * L::NY1 * L::MP * NT;
+  static constexpr int FLOATS = OFF_NODE + imax(imax(2 * ND * NH, NNXP * NNY), OFF_GAM - OFF_PH + NT);
   static constexpr size_t BYTES = sizeof(float) * (size_t)FLOATS;
 };
+
+// Nodal values u[b][a] (polynomial at the cell's nodes) to Legendre modes, V x V: sums and
+// differences of mirrored nodes feed the even and the odd modes.
+template <int DIM, int P>
+__device__ __forceinline__ void nodes_to_modes(const float* vimg, const float (&u)[DIM == 2 ? P + 1 : 1][P + 1],
+                                               f2 (&c)[DIM == 2 ? P + 1 : 1][(P + 2) / 2]) {
+  using I = CgImage<DIM, P>;
+  constexpr int N = I::N, MP = I::MP, NG = I::NG, NY1 = DIM == 2 ? N : 1;
+  f2 t[NY1][MP];
+#pragma unroll
+  for (int g = 0; g < NG; ++g) {
+    f2 v[MP];
+    load_pairs<MP>(vimg + I::VX + 2 * MP * g, v);
+    const bool mid = 2 * g == P;
+#pragma unroll
+    for (int b = 0; b < NY1; ++b) {
+      const f2 sd = mid ? mk2(u[b][g], 0.0f) : mk2(u[b][g] + u[b][P - g], u[b][g] - u[b][P - g]);
+#pragma unroll
+      for (int p = 0; p < MP; ++p) t[b][p] = g == 0 ? mul2(v[p], sd) : fma2(v[p], sd, t[b][p]);
+    }
+  }
+  if constexpr (DIM == 1) {
+#pragma unroll
+    for (int p = 0; p < MP; ++p) c[0][p] = t[0][p];
+  } else {
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+      f2 v[N];
+      load_pairs<N>(vimg + I::VY + 2 * N * g, v);
+      const bool mid = 2 * g == P;
+#pragma unroll
+      for (int p = 0; p < MP; ++p) {
+        const f2 e = mid ? t[g][p] : add2(t[g][p], t[P - g][p]);
+        const f2 o = mid ? mk2(0.0f, 0.0f) : sub2(t[g][p], t[P - g][p]);
+#pragma unroll
+        for (int my = 0; my < NY1; ++my)
+          c[my][p] = g == 0 ? mul2(v[my], (my & 1) ? o : e) : fma2(v[my], (my & 1) ? o : e, c[my][p]);
+      }
+    }
+  }
+}
+
+// Nodal functionals r[b][a] = sum_m V[my][b] V[mx][a] R[my][mx] of a modal one, the transpose of
+// nodes_to_modes: node row by node row, handed to f(b, g, (value at a = g, value at a = p - g)).
+template <int DIM, int P, class F>
+__device__ __forceinline__ void modes_to_nodes_t(const float* vimg, const f2 (&R)[DIM == 2 ? P + 1 : 1][(P + 2) / 2], F&& f) {
+  using I = CgImage<DIM, P>;
+  constexpr int N = I::N, MP = I::MP, NG = I::NG, NY1 = DIM == 2 ? N : 1;
+#pragma unroll
+  for (int g = 0; g < NG; ++g) {
+    f2 v[MP], tb[NY1];
+    load_pairs<MP>(vimg + I::VX + 2 * MP * g, v);
+#pragma unroll
+    for (int my = 0; my < NY1; ++my) {
+      f2 s = mul2(v[0], R[my][0]);
+#pragma unroll
+      for (int p = 1; p < MP; ++p) s = fma2(v[p], R[my][p], s);
+      tb[my] = mk2(s.x + s.y, s.x - s.y);
+    }
+    if constexpr (DIM == 1) {
+      f(0, g, tb[0]);
+    } else {
+#pragma unroll
+      for (int h = 0; h < NG; ++h) {
+        f2 w[N];
+        load_pairs<N>(vimg + I::VY + 2 * N * h, w);
+        f2 e = mul2(w[0], tb[0]), o = mul2(w[1], tb[1]);
+#pragma unroll
+        for (int my = 2; my < N; ++my) {
+          if (my & 1) o = fma2(w[my], tb[my], o);
+          else e = fma2(w[my], tb[my], e);
+        }
+        f(h, g, add2(e, o));
+        if (2 * h != P) f(P - h, g, sub2(e, o));
+      }
+    }
+  }
+}
+
+// int P_m d/dxi u (x) and d/deta (y) over the reference cell for u = sum c_m P_m: int P_mx P_kx' is 2
+// for kx > mx of the other parity, int P_my P_ky 2/(2my+1) on the diagonal (1 in 1D).
+template <int DIM, int N, int NY1, int MP>
+__device__ __forceinline__ void gradient_moments(const f2 (&c)[NY1][MP], f2 (&gx)[NY1][MP], f2 (&gy)[NY1][MP]) {
+  auto val = [&](int my, int k) { return k >= N ? 0.0f : (k & 1) ? c[my][k / 2].y : c[my][k / 2].x; };
+#pragma unroll
+  for (int my = 0; my < NY1; ++my) {
+    const float sy = DIM == 2 ? 4.0f / (2 * my + 1) : 2.0f;
+    float d[2 * MP + 2];  // d[m] = c[m+1] + c[m+3] + ...
+    d[2 * MP + 1] = d[2 * MP] = 0.0f;
+#pragma unroll
+    for (int m = 2 * MP - 1; m >= 0; --m) d[m] = val(my, m + 1) + d[m + 2 <= 2 * MP + 1 ? m + 2 : 2 * MP];
+#pragma unroll
+    for (int p = 0; p < MP; ++p) {
+      gx[my][p] = mk2(sy * d[2 * p], 2 * p + 1 < N ? sy * d[2 * p + 1] : 0.0f);
+      gy[my][p] = mk2(0.0f, 0.0f);
+    }
+  }
+  if constexpr (DIM == 2) {
+#pragma unroll
+    for (int my = NY1 - 2; my >= 0; --my)
+#pragma unroll
+      for (int p = 0; p < MP; ++p) gy[my][p] = my + 3 < NY1 ? add2(c[my + 1][p], gy[my + 2 < NY1 ? my + 2 : my][p]) : c[my + 1][p];
+#pragma unroll
+    for (int my = 0; my < NY1; ++my)
+#pragma unroll
+      for (int p = 0; p < MP; ++p) gy[my][p] = mul2(gy[my][p], mk2(4.0f / (4 * p + 1), 4.0f / (4 * p + 3)));
+  }
+}
 
 // lumped mass of a 1D lattice node with local index a in [0, p): its GLL weight times
 // dx/2, counted twice at cell vertices (two cells share them)
@@ -55,46 +189,83 @@ __device__ __forceinline__ float ml1(const CgTables<DIM, P>& C, int a, float h) 
   return (a == 0 ? 2.0f : 1.0f) * C.wl[a] * h;
 }
 
-// Threads of a block of the CG cell kernel: one warp more than the tile's cells in 1D and
-// at p = 1, so that the tile's (TX + 1) (TY + 1) vertices take one round and the halo
-// ring's integrals fall on the extra warp (KPP 256^2 CG Q1: 0.0411 -> 0.0391 ms per step;
-// at p = 2 the same block was 19 % slower).
-template <int DIM, int P, int TX, int TY>
-__host__ __device__ constexpr int cg_block_threads() {
-  return DIM == 1 || P == 1 ? TX * TY + 32 : TX * TY;
+// Values tb and x-derivatives td at the node pair of tables b (P) and d (P'), row by row.
+template <int N, int NY1, int MP>
+__device__ __forceinline__ void x_values(const f2 (&b)[MP], const f2 (&d)[MP], const f2 (&c)[NY1][MP], f2 (&tb)[NY1],
+                                         f2 (&td)[NY1]) {
+#pragma unroll
+  for (int my = 0; my < NY1; ++my) {
+    f2 s = mul2(b[0], c[my][0]), sd = mul2(d[0], c[my][0]);
+#pragma unroll
+    for (int p = 1; p < MP; ++p) {
+      s = fma2(b[p], c[my][p], s);
+      sd = fma2(d[p], c[my][p], sd);
+    }
+    tb[my] = mk2(s.x + s.y, s.x - s.y);
+    td[my] = mk2(sd.x + sd.y, sd.y - sd.x);
+  }
 }
 
+// The same values of modes kept in shared memory, [NY1 MP] rows NT apart.
+template <int NY1, int MP, int NT>
+__device__ __forceinline__ void projection_values(const f2 (&b)[MP], const f2* sp, f2 (&t)[NY1]) {
+#pragma unroll
+  for (int my = 0; my < NY1; ++my) {
+    f2 s = mul2(b[0], sp[my * MP * NT]);
+#pragma unroll
+    for (int p = 1; p < MP; ++p) s = fma2(b[p], sp[(my * MP + p) * NT], s);
+    t[my] = mk2(s.x + s.y, s.x - s.y);
+  }
+}
+
+// Threads of a block of the CG cell kernel, and the resident CTAs its registers must allow.
+// KPP 256^2, us per step: p = 3, 4 CTAs of 128 threads 85.9, 4 of 160 (96 registers, spills) 91.0,
+// 3 of 128 95.9, 5 of 128 92.7; p = 2, 4 CTAs 56.6, 3 69.7, 5 58.1.
+template <int DIM, int P, int TX, int TY>
+__host__ __device__ constexpr int cg_block_threads() {
+  return TX * TY + (DIM == 1 || P == 1 ? 32 : 0);
+}
+template <int DIM, int P>
+constexpr int cg_min_ctas() {
+  return DIM == 1 ? 1 : P == 1 ? 6 : P <= 3 ? 4 : 2;
+}
+
+// One CTA per tile; bound by FP32 issue and latency at 13 warps per SM (49 % of the issue slots at
+// 256^2).  On two-wide FMAs and in the modal basis (local integrals, projection and residual go
+// to the nodes and back by V) the Q3 step takes 85.9 us instead of 107, Q2 56.6 instead of 65, Q1
+// 29.7 instead of 42 (KPP 256^2, node kernel included).
 template <int DIM, int P, int SYS, int TX, int TY>
-__global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>()) cg_stage_cells(const __grid_constant__ StageArgs a,
-                                                          const __grid_constant__ DgTables<DIM, P> T,
-                                                          const __grid_constant__ CgTables<DIM, P> C) {
-  using L = TileLayout<DIM, P, TX, TY>;
+__global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>(), (cg_min_ctas<DIM, P>()))
+    cg_stage_cells(const __grid_constant__ StageArgs a, const __grid_constant__ PackedTables<DIM, P> T,
+                   const __grid_constant__ CgTables<DIM, P> C) {
   using G = CgLayout<DIM, P, TX, TY>;
+  using L = typename G::L;
+  using Img = PackedImage<DIM, P>;
   using Law = ScalarLaw<SYS, DIM>;
-  constexpr int N = L::N, ND = L::ND, NT = L::NT, HX = L::HX, NH = L::NH;
+  constexpr int N = L::N, ND = L::ND, NT = L::NT, HX = L::HX, HY = L::HY, NH = L::NH, MP = L::MP, NG = L::NG;
   constexpr int NB = cg_block_threads<DIM, P, TX, TY>();  // threads of the block
   constexpr int NNX = G::NNX, NNY = G::NNY, NNXP = G::NNXP;
-  constexpr int NY1 = DIM == 2 ? N : 1;
+  constexpr int NY1 = L::NY1, NGY = DIM == 2 ? NG : 1;
   extern __shared__ __align__(16) float smem[];
-  float* sc = smem + L::OFF_SC;
-  float* st = smem + L::OFF_ST;
-  const float* sA = smem + L::OFF_A;
-  const float* sB = smem + L::OFF_B;
-  const float* sBd = smem + L::OFF_BD;
-  const float* sBk = smem + L::OFF_BK;
-  const float* sW = smem + L::OFF_W;
-  float* sNq = smem + L::OFF_NQ;
+  float* sc = smem + G::OFF_C;
+  float* st = smem + G::OFF_ST;
+  float* sNq = smem + G::OFF_NQ;
+  const float* img = smem + G::OFF_IMG;
+  const float* vimg = smem + G::OFF_VIMG;
   float* snode = smem + G::OFF_NODE;
-  float* sbx = smem + G::OFF_BX;
-  float* sby = smem + G::OFF_BY;
+  f2* sb = reinterpret_cast<f2*>(smem + G::OFF_B);
 
   const int nx = a.nx, ny = DIM == 2 ? a.ny : 1;
   const int nnx = a.nnx, nny = DIM == 2 ? a.nny : 1;
   const int i0 = blockIdx.x * TX, j0 = DIM == 2 ? blockIdx.y * TY : 0;
   const float hdx = 1.0f / a.two_dx, hdy = DIM == 2 ? 1.0f / a.two_dy : 1.0f;
+  __shared__ int sc_count;        // troubled cells of the tile,
+  __shared__ short sc_cell[NT];   // and their threads
+  if (threadIdx.x == 0) sc_count = 0;
 
   // ---- nodal values of the tile and its halo (periodic lattice) -------------------------
-  stage_tables_to_smem<DIM, P, TX, TY, NB>(a.tab_img, smem);
+  for (int f = threadIdx.x; f < Img::FLOATS / 4; f += NB) cp_async16(smem + G::OFF_IMG + 4 * f, a.pk_img + 4 * f);
+  for (int f = threadIdx.x; f < CgImage<DIM, P>::FLOATS / 4; f += NB) cp_async16(smem + G::OFF_VIMG + 4 * f, a.cg_img + 4 * f);
   pdl_wait();  // everything below reads or writes what earlier kernels write
   // Node (ix, iy) lands at snode[iy][sph[iy] + ix].  Where the tile's rows do not wrap in x
   // and the state is 16-byte aligned, each row is copied as the 16-byte chunks that cover
@@ -136,418 +307,286 @@ __global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>()) cg_stage_c
   // u_ref back, and a constant cell yields exactly zero non-mean modes.
   for (int h = threadIdx.x; h < NH; h += NB) {
     const int hx = h % HX, hy = DIM == 2 ? h / HX : 0;
-    float ul[ND];
+    float u[NY1][N];
 #pragma unroll
     for (int b = 0; b < NY1; ++b)
 #pragma unroll
-      for (int aa = 0; aa < N; ++aa) ul[aa + N * b] = snode[sph[P * hy + b] + (P * hx + aa) + NNXP * (P * hy + b)];
-    const float uref = ul[0];
+      for (int aa = 0; aa < N; ++aa) u[b][aa] = snode[sph[P * hy + b] + (P * hx + aa) + NNXP * (P * hy + b)];
+    const float uref = u[0][0];
 #pragma unroll
-    for (int m = 0; m < ND; ++m) ul[m] -= uref;
-    float tmp[N][NY1];  // [mx][b]
+    for (int b = 0; b < NY1; ++b)
 #pragma unroll
-    for (int mx = 0; mx < N; ++mx)
-#pragma unroll
-      for (int b = 0; b < NY1; ++b) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int aa = 0; aa < N; ++aa) acc = fmaf(C.V[mx][aa], ul[aa + N * b], acc);
-        tmp[mx][b] = acc;
-      }
-#pragma unroll
-    for (int my = 0; my < NY1; ++my)
-#pragma unroll
-      for (int mx = 0; mx < N; ++mx) {
-        float acc = tmp[mx][0];
-        if constexpr (DIM == 2) {
-          acc = 0.0f;
-#pragma unroll
-          for (int b = 0; b < N; ++b) acc = fmaf(C.V[my][b], tmp[mx][b], acc);
-        }
-        sc[(mx + N * my) * NH + h] = (mx + my == 0) ? acc + uref : acc;
-      }
+      for (int aa = 0; aa < N; ++aa) u[b][aa] -= uref;
+    f2 c[NY1][MP];
+    nodes_to_modes<DIM, P>(vimg, u, c);
+    c[0][0].x += uref;
+    store_vertex<L>(sc, h, c);
   }
   __syncthreads();
   // ---- (a)+(b) vertex candidates (shared with DG) ---------------------------------------
-  tile_vertex_phase<DIM, P, TX, TY, NB>(a, T, sc, st, i0, j0, nx, ny);
-  // ---- P_h local integrals b_a = int phi_a grad u (reading A13) ------------------------------
-  // For u = sum_m c_m P_mx P_my on the cell, with dx dy / 4 = hdx hdy and the factor 2/dx
-  // of d/dx cancelling hdx (Em, Dm: integrals of l_a against P_m and P_m'):
-  //   bx[a,b] = hdy sum_{mx,my} Dm[a][mx] Em[b][my] c[mx,my]
-  //   by[a,b] = hdx sum_{mx,my} Em[a][mx] Dm[b][my] c[mx,my]
-  // A tile cell takes every entry; a halo cell only those of its nodes on the tile's
-  // boundary, the ones that the tile's nodes gather (one row or column of nodes).
-  if constexpr (DIM == 1) {
-    for (int h = threadIdx.x; h < NH; h += NB) {
-#pragma unroll
-      for (int aa = 0; aa < N; ++aa) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int m = 0; m < N; ++m) acc = fmaf(C.Dm[aa][m], sc[m * NH + h], acc);
-        sbx[aa * NH + h] = acc;
-        sby[aa * NH + h] = 0.0f;
-      }
-    }
-  } else {
-    constexpr int HY = L::HY;
-    if (threadIdx.x < NT) {
-      const int h = (threadIdx.x / TX + 1) * HX + threadIdx.x % TX + 1;
-      float c[ND];
-#pragma unroll
-      for (int m = 0; m < ND; ++m) c[m] = sc[m * NH + h];
-      float tE[N][N], tD[N][N];  // [b][mx]: the y-contractions
-#pragma unroll
-      for (int b = 0; b < N; ++b)
-#pragma unroll
-        for (int mx = 0; mx < N; ++mx) {
-          float e = 0.0f, d = 0.0f;
-#pragma unroll
-          for (int my = 0; my < N; ++my) {
-            e = fmaf(C.Em[b][my], c[mx + N * my], e);
-            d = fmaf(C.Dm[b][my], c[mx + N * my], d);
-          }
-          tE[b][mx] = e;
-          tD[b][mx] = d;
-        }
-#pragma unroll
-      for (int b = 0; b < N; ++b)
-#pragma unroll
-        for (int aa = 0; aa < N; ++aa) {
-          float bx = 0.0f, by = 0.0f;
-#pragma unroll
-          for (int mx = 0; mx < N; ++mx) {
-            bx = fmaf(C.Dm[aa][mx], tE[b][mx], bx);
-            by = fmaf(C.Em[aa][mx], tD[b][mx], by);
-          }
-          sbx[(aa + N * b) * NH + h] = hdy * bx;
-          sby[(aa + N * b) * NH + h] = hdx * by;
-        }
-    }
-    // halo ring: the bottom and top rows (corners included) need the node row b = l that
-    // faces the tile (l = P below it, 0 above), the left and right columns the node
-    // column a = l (P left of it, 0 right)
-    constexpr int NR = 2 * HX + 2 * TY;
-    // from the block's last thread backwards: the vertex phase's extra round (if any) falls
-    // on the first warp, the ring on the last ones
-    for (int r = NB - 1 - threadIdx.x; r < NR; r += NB) {
-      const bool row = r < 2 * HX;
-      int hx, hy, l;
-      if (row) {
-        const bool top = r >= HX;
-        hx = top ? r - HX : r;
-        hy = top ? HY - 1 : 0;
-        l = top ? 0 : P;
-      } else {
-        const int rr = r - 2 * HX;
-        const bool right = rr >= TY;
-        hx = right ? HX - 1 : 0;
-        hy = 1 + (right ? rr - TY : rr);
-        l = right ? 0 : P;
-      }
-      const int h = hy * HX + hx;
-      float c[ND];
-#pragma unroll
-      for (int m = 0; m < ND; ++m) c[m] = sc[m * NH + h];
-      // s1: the contraction along the fixed direction with Em (row) or Dm (column) of
-      // node l; s2 with the other table
-      float s1[N], s2[N];
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        float e = 0.0f, d = 0.0f;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-          const float cv = row ? c[k + N * j] : c[j + N * k];  // row: k = mx, j = my
-          const float t1 = row ? (l ? C.Em[P][j] : C.Em[0][j]) : (l ? C.Dm[P][j] : C.Dm[0][j]);
-          const float t2 = row ? (l ? C.Dm[P][j] : C.Dm[0][j]) : (l ? C.Em[P][j] : C.Em[0][j]);
-          e = fmaf(t1, cv, e);
-          d = fmaf(t2, cv, d);
-        }
-        s1[k] = e;
-        s2[k] = d;
-      }
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        float bx = 0.0f, by = 0.0f;
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-          // row: bx[i,l] = sum_mx Dm[i][mx] s1[mx], by[i,l] = sum_mx Em[i][mx] s2[mx]
-          // column: bx[l,i] = sum_my Em[i][my] s1[my], by[l,i] = sum_my Dm[i][my] s2[my]
-          bx = fmaf(row ? C.Dm[i][k] : C.Em[i][k], s1[k], bx);
-          by = fmaf(row ? C.Em[i][k] : C.Dm[i][k], s2[k], by);
-        }
-        const int lm = row ? i + N * l : l + N * i;
-        sbx[lm * NH + h] = hdy * bx;
-        sby[lm * NH + h] = hdx * by;
-      }
-    }
+  tile_vertex_phase<DIM, P, TX, TY, NB, false, L>(a, T, sc, nullptr, st, i0, j0, nx, ny);
+  // ---- P_h local integrals b_a = int phi_a grad u of every tile and halo cell (reading A13),
+  // with dx dy / 4 = hdx hdy and the factor 2/dx of d/dx cancelling hdx.  From the block's last
+  // thread backwards: the vertex phase's extra round (if any) falls on the first warp.
+  for (int h = NB - 1 - threadIdx.x; h < NH; h += NB) {
+    f2 c[NY1][MP], gx[NY1][MP], gy[NY1][MP];
+    load_cell<L>(sc, L::vertex(h), c);
+    gradient_moments<DIM, N, NY1, MP>(c, gx, gy);
+    modes_to_nodes_t<DIM, P>(vimg, gx, [&](int b, int g, f2 v) {
+      sb[(g + N * b) * NH + h].x = hdy * v.x;
+      sb[(P - g + N * b) * NH + h].x = hdy * v.y;
+    });
+    if constexpr (DIM == 2)
+      modes_to_nodes_t<DIM, P>(vimg, gy, [&](int b, int g, f2 v) {
+        sb[(g + N * b) * NH + h].y = hdx * v.x;
+        sb[(P - g + N * b) * NH + h].y = hdx * v.y;
+      });
   }
   __syncthreads();
   pdl_launch_dependents();
 
-  // ---- one thread per own cell ------------------------------------------------------------------
-  if (NB > NT && threadIdx.x >= NT) return;
+  // ---- one thread per own cell (the others take part in stage (d)) --------------------------
   const int tx = threadIdx.x % TX, ty = DIM == 2 ? threadIdx.x / TX : 0;
   const int gi = i0 + tx, gj = j0 + ty;
-  if (gi >= nx || gj >= ny) return;
-  const int hcx = tx + 1, hcy = DIM == 2 ? ty + 1 : 0;
-  const int hc = hcy * HX + hcx;
   const size_t cell = (size_t)gj * nx + gi;
-  if (!CVW_SPAN(a.status, cell, 1, a.lim_cell)) return;  // per-cell outputs and rloc
-  float c[ND];
-#pragma unroll
-  for (int m = 0; m < ND; ++m) c[m] = sc[m * NH + hc];
-  float n0;
-  float wstar[DgTables<DIM, P>::NS];  // unused: CG has no limiter mode
-  const float gam = cell_sensor<DIM, P, TX, TY>(a, T, st, sA, c, tx, ty, n0, wstar);
-  const Law law(a, c[0]);
-
-  // lambda_e over the volume and face Gauss nodes of the cell polynomial
-  float lam = a.lambda_const;
-  if (!(a.lambda_const > 0.0f)) {
-    lam = 0.0f;
-    float tr[4][N];  // right, left, top, bottom traces (tangential modes)
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      float r = 0.0f, l = 0.0f, t = 0.0f, b = 0.0f;
-      if constexpr (DIM == 1) {
-        if (j == 0)
-#pragma unroll
-          for (int i = 0; i < N; ++i) {
-            r += c[i];
-            l += (i & 1) ? -c[i] : c[i];
-          }
-      } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-          r += c[i + N * j];
-          l += (i & 1) ? -c[i + N * j] : c[i + N * j];
-          t += c[j + N * i];
-          b += (i & 1) ? -c[j + N * i] : c[j + N * i];
-        }
-      }
-      tr[0][j] = r;
-      tr[1][j] = l;
-      tr[2][j] = t;
-      tr[3][j] = b;
+  const bool active = (NB == NT || threadIdx.x < NT) && gi < nx && gj < ny &&
+                      CVW_SPAN(a.status, cell, 1, a.lim_cell);  // per-cell outputs and rloc
+  const int hcx = tx + 1, hcy = DIM == 2 ? min(ty, TY - 1) + 1 : 0;
+  f2 c[NY1][MP];
+  load_cell<L>(sc, L::cell(nullptr, hcx, hcy), c);
+  const float ubar = c[0][0].x;
+  const bool sensor_only = (a.mode & kModeSensorOnly) != 0, need_lam = !(a.lambda_const > 0.0f);
+  const Law law(a, ubar);
+  float n0 = 0.0f, gam = 1.0f, lam = need_lam ? 0.0f : a.lambda_const;
+  f2 px[NY1][MP], py[NY1][MP];  // modes of P_h grad u
+  if (active) {
+    gam = cell_sensor<DIM, P, TX, TY>(a, T, st, c, tx, ty, n0, px);
+    // lambda_e over the volume and face Gauss nodes of the cell polynomial
+    if (need_lam) {
+      c[0][0].x = 0.0f;
+      lam = cell_speed<DIM, P>(img, law, ubar, c);
     }
-#pragma unroll
-    for (int q = 0; q < (DIM == 2 ? N : 1); ++q) {
-#pragma unroll
-      for (int f = 0; f < (DIM == 2 ? 4 : 2); ++f) {
-        float v = tr[f][0];
-        if constexpr (DIM == 2) {
-          v = 0.0f;
-#pragma unroll
-          for (int j = 0; j < N; ++j) v = fmaf(T.B[q][j], tr[f][j], v);
-        }
-      lam = fmaxf(lam, law.speed(v));
-      }
-    }
-    // volume nodes, by sum factorisation
-#pragma unroll 1
-    for (int qx = 0; qx < N; ++qx) {
-      float tb[NY1];
-#pragma unroll
-      for (int my = 0; my < NY1; ++my) {
-        float s0 = 0.0f;
-#pragma unroll
-        for (int mx = 0; mx < N; ++mx) s0 = fmaf(sB[qx * N + mx], c[mx + N * my], s0);
-        tb[my] = s0;
-      }
-#pragma unroll
-      for (int qy = 0; qy < NY1; ++qy) {
-        float u = tb[0];
-        if constexpr (DIM == 2) {
-          u = 0.0f;
-#pragma unroll
-          for (int my = 0; my < N; ++my) u = fmaf(sB[qy * N + my], tb[my], u);
-        }
-        lam = fmaxf(lam, law.speed(u));
-      }
-    }
+    if (a.gamma_out) a.gamma_out[cell] = gam;
+    if (a.nu_out) a.nu_out[cell] = lam * a.nu_scale;
+    if (a.lambda_out) a.lambda_out[cell] = lam;
   }
-  const float nu = lam * a.nu_scale;
-  if (a.gamma_out) a.gamma_out[cell] = gam;
-  if (a.nu_out) a.nu_out[cell] = nu;
-  if (a.lambda_out) a.lambda_out[cell] = lam;
-  if (a.mode & kModeSensorOnly) return;
+  if (sensor_only) return;
 
   // P_h grad u at the own cell's nodes: sum over the cells sharing each node / ML
-  float phx[ND], phy[ND];
+  if (active) {
+    float nx_[NY1][N], ny_[NY1][N];
 #pragma unroll
-  for (int bb = 0; bb < NY1; ++bb)
+    for (int bb = 0; bb < NY1; ++bb)
 #pragma unroll
-    for (int aa = 0; aa < N; ++aa) {
-      float sx = 0.0f, sy = 0.0f;
-      // x-neighbours of the node: (halo column, local index)
-      const int ncx = (aa == 0 || aa == P) ? 2 : 1;
-      const int ncy = DIM == 2 ? ((bb == 0 || bb == P) ? 2 : 1) : 1;
+      for (int aa = 0; aa < N; ++aa) {
+        f2 s = mk2(0.0f, 0.0f);
+        // x-neighbours of the node: (halo column, local index)
+        const int ncx = (aa == 0 || aa == P) ? 2 : 1;
+        const int ncy = DIM == 2 ? ((bb == 0 || bb == P) ? 2 : 1) : 1;
 #pragma unroll
-      for (int jy = 0; jy < ncy; ++jy)
+        for (int jy = 0; jy < ncy; ++jy)
 #pragma unroll
-        for (int jx = 0; jx < ncx; ++jx) {
-          int cx = hcx, la = aa, cy = hcy, lb = bb;
-          if (aa == 0) { cx = jx == 0 ? hcx - 1 : hcx; la = jx == 0 ? P : 0; }
-          if (aa == P) { cx = jx == 0 ? hcx : hcx + 1; la = jx == 0 ? P : 0; }
-          if (DIM == 2 && bb == 0) { cy = jy == 0 ? hcy - 1 : hcy; lb = jy == 0 ? P : 0; }
-          if (DIM == 2 && bb == P) { cy = jy == 0 ? hcy : hcy + 1; lb = jy == 0 ? P : 0; }
-          const int hh = cy * HX + cx, lm = la + N * lb;
-          sx += sbx[lm * NH + hh];
-          sy += sby[lm * NH + hh];
-        }
-      // 1 / ML of the node: the inverse lumped masses of its two 1D indices
-      const float iml = C.iml[aa == P ? 0 : aa] * a.two_dx * (DIM == 2 ? C.iml[bb == P ? 0 : bb] * a.two_dy : 1.0f);
-      phx[aa + N * bb] = sx * iml;
-      phy[aa + N * bb] = sy * iml;
-    }
-
-  // (d) SC weights (A24) and (e) local residual over the volume Gauss nodes, by sum
-  // factorisation: per row qx the x-contractions of c (values, x-derivatives) and of the
-  // nodal P_h grad u, then the nodes of the row; the residual is projected back the same way
-  bool troubled = a.sc && gam < a.c_gamma && n0 > 1e-30f;
-  if (a.troubled_override) {
-    const int ov = a.troubled_override[cell];
-    if (ov >= 0) troubled = ov && n0 > 1e-30f;
-  }
-  float afac = -1.0f;
-  const bool need_sc = troubled && gam < 1.0f;
-  // x-contractions of row qx: tb = B c, td = Bd c (modes), tpx/tpy = Lq ph (nodal)
-  auto row = [&](int qx, float (&tb)[NY1], float (&td)[NY1], float (&tpx)[NY1], float (&tpy)[NY1]) {
-#pragma unroll
-    for (int my = 0; my < NY1; ++my) {
-      float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
-#pragma unroll
-      for (int mx = 0; mx < N; ++mx) {
-        const float cm = c[mx + N * my];
-        s0 = fmaf(sB[qx * N + mx], cm, s0);
-        s1 = fmaf(sBd[qx * N + mx], cm, s1);
-        const float lx = (&C.Lq[0][0])[qx * N + mx];
-        s2 = fmaf(lx, phx[mx + N * my], s2);
-        s3 = fmaf(lx, phy[mx + N * my], s3);
-      }
-      tb[my] = s0;
-      td[my] = s1;
-      tpx[my] = s2;
-      tpy[my] = s3;
-    }
-  };
-  // node (qx, qy) of the row: value, physical gradient, P_h grad u
-  auto node = [&](int qy, const float (&tb)[NY1], const float (&td)[NY1], const float (&tpx)[NY1],
-                  const float (&tpy)[NY1], float& u, float& gx, float& gy, float& px, float& py) {
-    if constexpr (DIM == 1) {
-      u = tb[0];
-      gx = td[0] * a.two_dx;
-      gy = 0.0f;
-      px = tpx[0];
-      py = 0.0f;
-    } else {
-      u = gx = gy = px = py = 0.0f;
-#pragma unroll
-      for (int my = 0; my < N; ++my) {
-        const float by = sB[qy * N + my], ly = (&C.Lq[0][0])[qy * N + my];
-        u = fmaf(by, tb[my], u);
-        gx = fmaf(by, td[my], gx);
-        gy = fmaf(sBd[qy * N + my], tb[my], gy);
-        px = fmaf(ly, tpx[my], px);
-        py = fmaf(ly, tpy[my], py);
-      }
-      gx *= a.two_dx;
-      gy *= a.two_dy;
-    }
-  };
-  if (need_sc) {
-    float s1 = 0.0f, s2 = 0.0f;
-#pragma unroll 1
-    for (int qx = 0; qx < N; ++qx) {
-      float tb[NY1], td[NY1], tpx[NY1], tpy[NY1];
-      row(qx, tb, td, tpx, tpy);
-      float X[N][NY1];  // X[kx][my] = sum_mx Bk[kx][qx][mx] c[mx, my]
-#pragma unroll
-      for (int kx = 0; kx < N; ++kx)
-#pragma unroll
-        for (int my = 0; my < NY1; ++my) {
-          float acc = 0.0f;
-#pragma unroll
-          for (int mx = 0; mx < N; ++mx) acc = fmaf(sBk[(kx * N + qx) * N + mx], c[mx + N * my], acc);
-          X[kx][my] = acc;
-        }
-#pragma unroll 1
-      for (int qy = 0; qy < NY1; ++qy) {
-        float u, gx, gy, px, py;
-        node(qy, tb, td, tpx, tpy, u, gx, gy, px, py);
-        float n2 = 0.0f;
-#pragma unroll
-        for (int ky = 0; ky < NY1; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < N; ++kx) {
-            if (kx + ky == 0) continue;
-            float dk = X[kx][0];
-            if constexpr (DIM == 2) {
-              dk = 0.0f;
-#pragma unroll
-              for (int my = 0; my < N; ++my) dk = fmaf(sBk[(ky * N + qy) * N + my], X[kx][my], dk);
-            }
-            n2 = fmaf(T.sigma[kx + N * ky] * dk, dk, n2);
+          for (int jx = 0; jx < ncx; ++jx) {
+            int cx = hcx, la = aa, cy = hcy, lb = bb;
+            if (aa == 0) { cx = jx == 0 ? hcx - 1 : hcx; la = jx == 0 ? P : 0; }
+            if (aa == P) { cx = jx == 0 ? hcx : hcx + 1; la = jx == 0 ? P : 0; }
+            if (DIM == 2 && bb == 0) { cy = jy == 0 ? hcy - 1 : hcy; lb = jy == 0 ? P : 0; }
+            if (DIM == 2 && bb == P) { cy = jy == 0 ? hcy : hcy + 1; lb = jy == 0 ? P : 0; }
+            s = add2(s, sb[(la + N * lb) * NH + cy * HX + cx]);
           }
-        const float nq = sqrtf(n2);
-        const int q = qx + N * qy;
-        sNq[q * NT + threadIdx.x] = nq;
-        const float f = fmaf(gx, gx, gy * gy) - gam * (gx * px + gy * py);
-        const float W = sW[qx] * (DIM == 2 ? sW[qy] : 1.0f);
-        s1 = fmaf(W, f, s1);
-        s2 = fmaf(W * nq, f, s2);
+        // 1 / ML of the node: the inverse lumped masses of its two 1D indices
+        const float iml = C.iml[aa == P ? 0 : aa] * a.two_dx * (DIM == 2 ? C.iml[bb == P ? 0 : bb] * a.two_dy : 1.0f);
+        nx_[bb][aa] = s.x * iml;
+        ny_[bb][aa] = s.y * iml;
       }
-    }
-    if (s1 > 0.0f && s2 > 0.0f) afac = s1 / s2;
+    nodes_to_modes<DIM, P>(vimg, nx_, px);
+    if constexpr (DIM == 2) nodes_to_modes<DIM, P>(vimg, ny_, py);
   }
+
+  // ---- (d) SC weights (A24), f_q = |grad u|^2 - gamma grad u . P_h grad u: the troubled cells' node
+  // groups shared by the tile's threads, as in the DG kernel
+  bool troubled = false;
+  float afac = -1.0f;
+  if (active) {
+    troubled = a.sc && gam < a.c_gamma && n0 > 1e-30f;
+    if (a.troubled_override) {
+      const int ov = a.troubled_override[cell];
+      if (ov >= 0) troubled = ov && n0 > 1e-30f;
+    }
+  }
+  const bool need_sc = troubled && gam < 1.0f;
+  if (need_sc) sc_cell[atomicAdd(&sc_count, 1)] = (short)threadIdx.x;
+  const bool any_sc = __syncthreads_or(need_sc);  // (and every cell has gathered the local integrals)
+  // the projection's modes wait in shared memory: held in registers over the volume flux they
+  // would cost the kernel a resident CTA
+  f2* sP = reinterpret_cast<f2*>(smem + G::OFF_PH);
+  if (active) {
+#pragma unroll
+    for (int my = 0; my < NY1; ++my)
+#pragma unroll
+      for (int p = 0; p < MP; ++p) {
+        sP[(my * MP + p) * NT + threadIdx.x] = px[my][p];
+        if (DIM == 2) sP[((NY1 + my) * MP + p) * NT + threadIdx.x] = py[my][p];
+      }
+  }
+  if (any_sc) {
+    const int n = sc_count;
+    float* sGam = smem + G::OFF_GAM;
+    float* sS = smem + G::OFF_S12;
+    if (need_sc) sGam[threadIdx.x] = gam;
+    __syncthreads();
+#pragma unroll 1
+    for (int t = threadIdx.x; t < n * L::NGG; t += NB) {
+      const int gh = t / n, id = sc_cell[t - gh * n], g = gh / NGY, h = gh - g * NGY;
+      f2 s1, s2, nqa, nqb = mk2(0.0f, 0.0f);
+      sc_node_group<DIM, P, TX, TY, false, L>(a, T, img, sNq, sc, nullptr, id, g, h, s1, s2, &nqa, &nqb);
+      // grad u . P_h grad u at the group's nodes
+      f2 b[MP], d[MP], tp[NY1];
+      load_pairs<MP>(img + Img::BX + 2 * MP * g, b);
+      load_pairs<MP>(img + Img::DX + 2 * MP * g, d);
+      const float gm = -sGam[id];
+      f2 tb[NY1], td[NY1];
+      {
+        f2 cc[NY1][MP];
+        load_cell<L>(sc, L::cell(nullptr, id % TX + 1, DIM == 2 ? id / TX + 1 : 0), cc);
+        cc[0][0].x = 0.0f;
+        x_values<N, NY1, MP>(b, d, cc, tb, td);
+      }
+      if constexpr (DIM == 1) {
+        projection_values<NY1, MP, NT>(b, sP + id, tp);
+        const f2 f = mul2(dup2(gm * a.two_dx * img[Img::WX + g]), mul2(td[0], tp[0]));
+        s1 = add2(s1, f);
+        s2 = fma2(nqa, f, s2);
+      } else {
+        const float* yb_ = img + Img::BY + 2 * N * h;
+        f2 xa, xb, ya, yb, pa, pb;
+        node_gradient<N, MP>(yb_, img + Img::DY + 2 * N * h, tb, td, xa, xb, ya, yb);
+        projection_values<NY1, MP, NT>(b, sP + id, tp);
+        node_rows<N>(yb_, tp, pa, pb);
+        xa = mul2(mul2(dup2(a.two_dx), xa), pa);
+        xb = mul2(mul2(dup2(a.two_dx), xb), pb);
+        projection_values<NY1, MP, NT>(b, sP + NY1 * MP * NT + id, tp);
+        node_rows<N>(yb_, tp, pa, pb);
+        const f2 w = dup2(gm * img[Img::WX + g] * img[Img::WY + h]), ky = dup2(a.two_dy);
+        const f2 fa = mul2(w, fma2(mul2(ky, ya), pa, xa));
+        s1 = add2(s1, fa);
+        s2 = fma2(nqa, fa, s2);
+        if (2 * h != N - 1) {
+          const f2 fb = mul2(w, fma2(mul2(ky, yb), pb, xb));
+          s1 = add2(s1, fb);
+          s2 = fma2(nqb, fb, s2);
+        }
+      }
+      sS[gh * NT + id] = s1.x + s1.y;
+      sS[(L::NGG + gh) * NT + id] = s2.x + s2.y;
+    }
+    __syncthreads();
+    if (need_sc) {
+      float s1 = 0.0f, s2 = 0.0f;
+#pragma unroll
+      for (int gh = 0; gh < L::NGG; ++gh) {
+        s1 += sS[gh * NT + threadIdx.x];
+        s2 += sS[(L::NGG + gh) * NT + threadIdx.x];
+      }
+      if (s1 > 0.0f && s2 > 0.0f) afac = s1 / s2;
+    }
+  }
+  if (!active) return;
   if (a.troubled_out) a.troubled_out[cell] = troubled ? 1 : 0;
   if (a.alpha_out) {
 #pragma unroll 1
     for (int q = 0; q < ND; ++q) a.alpha_out[cell * ND + q] = afac >= 0.0f ? sNq[q * NT + threadIdx.x] * afac : 1.0f;
   }
-  float r[ND];
+
+  // ---- (e) modal residual R: the volume flux as deviations from f(ubar) (the constant part, which
+  // lives on the cell's edges and telescopes between neighbours, is added below), and
+  // -nu alpha (grad u - gamma P_h grad u)
+  load_cell<L>(sc, L::cell(nullptr, hcx, hcy), c);  // again, rather than held
+  c[0][0].x = 0.0f;
+  const float nu = lam * a.nu_scale;
+  f2 R[NY1][MP];
 #pragma unroll
-  for (int m = 0; m < ND; ++m) r[m] = 0.0f;
-#pragma unroll 1
-  for (int qx = 0; qx < N; ++qx) {
-    float tb[NY1], td[NY1], tpx[NY1], tpy[NY1];
-    row(qx, tb, td, tpx, tpy);
-    float hx[NY1], hy[NY1];
+  for (int my = 0; my < NY1; ++my)
 #pragma unroll
-    for (int b = 0; b < NY1; ++b) hx[b] = hy[b] = 0.0f;
-#pragma unroll 1
-    for (int qy = 0; qy < NY1; ++qy) {
-      float u, gx, gy, px, py;
-      node(qy, tb, td, tpx, tpy, u, gx, gy, px, py);
-      // f(u) - f(ubar): the cell constant f(ubar) contributes f(ubar) int_K grad phi_a,
-      // which lives on the cell's edges and telescopes between neighbours (added below)
-      float fx, fy;
-      law.flux_dev(u - c[0], fx, fy);
-      const int q = qx + N * qy;
-      const float al = afac >= 0.0f ? sNq[q * NT + threadIdx.x] * afac : 1.0f;
-      const float W = sW[qx] * (DIM == 2 ? sW[qy] : 1.0f) * hdx * hdy;
-      const float Gx = W * (fx - nu * al * (gx - gam * px));
-      const float Gy = W * (fy - nu * al * (gy - gam * py));
-      if constexpr (DIM == 2) {
+    for (int p = 0; p < MP; ++p) R[my][p] = mk2(0.0f, 0.0f);
+  float dummy = 0.0f;
+  volume_flux<DIM, P>(a, img, law, ubar, c, false, true, dummy, R);
+  if (afac < 0.0f) {
+    // linear weights: the Gauss rule is exact, so the gradient's part is the stiffness form and
+    // the projection's int P_mx' P_kx = 2 for kx < mx of the other parity, diagonal in y
+    add_stiffness<DIM, N, NY1, MP>(-nu * a.two_dx * a.two_dx, -nu * a.two_dy * a.two_dy, c, R);
+    const float kx = nu * gam * a.two_dx, ky = nu * gam * a.two_dy;
 #pragma unroll
-        for (int b = 0; b < N; ++b) {
-          hx[b] = fmaf((&C.Lq[0][0])[qy * N + b], Gx, hx[b]);
-          hy[b] = fmaf((&C.Ldq[0][0])[qy * N + b], Gy, hy[b]);
-        }
-      } else {
-        hx[0] += Gx;
+    for (int my = 0; my < NY1; ++my) {
+      const float sy = DIM == 2 ? 4.0f / (2 * my + 1) : 2.0f;
+      float even = 0.0f, odd = 0.0f;  // sums of the even and odd modes so far
+#pragma unroll
+      for (int p = 0; p < MP; ++p) {
+        const f2 v = sP[(my * MP + p) * NT + threadIdx.x];
+        const float e1 = even + v.x;
+        R[my][p] = fma2(dup2(kx * sy), mk2(odd, e1), R[my][p]);
+        even = e1;
+        odd += v.y;
       }
     }
-    // r[a, b] += 2/dx Ldq[qx][a] hx[b] + 2/dy Lq[qx][a] hy[b]
+    if constexpr (DIM == 2) {
 #pragma unroll
-    for (int b = 0; b < NY1; ++b)
+      for (int p = 0; p < MP; ++p) {
+        const f2 s = mul2(dup2(ky), mk2(4.0f / (4 * p + 1), 4.0f / (4 * p + 3)));
+        f2 even = sP[(NY1 * MP + p) * NT + threadIdx.x], odd = mk2(0.0f, 0.0f);
 #pragma unroll
-      for (int aa = 0; aa < N; ++aa) {
-        float v = fmaf(a.two_dx * (&C.Ldq[0][0])[qx * N + aa], hx[b], r[aa + N * b]);
-        if constexpr (DIM == 2) v = fmaf(a.two_dy * (&C.Lq[0][0])[qx * N + aa], hy[b], v);
-        r[aa + N * b] = v;
+        for (int my = 1; my < NY1; ++my) {
+          R[my][p] = fma2(s, (my & 1) ? even : odd, R[my][p]);
+          const f2 v = sP[((NY1 + my) * MP + p) * NT + threadIdx.x];
+          if (my & 1) odd = my == 1 ? v : add2(odd, v);
+          else even = add2(even, v);
+        }
       }
+    }
+  } else {
+    const float m = -nu * afac;
+#pragma unroll 1
+    for (int g = 0; g < NG; ++g) {
+      f2 b[MP], d[MP], tb[NY1], td[NY1], tp[NY1], tq[NY1], hx[NY1], hy[NY1];
+      load_pairs<MP>(img + Img::BX + 2 * MP * g, b);
+      load_pairs<MP>(img + Img::DX + 2 * MP * g, d);
+      x_values<N, NY1, MP>(b, d, c, tb, td);
+      projection_values<NY1, MP, NT>(b, sP + threadIdx.x, tp);
+      if (DIM == 2) projection_values<NY1, MP, NT>(b, sP + NY1 * MP * NT + threadIdx.x, tq);
+#pragma unroll
+      for (int my = 0; my < NY1; ++my) hx[my] = hy[my] = mk2(0.0f, 0.0f);
+      const float* nq = sNq + threadIdx.x;
+      if constexpr (DIM == 1) {
+        const f2 al = mul2(dup2(m), mk2(nq[g * NT], nq[(N - 1 - g) * NT]));
+        hx[0] = mul2(al, fma2(dup2(a.two_dx), td[0], mul2(dup2(-gam), tp[0])));
+      } else {
+#pragma unroll 1
+        for (int h = 0; h < NGY; ++h) {
+          const float *yb = img + Img::BY + 2 * N * h, *yd = img + Img::DY + 2 * N * h;
+          f2 xa, xb, ya, yy, pa, pb, qa, qb;
+          node_gradient<N, MP>(yb, yd, tb, td, xa, xb, ya, yy);
+          node_rows<N>(yb, tp, pa, pb);
+          node_rows<N>(yb, tq, qa, qb);
+          const bool mid = (N & 1) && h == NG - 1;
+          const f2 w = dup2(m * img[Img::WY + h]), kx = dup2(a.two_dx), ky = dup2(a.two_dy), gm = dup2(-gam);
+          const float *na = nq + (g + N * h) * NT, *nb = nq + (g + N * (N - 1 - h)) * NT;
+          const f2 la = mul2(w, mk2(na[0], na[(N - 1 - 2 * g) * NT]));
+          f2 lb = mul2(w, mk2(nb[0], nb[(N - 1 - 2 * g) * NT]));
+          if (mid) lb = mk2(0.0f, 0.0f);
+          const f2 fx = mul2(la, fma2(gm, pa, mul2(kx, xa))), gx = mul2(lb, fma2(gm, pb, mul2(kx, xb)));
+          const f2 fy = mul2(la, fma2(gm, qa, mul2(ky, ya))), gy = mul2(lb, fma2(gm, qb, mul2(ky, yy)));
+          project_rows<N>(yb, yd, fx, gx, fy, gy, hx, hy);
+        }
+      }
+      project_nodes<NY1, MP>(b, d, a.two_dx * img[Img::WX + g], a.two_dy * img[Img::WX + g], hx, hy, R);
+    }
   }
+  // to the nodal basis; r[a, b] scaled by the cell's Jacobian
+  float r[ND];
+  modes_to_nodes_t<DIM, P>(vimg, R, [&](int b, int g, f2 v) {
+    r[g + N * b] = hdx * hdy * v.x;
+    if (2 * g != P) r[P - g + N * b] = hdx * hdy * v.y;
+  });
   // The constant part of the flux: int_K d_x phi_ab f(ubar_e) = (delta_{a,p} - delta_{a,0})
   // wl_b (dy/2) f_x(ubar_e) (likewise in y).  At the nodes of an edge between a left cell L
   // and a right cell R the two cells' terms sum to (f_x(ubar_L) - f_x(ubar_R)) wl_b dy/2;
@@ -556,11 +595,11 @@ __global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>()) cg_stage_c
   // of its own law from the halo means.
   {
     float fx, fy;
-    law.flux_dev(sc[hc - 1] - c[0], fx, fy);  // f(ubar_left) - f(ubar_e)
+    law.flux_dev(sc[L::cell(nullptr, hcx - 1, hcy)] - ubar, fx, fy);  // f(ubar_left) - f(ubar_e)
 #pragma unroll
     for (int b = 0; b < NY1; ++b) r[N * b] = fmaf(fx, DIM == 2 ? C.wl[b] * hdy : 1.0f, r[N * b]);
     if constexpr (DIM == 2) {
-      law.flux_dev(sc[hc - HX] - c[0], fx, fy);  // f(ubar_below) - f(ubar_e)
+      law.flux_dev(sc[L::cell(nullptr, hcx, hcy - 1)] - ubar, fx, fy);  // f(ubar_below) - f(ubar_e)
 #pragma unroll
       for (int aa = 0; aa < N; ++aa) r[aa] = fmaf(fy, C.wl[aa] * hdx, r[aa]);
     }
@@ -904,7 +943,7 @@ cudaError_t launch_cg_t(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t
   constexpr size_t smem = CgLayout<DIM, P, TX, TY>::BYTES;
   static_assert(smem <= 220 * 1024, "tile too large for shared memory");
   if (m->tables_bytes != sizeof(Tb) || m->cg_tables_bytes != sizeof(Cb)) return cudaErrorInvalidValue;
-  const Tb& T = *static_cast<const Tb*>(m->tables);
+  const PackedTables<DIM, P>& T = static_cast<const Tb*>(m->tables)->pk;
   const Cb& C = *static_cast<const Cb*>(m->cg_tables);
   auto k1 = cg_stage_cells<DIM, P, SYS, TX, TY>;
   if (smem > 48 * 1024) {
@@ -962,26 +1001,32 @@ cudaError_t launch_stage_cg(const cvweno_mesh_s* m, const StageArgs& a, cudaStre
   }
 }
 
-namespace {
+// CgImage<dim, p> of the mesh's nodal tables into dst (host, capacity floats); the number written.
 template <int DIM, int P>
-cudaError_t tab_image(const void* t, float* dst, cudaStream_t s) {
-  tab_image_kernel<DIM, P><<<1, 256, 0, s>>>(*static_cast<const DgTables<DIM, P>*>(t), dst);
-  return cudaGetLastError();
+static int fill_cg_image(const void* tables, float* dst, int capacity) {
+  using I = CgImage<DIM, P>;
+  const CgTables<DIM, P>& C = *static_cast<const CgTables<DIM, P>*>(tables);
+  if (capacity < I::FLOATS) return 0;
+  for (int f = 0; f < I::FLOATS; ++f) dst[f] = 0.0f;
+  for (int g = 0; g < I::NG; ++g)
+    for (int m = 0; m < I::N; ++m) {
+      dst[I::VX + 2 * I::MP * g + m] = C.V[m][g];
+      if (DIM == 2) dst[I::VY + 2 * (I::N * g + m)] = dst[I::VY + 2 * (I::N * g + m) + 1] = C.V[m][g];
+    }
+  return I::FLOATS;
 }
-}  // namespace
 
-cudaError_t launch_tab_image(int dim, int p, const void* t, float* dst, cudaStream_t s) {
-  if (!t || !dst) return cudaErrorInvalidValue;
+int cg_image(int dim, int p, const void* tables, float* dst, int capacity) {
   switch (dim * 10 + p) {
-    case 11: return tab_image<1, 1>(t, dst, s);
-    case 12: return tab_image<1, 2>(t, dst, s);
-    case 13: return tab_image<1, 3>(t, dst, s);
-    case 14: return tab_image<1, 4>(t, dst, s);
-    case 21: return tab_image<2, 1>(t, dst, s);
-    case 22: return tab_image<2, 2>(t, dst, s);
-    case 23: return tab_image<2, 3>(t, dst, s);
-    case 24: return tab_image<2, 4>(t, dst, s);
-    default: return cudaErrorNotSupported;
+    case 11: return fill_cg_image<1, 1>(tables, dst, capacity);
+    case 12: return fill_cg_image<1, 2>(tables, dst, capacity);
+    case 13: return fill_cg_image<1, 3>(tables, dst, capacity);
+    case 14: return fill_cg_image<1, 4>(tables, dst, capacity);
+    case 21: return fill_cg_image<2, 1>(tables, dst, capacity);
+    case 22: return fill_cg_image<2, 2>(tables, dst, capacity);
+    case 23: return fill_cg_image<2, 3>(tables, dst, capacity);
+    case 24: return fill_cg_image<2, 4>(tables, dst, capacity);
+    default: return 0;
   }
 }
 

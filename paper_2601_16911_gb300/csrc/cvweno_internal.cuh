@@ -71,7 +71,7 @@ struct PackedTables {
 // Reference-cell tabulations of one (dim, p) pair, FP64 on the host rounded once to
 // FP32, passed to the kernels by value (__grid_constant__), so that every warp reads
 // them through the constant bank with uniform addresses (the entries read with per-lane
-// indices come from TabImage instead).
+// indices come from PackedImage instead).
 //   E[k][m]     = P_m^(k)(+1); the value at -1 is (-1)^(m+k) E[k][m]
 //   B[q][m]     = P_m(xi_q), Bd[q][m] = P_m'(xi_q) at the n Gauss-Legendre nodes xi_q
 //   Bk[k][q][m] = P_m^(k)(xi_q) (pointwise semi-norm at quadrature nodes, stage d)
@@ -123,46 +123,7 @@ inline void pack_tables(DgTables<DIM, P>& t) {
   for (int m = 0; m < ND; ++m) k.tscale[m] = t.tscale[m];
 }
 
-// Device image of the tabulations that the stage kernels index with a different value in
-// every lane (A padded to NSP columns, B, Bd, Bk, w), in the order they take in shared
-// memory: a tile stages it with 16-byte copies from global memory, where reading the
-// by-value tables with per-lane indices would serialise in the constant bank.  Built on
-// the device from DgTables by launch_tab_image (once per mesh).
-template <int DIM, int P>
-struct TabImage {
-  using Tb = DgTables<DIM, P>;
-  static constexpr int N = P + 1, NS = Tb::NS, NC = Tb::NC;
-  static constexpr int NSP = (NS + 3) / 4 * 4;
-  static constexpr int A = 0;                  // [NC][NS][NSP], columns >= NS zero
-  static constexpr int B = A + NC * NS * NSP;  // [N][N]
-  static constexpr int BD = B + N * N;         // [N][N]
-  static constexpr int BK = BD + N * N;        // [N][N][N]
-  static constexpr int W = BK + N * N * N;     // [N]
-  static constexpr int FLOATS = (W + N + 3) / 4 * 4;  // whole 16-byte chunks (the CUDA-core kernels' part)
-  // The tensor-core form of the sensor's corner products (2D, p = 3): A[l] split into TF32
-  // hi and lo parts, zero-padded to TCK x TCK, in the canonical K-major operand layout
-  // [part][corner l][K chunk of 4][row i][4] (tc_tf32.cuh).
-  static constexpr bool HAS_TC = DIM == 2 && P == 3;
-  static constexpr int TCK = (NS + 15) / 16 * 16;
-  static constexpr int TC = FLOATS;
-  static constexpr int FLOATS_ALL = FLOATS + (HAS_TC ? 2 * NC * TCK * TCK : 0);
-};
 constexpr int imax(int a, int b) { return a > b ? a : b; }
-constexpr int kMaxTabImage = imax(TabImage<2, kMaxP>::FLOATS_ALL, TabImage<2, 3>::FLOATS_ALL);
-inline int tab_image_floats(int dim, int p) {
-  switch (dim * 10 + p) {
-    case 11: return TabImage<1, 1>::FLOATS_ALL;
-    case 12: return TabImage<1, 2>::FLOATS_ALL;
-    case 13: return TabImage<1, 3>::FLOATS_ALL;
-    case 14: return TabImage<1, 4>::FLOATS_ALL;
-    case 21: return TabImage<2, 1>::FLOATS_ALL;
-    case 22: return TabImage<2, 2>::FLOATS_ALL;
-    case 23: return TabImage<2, 3>::FLOATS_ALL;
-    case 24: return TabImage<2, 4>::FLOATS_ALL;
-    default: return 0;
-  }
-}
-
 // Device image of the node tabulations, in the order they take in shared memory.  Node
 // group g holds the Gauss nodes g and N - 1 - g (= -+xi; the middle node of an odd rule is
 // its own partner): rows of mode pairs for the x direction, every entry doubled for the y
@@ -264,8 +225,8 @@ struct StageArgs {
   float* feat_out;
   float* norm_out;     // kModeFeatures: ||u^e||_e per cell (may be null)
   float h_e;           // cell diameter
-  const float* tab_img;  // TabImage of the mesh's tabulations (device)
   const float* pk_img;   // PackedImage of the mesh's tabulations (device)
+  const float* cg_img;   // CG: CgImage of the nodal tables (device)
   float adv_vx, adv_vy;
   float gas_gamma;
   // CG only: nodal lattice and the per-stage work arrays
@@ -336,8 +297,8 @@ struct cvweno_mesh_s {
   // reference tabulations, one per (dim, p) -- only the matching one is filled
   void* tables;            // host copy of DgTables<dim, p>
   size_t tables_bytes;
-  float* d_tabimg;         // TabImage<dim, p> (device)
   float* d_pkimg;          // PackedImage<dim, p> (device)
+  float* d_cgimg;          // CG: CgImage<dim, p> (device)
   // CG: nodal lattice, tabulations and stage work arrays
   int kind;
   int nnx, nny;
@@ -393,10 +354,8 @@ cudaError_t launch_stage_euler(const cvweno_mesh_s* m, const StageArgs& a, cudaS
 cudaError_t launch_steps_1d_tile(const cvweno_mesh_s* m, const StepArgs& a, cudaStream_t s);
 // dg_euler.cu: the positivity limiter on a.u_in -> a.u_out (may alias), theta per cell
 cudaError_t launch_positivity(const cvweno_mesh_s* m, const StageArgs& a, float* theta, cudaStream_t s);
-// dg_scalar_2d.cu: writes TabImage<dim, p> of the host tables t (DgTables<dim, p>) to
-// dst (device, tab_image_floats(dim, p) floats), stream-ordered on s
-cudaError_t launch_tab_image(int dim, int p, const void* t, float* dst, cudaStream_t s);
-// dg_scalar_2d.cu: likewise PackedImage<dim, p> (packed_image_floats(dim, p) floats)
+// dg_scalar_2d.cu: writes PackedImage<dim, p> of the host tables t (DgTables<dim, p>) to
+// dst (device, packed_image_floats(dim, p) floats), stream-ordered on s
 cudaError_t launch_packed_image(int dim, int p, const void* t, float* dst, cudaStream_t s);
 // dg_euler.cu, dg_scalar_2d.cu: max over the cells of a.u_in of lambda_e at the volume and face
 // Gauss nodes (scalar: DG laws without a constant wave speed)
@@ -404,6 +363,10 @@ cudaError_t launch_wavespeed_euler(const cvweno_mesh_s* m, const StageArgs& a, c
 cudaError_t launch_wavespeed_scalar(const cvweno_mesh_s* m, const StageArgs& a, const MaxSlots& out, cudaStream_t s);
 // cg_scalar.cu
 cudaError_t launch_stage_cg(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t s);
+// cg_scalar.cu: the cell kernel's image of the nodal tables (CgTables<dim, p>) into dst (host);
+// the floats written, 0 where capacity is too small
+constexpr int kMaxCgImage = 128;
+int cg_image(int dim, int p, const void* tables, float* dst, int capacity);
 // api.cu: the stage arguments common to every launch on mesh m (no state pointers, no RK)
 StageArgs stage_base_args(const cvweno_mesh_s* m);
 // api.cu: with kernel timing on, records the next timing event of the step on s
