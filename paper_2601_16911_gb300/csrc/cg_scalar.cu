@@ -604,55 +604,48 @@ __global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>(), (cg_min_ct
       for (int aa = 0; aa < N; ++aa) r[aa] = fmaf(fy, C.wl[aa] * hdx, r[aa]);
     }
   }
-  if constexpr (ND % 4 == 0) {  // rloc is mesh-owned (aligned): 16-byte stores
+  // node row b of the cells of a mesh row is contiguous in rloc (mesh-owned, aligned): the warp's
+  // stores and the node kernel's gathers are whole lines
+  const size_t rowlen = (size_t)nx * N, row0 = DIM == 2 ? (size_t)gj * N * rowlen : 0;
 #pragma unroll
-    for (int q = 0; q < ND / 4; ++q)
-      reinterpret_cast<float4*>(a.rloc + cell * ND)[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-  } else {
+  for (int b = 0; b < NY1; ++b) {
+    const size_t k = row0 + b * rowlen + (size_t)gi * N;
+    if (!CVW_SPAN(a.status, k, N, CVW_EXTENT(a, lim_cell) * ND)) continue;
+    if constexpr (N == 4) {
+      *reinterpret_cast<float4*>(a.rloc + k) = make_float4(r[N * b], r[N * b + 1], r[N * b + N - 2], r[N * b + N - 1]);
+    } else if constexpr (N == 2) {
+      *reinterpret_cast<float2*>(a.rloc + k) = make_float2(r[N * b], r[N * b + 1]);
+    } else {
 #pragma unroll
-    for (int m = 0; m < ND; ++m) a.rloc[cell * ND + m] = r[m];
+      for (int m = 0; m < N; ++m) a.rloc[k + m] = r[N * b + m];
+    }
   }
 }
 
-// Nodal assembly r_j at lattice node (I, J), 0 <= I < nnx, 0 <= J < nny: the sum of the
-// cell-local residuals (which carry the telescoped flux of the cell means) over the
-// cells containing the node, in a fixed order: the cell below-left of the node first,
-// then the one to its right, then the row above.  A node with local index a = 0 in x
-// lies in cell i - 1 (as its local p) and cell i (as its local 0); likewise in y.
-template <int DIM, int P>
-__device__ __forceinline__ float node_residual(const StageArgs& a, int I, int J) {
-  constexpr int N = P + 1, ND = DIM == 2 ? N * N : N;
-  const int nx = a.nx;
+// 1D nodal assembly r_j at lattice node I, 0 <= I < nnx: the sum of the cell-local residuals
+// (which carry the telescoped flux of the cell means) over the cells containing the node, the
+// left one first.  A node with local index 0 lies in cell i - 1 (as its local p) and cell i.
+template <int P>
+__device__ __forceinline__ float node_residual(const StageArgs& a, int I) {
+  constexpr int N = P + 1;
   const int i = I / P, aa = I - i * P;
-  const int cx0 = aa == 0 ? (i == 0 ? nx - 1 : i - 1) : i, lx0 = aa == 0 ? P : aa;
-  const int64_t lim = CVW_EXTENT(a, lim_cell) * ND;
+  const int cx0 = aa == 0 ? (i == 0 ? a.nx - 1 : i - 1) : i, lx0 = aa == 0 ? P : aa;
+  const int64_t lim = CVW_EXTENT(a, lim_cell) * N;
   auto rl = [&](size_t k) { return CVW_SPAN(a.status, k, 1, lim) ? a.rloc[k] : 0.0f; };
-  if constexpr (DIM == 1) {
-    float r = rl((size_t)cx0 * ND + lx0);
-    if (aa == 0) r += rl((size_t)i * ND);
-    return r;
-  } else {
-    const int j = J / P, bb = J - j * P;
-    const int cy0 = bb == 0 ? (j == 0 ? a.ny - 1 : j - 1) : j, ly0 = bb == 0 ? P : bb;
-    const size_t row0 = (size_t)cy0 * nx, row1 = (size_t)j * nx;
-    float r = rl((row0 + cx0) * ND + lx0 + N * ly0);
-    if (aa == 0) r += rl((row0 + i) * ND + N * ly0);
-    if (bb == 0) {
-      r += rl((row1 + cx0) * ND + lx0);
-      if (aa == 0) r += rl((row1 + i) * ND);
-    }
-    return r;
-  }
+  float r = rl((size_t)cx0 * N + lx0);
+  if (aa == 0) r += rl((size_t)i * N);
+  return r;
 }
 
 // 1D nodal assembly: r_j and du = r_j / ML_j.
 template <int DIM, int P>
 __global__ void cg_node_rhs(const __grid_constant__ StageArgs a, const __grid_constant__ CgTables<DIM, P> C) {
+  static_assert(DIM == 1, "2D: cg_node_stage2d");
   const int64_t nn = (int64_t)a.nnx * (DIM == 2 ? a.nny : 1);
   const float hdx = 1.0f / a.two_dx, hdy = DIM == 2 ? 1.0f / a.two_dy : 1.0f;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nn; j += (int64_t)gridDim.x * blockDim.x) {
     const int I = (int)(j % a.nnx), J = (int)(j / a.nnx);
-    const float r = node_residual<DIM, P>(a, I, J);
+    const float r = node_residual<P>(a, I);
     const float ml = ml1(C, I % P, hdx) * (DIM == 2 ? ml1(C, J % P, hdy) : 1.0f);
     if (!CVW_SPAN(a.status, j, 1, a.lim_out)) continue;
     a.rnode[j] = r;
@@ -726,23 +719,32 @@ __global__ void cg_node_sweep(const __grid_constant__ StageArgs a, const __grid_
 // x (each node sums M1[local][b] du over the nodes of the up to two cells containing it),
 // then along y.  The halo values are recomputed by every tile that needs them, in the same
 // arithmetic, so neighbouring tiles agree bitwise.
-// 32x32 tiles of 1024 threads from p = 3 on, 32x16 of 512 threads below (measured)
-constexpr int kNdX = 32;
+// The kernel is bound by its barriers and the halo (a 32x32 tile at p = 3 forms r on 44x44 nodes):
+// 32x32 tiles of 1024 threads (or 64x32 of 512, launch_cg_t) from p = 3 on, 32x16 of 512 below.
+// The gathers read node rows of the cells of a mesh row, contiguous in rloc (KPP Q3 256^2 85.9 ->
+// 84.4 us per step against cell by cell, both kernels).
 template <int P>
 __host__ __device__ constexpr int node_tile_y() { return P >= 3 ? 32 : 16; }
+template <int P, int kNdX>
+struct NodeLayout {
+  static constexpr int kNdY = node_tile_y<P>();
+  static constexpr int RX = kNdX + 4 * P, RY = kNdY + 4 * P;  // r and du0 window (halo 2p)
+  static constexpr int DX = kNdX + 2 * P, DY = kNdY + 2 * P;  // du1 window (halo p)
+  static constexpr size_t BYTES = sizeof(float) * (2 * RY * RX + RY * DX + DY * DX);
+};
 
-
-template <int P>
-__global__ void __launch_bounds__(kNdX* node_tile_y<P>(), 2048 / (kNdX * node_tile_y<P>()))
+template <int P, int kNdX, int NT, int CTAS>
+__global__ void __launch_bounds__(NT, CTAS)
     cg_node_stage2d(const __grid_constant__ StageArgs a, const __grid_constant__ CgTables<2, P> C) {
-  constexpr int kNdY = node_tile_y<P>();
-  constexpr int N = P + 1, NT = kNdX * kNdY;
-  constexpr int RX = kNdX + 4 * P, RY = kNdY + 4 * P;  // r and du0 window (halo 2p)
-  constexpr int DX = kNdX + 2 * P, DY = kNdY + 2 * P;  // du1 window (halo p)
-  __shared__ float sr[RY][RX];
-  __shared__ float sd0[RY][RX];
-  __shared__ float sxp[RY * DX];  // x-pass of M_C du0 [RY][DX], then of M_C du1 [DY][kNdX]
-  __shared__ float sd1[DY][DX];
+  using L = NodeLayout<P, kNdX>;
+  constexpr int N = P + 1, kNdY = L::kNdY, RX = L::RX, RY = L::RY, DX = L::DX, DY = L::DY;
+  constexpr int NO = kNdX * kNdY / NT, TR = NT / kNdX;  // output nodes of a thread, rows apart
+  static_assert(NO * NT == kNdX * kNdY && TR * kNdX == NT && RX + RY <= NT, "threads of a node tile");
+  extern __shared__ __align__(16) float nsm[];
+  float (*sr)[RX] = reinterpret_cast<float (*)[RX]>(nsm);
+  float (*sd0)[RX] = reinterpret_cast<float (*)[RX]>(nsm + RY * RX);
+  float (*sd1)[DX] = reinterpret_cast<float (*)[DX]>(nsm + 2 * RY * RX);
+  float* sxp = nsm + 2 * RY * RX + DY * DX;  // x-pass of M_C du0 [RY][DX], then of M_C du1 [DY][kNdX]
   __shared__ float sM1[N][N];
   // per window column rx (lattice column I0 - 2p + rx) and row ry: the offsets of the
   // local residual entries the node gathers (B: the second cell, -1 if none), the node's
@@ -754,15 +756,14 @@ __global__ void __launch_bounds__(kNdX* node_tile_y<P>(), 2048 / (kNdX * node_ti
   const int I0 = blockIdx.x * kNdX, J0 = blockIdx.y * kNdY;
   const float hh = (1.0f / a.two_dx) * (1.0f / a.two_dy), k2 = a.two_dx * a.two_dy;
   if (threadIdx.x < N * N) sM1[threadIdx.x / N][threadIdx.x % N] = (&C.M1[0][0])[threadIdx.x];
-  // this thread's output node; its RK inputs are loaded right after pdl_wait, so that their
+  // this thread's output nodes; their RK inputs are loaded right after pdl_wait, so that their
   // latency overlaps the window (u_n may alias u_out: only this thread reads or writes
-  // node j)
-  const int tx = threadIdx.x % kNdX, ty = threadIdx.x / kNdX;
-  const int I = I0 + tx, J = J0 + ty;
-  const bool own = I < nnx && J < nny;
-  const size_t j = own ? (size_t)J * nnx + I : 0;
+  // its nodes)
+  const int tx = threadIdx.x % kNdX, ty0 = threadIdx.x / kNdX;
   const bool rk = (a.mode & kModeRK) != 0, with_un = rk && a.rk_a != 0.0f;
-  float uin = 0.0f, un = 0.0f;
+  float uin[NO], un[NO];
+  auto own = [&](int k) { return I0 + tx < nnx && J0 + ty0 + k * TR < nny; };
+  auto node = [&](int k) { return (size_t)(J0 + ty0 + k * TR) * nnx + I0 + tx; };
   // 1 / (m_l wl[l]) of 1D local index l in [0, p)
   auto iml = [&](int l) {
     float v = C.iml[0];
@@ -775,23 +776,26 @@ __global__ void __launch_bounds__(kNdX* node_tile_y<P>(), 2048 / (kNdX * node_ti
   if (threadIdx.x < RX) {
     const int rx = threadIdx.x, Iw = wrap_index(I0 - 2 * P + rx, nnx), i = Iw / P, aa = Iw - i * P;
     const int cx0 = aa == 0 ? (i == 0 ? a.nx - 1 : i - 1) : i;
-    scolA[rx] = cx0 * (N * N) + (aa == 0 ? P : aa);
-    scolB[rx] = aa == 0 ? i * (N * N) : -1;
+    scolA[rx] = cx0 * N + (aa == 0 ? P : aa);
+    scolB[rx] = aa == 0 ? i * N : -1;
     slx[rx] = aa;
     simlx[rx] = iml(aa);
   } else if (threadIdx.x < RX + RY) {
     const int ry = threadIdx.x - RX, Jw = wrap_index(J0 - 2 * P + ry, nny), jc = Jw / P, bb = Jw - jc * P;
     const int cy0 = bb == 0 ? (jc == 0 ? a.ny - 1 : jc - 1) : jc;
-    const long long rowlen = (long long)a.nx * (N * N);
-    srowA[ry] = cy0 * rowlen + N * (bb == 0 ? P : bb);
-    srowB[ry] = bb == 0 ? jc * rowlen : -1;
+    const long long rowlen = (long long)a.nx * N;
+    srowA[ry] = (cy0 * N + (bb == 0 ? P : bb)) * rowlen;
+    srowB[ry] = bb == 0 ? jc * N * rowlen : -1;
     sly[ry] = bb;
     simly[ry] = iml(bb);
   }
   pdl_wait();  // everything below reads or writes what earlier kernels write
-  const bool own_ok = own && CVW_SPAN(a.status, j, 1, a.lim_in) && CVW_SPAN(a.status, j, 1, a.lim_out);
-  if (own_ok && rk) uin = a.u_in[j];
-  if (own_ok && with_un) un = a.u_n[j];
+#pragma unroll
+  for (int k = 0; k < NO; ++k) {
+    const bool ok = own(k) && CVW_SPAN(a.status, node(k), 1, a.lim_in) && CVW_SPAN(a.status, node(k), 1, a.lim_out);
+    uin[k] = ok && rk ? a.u_in[node(k)] : 0.0f;
+    un[k] = ok && with_un ? a.u_n[node(k)] : 0.0f;
+  }
   __syncthreads();
   // ---- r and du0 on the window: every gather of the thread in flight before the first use -----
   constexpr int NW = (RX * RY + NT - 1) / NT;
@@ -914,26 +918,39 @@ __global__ void __launch_bounds__(kNdX* node_tile_y<P>(), 2048 / (kNdX * node_ti
   }
   __syncthreads();
   pdl_launch_dependents();
-  if (!own_ok) return;
-  // ---- second sweep: y-pass at this thread's node, and the stage output ----------------------
-  const int ay = sly[ty + 2 * P], ly0 = ay == 0 ? P : ay, dy = ty + P;
-  float mc = 0.0f;
+  // ---- second sweep: y-pass at this thread's nodes, and the stage output --------------------
 #pragma unroll
-  for (int d = 0; d <= P; ++d) mc = fmaf(sM1[ly0][d], sxp[(dy - ly0 + d) * kNdX + tx], mc);
-  if (ay == 0) {
+  for (int k = 0; k < NO; ++k) {
+    if (!own(k)) continue;
+    const size_t j = node(k);
+    if (!CVW_SPAN(a.status, j, 1, a.lim_in) || !CVW_SPAN(a.status, j, 1, a.lim_out)) continue;
+    const int ty = ty0 + k * TR, ay = sly[ty + 2 * P], ly0 = ay == 0 ? P : ay, dy = ty + P;
+    float mc = 0.0f;
 #pragma unroll
-    for (int d = 0; d <= P; ++d) mc = fmaf(sM1[0][d], sxp[(dy + d) * kNdX + tx], mc);
-  }
-  const float du = sd1[dy][tx + P] + (sr[ty + 2 * P][tx + 2 * P] - mc * hh) * (simlx[tx + 2 * P] * simly[ty + 2 * P] * k2);
-  if (rk) {
-    float v = fmaf(a.dt, du, uin);
-    if (with_un) v = fmaf(a.rk_b, v - un, un);
+    for (int d = 0; d <= P; ++d) mc = fmaf(sM1[ly0][d], sxp[(dy - ly0 + d) * kNdX + tx], mc);
+    if (ay == 0) {
+#pragma unroll
+      for (int d = 0; d <= P; ++d) mc = fmaf(sM1[0][d], sxp[(dy + d) * kNdX + tx], mc);
+    }
+    float v = sd1[dy][tx + P] + (sr[ty + 2 * P][tx + 2 * P] - mc * hh) * (simlx[tx + 2 * P] * simly[ty + 2 * P] * k2);
+    if (rk) {
+      v = fmaf(a.dt, v, uin[k]);
+      if (with_un) v = fmaf(a.rk_b, v - un[k], un[k]);
+    }
     a.u_out[j] = v;
     if (!isfinite(v)) atomicOr(a.status, kStatNonfinite);
-  } else {
-    a.u_out[j] = du;
-    if (!isfinite(du)) atomicOr(a.status, kStatNonfinite);
   }
+}
+
+template <int P, int W, int NT, int CTAS>
+cudaError_t launch_nodes(const StageArgs& a, const CgTables<2, P>& C, cudaStream_t s) {
+  using L = NodeLayout<P, W>;
+  auto kern = cg_node_stage2d<P, W, NT, CTAS>;
+  if (L::BYTES > 40 * 1024) {  // (beside the static arrays)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_pdl(kern, dim3((a.nnx + W - 1) / W, (a.nny + L::kNdY - 1) / L::kNdY), dim3(NT), L::BYTES, s, a, C);
 }
 
 template <int DIM, int P, int SYS, int TX, int TY>
@@ -956,9 +973,18 @@ cudaError_t launch_cg_t(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t
   if (a.mode & kModeSensorOnly) return cudaGetLastError();
   kernel_mark(m, s);
   if constexpr (DIM == 2) {
-    constexpr int kNdY = node_tile_y<P>();
-    const dim3 ng((a.nnx + kNdX - 1) / kNdX, (a.nny + kNdY - 1) / kNdY);
-    e = launch_pdl(cg_node_stage2d<P>, ng, dim3(kNdX * kNdY), 0, s, a, C);
+    // 32-wide tiles of 1024 threads are resident 2 per SM (2 x 152 on the chip).  From one and a half
+    // such waves on, 64-wide tiles of 512 threads recompute less halo in half the waves (us per step,
+    // 32 / 64 wide: KPP Q3 256^2 cells 84.7 / 82.4, 512^2 266 / 244.5, Burgers Q4 256^2 248 / 245);
+    // at 324 tiles a few SMs would hold two wide ones (Q4 144^2 126.9 / 131.3).  Below p = 3 the
+    // halo is thin and width gains nothing (Q1 256^2 31.4 / 31.7).
+    constexpr int kNdY = node_tile_y<P>(), NT1 = 32 * kNdY;
+    const int64_t tiles = (int64_t)((a.nnx + 31) / 32) * ((a.nny + kNdY - 1) / kNdY);
+    const bool wide = P >= 3 && tiles > 3 * 152;
+    if constexpr (P >= 3)
+      e = wide ? launch_nodes<P, 64, 512, 2>(a, C, s) : launch_nodes<P, 32, NT1, 2048 / NT1>(a, C, s);
+    else
+      e = launch_nodes<P, 32, NT1, 2048 / NT1>(a, C, s);
     if (e != cudaSuccess) return e;
     kernel_mark(m, s);
   } else {

@@ -231,7 +231,7 @@ struct StageArgs {
   float gas_gamma;
   // CG only: nodal lattice and the per-stage work arrays
   int nnx, nny;
-  float* rloc;  // [ncell][nd] cell-local residuals
+  float* rloc;  // cell-local residuals, [ny][p + 1][nx][p + 1]: node rows of the cells of a mesh row
   float* rnode; // [nnode] assembled residual (1D)
   float* du;    // [nnode] du/dt iterate (1D)
   float* du2;   // [nnode] second defect-correction iterate (1D)
