@@ -364,7 +364,9 @@ __global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>(), (cg_min_ct
     // lambda_e over the volume and face Gauss nodes of the cell polynomial
     if (need_lam) {
       c[0][0].x = 0.0f;
-      lam = cell_speed<DIM, P>(img, law, ubar, c);
+      // (the mean's speed, never above the nodes', keeps an infinite state's speed infinite where the
+      // deviations are NaN)
+      lam = fmaxf(cell_speed<DIM, P>(img, law, ubar, c), law.speed(ubar));
     }
     if (a.gamma_out) a.gamma_out[cell] = gam;
     if (a.nu_out) a.nu_out[cell] = lam * a.nu_scale;
