@@ -44,13 +44,20 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
 }
 
-// GELU, tanh form, with the hardware tanh approximation (its error, ~2^-11 relative, is
-// below the bf16 rounding that follows).
-__device__ __forceinline__ float gelu_fast(float x) {
-  const float u = 0.7978845608028654f * fmaf(0.044715f * x * x, x, x);
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
-  return 0.5f * x * (1.0f + t);
+// GELU of two activations, tanh form, as the packed pair of the next layer's fragment.  The
+// hardware tanh approximation's error (~2^-11 relative) is below the bf16 rounding that
+// follows.  A cell takes 128 of them, most of the network's issue slots; on two-wide FP32
+// operations a pair is five of them beside the two tanh.
+__device__ __forceinline__ uint32_t gelu_pair(float a, float b) {
+  constexpr float kC = 0.7978845608028654f, kC3 = 0.7978845608028654f * 0.044715f;
+  const float2 x = make_float2(a, b);
+  const float2 q = __ffma2_rn(__fmul2_rn(x, x), make_float2(kC3, kC3), make_float2(kC, kC));
+  const float2 u = __fmul2_rn(x, q), h = __fmul2_rn(x, make_float2(0.5f, 0.5f));
+  float2 t;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(t.x) : "f"(u.x));
+  asm("tanh.approx.f32 %0, %1;" : "=f"(t.y) : "f"(u.y));
+  const float2 g = __ffma2_rn(h, t, h);
+  return pack_bf16x2(g.x, g.y);
 }
 
 // One warp, 32 samples.  x: this lane's 12 inputs; xs: 32 x 16 bf16 warp scratch in shared
@@ -80,8 +87,8 @@ __device__ __forceinline__ void mlp_warp(const MlpPacked& W, const float (&x)[kM
       const float bl = W.b1[8 * nt + 2 * t], bh = W.b1[8 * nt + 2 * t + 1];
       float c[4] = {bl, bh, bl, bh};
       mma_bf16_16816(c, a_in, W.w1[nt][lane]);
-      const uint32_t lo = pack_bf16x2(gelu_fast(c[0]), gelu_fast(c[1]));
-      const uint32_t hi = pack_bf16x2(gelu_fast(c[2]), gelu_fast(c[3]));
+      const uint32_t lo = gelu_pair(c[0], c[1]);
+      const uint32_t hi = gelu_pair(c[2], c[3]);
       a1[nt >> 1][(nt & 1) ? 2 : 0] = lo;
       a1[nt >> 1][(nt & 1) ? 3 : 1] = hi;
     }
@@ -93,8 +100,8 @@ __device__ __forceinline__ void mlp_warp(const MlpPacked& W, const float (&x)[kM
       float c[4] = {bl, bh, bl, bh};
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) mma_bf16_16816(c, a1[kk], W.w2[kk][nt][lane]);
-      const uint32_t lo = pack_bf16x2(gelu_fast(c[0]), gelu_fast(c[1]));
-      const uint32_t hi = pack_bf16x2(gelu_fast(c[2]), gelu_fast(c[3]));
+      const uint32_t lo = gelu_pair(c[0], c[1]);
+      const uint32_t hi = gelu_pair(c[2], c[3]);
       a2[nt >> 1][(nt & 1) ? 2 : 0] = lo;
       a2[nt >> 1][(nt & 1) ? 3 : 1] = hi;
     }
