@@ -221,21 +221,21 @@ __device__ __forceinline__ void projection_values(const f2 (&b)[MP], const f2* s
 // Threads of a block of the CG cell kernel, and the resident CTAs its registers must allow.
 // KPP 256^2, us per step: p = 3, 4 CTAs of 128 threads 85.9, 4 of 160 (96 registers, spills) 91.0,
 // 3 of 128 95.9, 5 of 128 92.7; p = 2, 4 CTAs 56.6, 3 69.7, 5 58.1.
-template <int DIM, int P, int TX, int TY>
+template <int DIM, int P, int TX, int TY, bool FEW = false>
 __host__ __device__ constexpr int cg_block_threads() {
-  return TX * TY + (DIM == 1 || P == 1 ? 32 : 0);
+  return TX * TY + (DIM == 1 || P == 1 || FEW ? 32 : 0);
 }
-template <int DIM, int P>
+template <int DIM, int P, bool FEW = false>
 constexpr int cg_min_ctas() {
-  return DIM == 1 ? 1 : P == 1 ? 6 : P <= 3 ? 4 : 2;
+  return DIM == 1 || FEW ? 1 : P == 1 ? 6 : P <= 3 ? 4 : 2;
 }
 
 // One CTA per tile; bound by FP32 issue and latency at 13 warps per SM (49 % of the issue slots at
 // 256^2).  On two-wide FMAs and in the modal basis (local integrals, projection and residual go
 // to the nodes and back by V) the Q3 step takes 85.9 us instead of 107, Q2 56.6 instead of 65, Q1
 // 29.7 instead of 42 (KPP 256^2, node kernel included).
-template <int DIM, int P, int SYS, int TX, int TY>
-__global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>(), (cg_min_ctas<DIM, P>()))
+template <int DIM, int P, int SYS, int TX, int TY, bool FEW = false>
+__global__ void __launch_bounds__((cg_block_threads<DIM, P, TX, TY, FEW>()), (cg_min_ctas<DIM, P, FEW>()))
     cg_stage_cells(const __grid_constant__ StageArgs a, const __grid_constant__ PackedTables<DIM, P> T,
                    const __grid_constant__ CgTables<DIM, P> C) {
   using G = CgLayout<DIM, P, TX, TY>;
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(cg_block_threads<DIM, P, TX, TY>(), (cg_min_ct
   using Img = PackedImage<DIM, P>;
   using Law = ScalarLaw<SYS, DIM>;
   constexpr int N = L::N, ND = L::ND, NT = L::NT, HX = L::HX, HY = L::HY, NH = L::NH, MP = L::MP, NG = L::NG;
-  constexpr int NB = cg_block_threads<DIM, P, TX, TY>();  // threads of the block
+  constexpr int NB = cg_block_threads<DIM, P, TX, TY, FEW>();  // threads of the block
   constexpr int NNX = G::NNX, NNY = G::NNY, NNXP = G::NNXP;
   constexpr int NY1 = L::NY1, NGY = DIM == 2 ? NG : 1;
   extern __shared__ __align__(16) float smem[];
@@ -964,13 +964,23 @@ cudaError_t launch_cg_t(const cvweno_mesh_s* m, const StageArgs& a, cudaStream_t
   if (m->tables_bytes != sizeof(Tb) || m->cg_tables_bytes != sizeof(Cb)) return cudaErrorInvalidValue;
   const PackedTables<DIM, P>& T = static_cast<const Tb*>(m->tables)->pk;
   const Cb& C = *static_cast<const Cb*>(m->cg_tables);
+  dim3 grid((a.nx + TX - 1) / TX, DIM == 2 ? (a.ny + TY - 1) / TY : 1);
   auto k1 = cg_stage_cells<DIM, P, SYS, TX, TY>;
+  int threads = cg_block_threads<DIM, P, TX, TY>();
+  // FEW: at most one block per SM, where only a block's latency counts: a warp more, so that the
+  // tile's vertices take one round, and registers uncapped.  CG Q2 per step, plain / FEW: Burgers
+  // 60^2 36.5 / 34.5 us, 110^2 38.4 / 37.0; on larger grids the fifth warp spills at 4 blocks per SM.
+  if constexpr (DIM == 2 && P == 2) {
+    if ((int64_t)grid.x * grid.y <= 152) {
+      k1 = cg_stage_cells<DIM, P, SYS, TX, TY, true>;
+      threads = cg_block_threads<DIM, P, TX, TY, true>();
+    }
+  }
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  dim3 grid((a.nx + TX - 1) / TX, DIM == 2 ? (a.ny + TY - 1) / TY : 1);
-  cudaError_t e = launch_pdl(k1, grid, dim3(cg_block_threads<DIM, P, TX, TY>()), smem, s, a, T, C);
+  cudaError_t e = launch_pdl(k1, grid, dim3(threads), smem, s, a, T, C);
   if (e != cudaSuccess) return e;
   if (a.mode & kModeSensorOnly) return cudaGetLastError();
   kernel_mark(m, s);
