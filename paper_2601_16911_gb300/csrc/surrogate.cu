@@ -89,9 +89,11 @@ __device__ __forceinline__ void dot_tile(const float* v, int vstride, const floa
 // minibatch of 4,096 128 blocks.  Bound by FP32 issue (tanhf and the products).
 // Minibatch 4,096: 20 us (one output per thread and step, W2 rows 64 floats apart: every
 // load of a warp hit one bank: 65 us).
+// Plain pointers, here and in the reduction: a block may be resident before pdl_wait() while the
+// kernel before it writes params (or gpart), so nothing may be read as unchanging data.
 __global__ void __launch_bounds__(kGradThreads, 2)
-    mlp_grad_kernel(const float* __restrict__ params, const float* __restrict__ X, const float* __restrict__ y,
-                    int64_t n, int64_t per_block, float* __restrict__ gpart, float* __restrict__ lpart) {
+    mlp_grad_kernel(const float* params, const float* X, const float* y, int64_t n, int64_t per_block, float* gpart,
+                    float* lpart) {
   extern __shared__ __align__(16) float sm[];
   using L = GradLayout;
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -267,8 +269,7 @@ __device__ __forceinline__ void adam_update(const AdamArgs& a, int p, float g) {
 constexpr int kRedParams = 32, kRedSlices = 8;
 template <bool ADAM>
 __global__ void __launch_bounds__(kRedParams* kRedSlices)
-    mlp_reduce_kernel(const float* __restrict__ gpart, const float* __restrict__ lpart, int nblk, float* __restrict__ grad,
-                      float* __restrict__ loss, AdamArgs a) {
+    mlp_reduce_kernel(const float* gpart, const float* lpart, int nblk, float* grad, float* loss, AdamArgs a) {
   __shared__ float part[kRedSlices][kRedParams];
   const int c = threadIdx.x % kRedParams, sl = threadIdx.x / kRedParams, p = blockIdx.x * kRedParams + c;
   pdl_wait();
