@@ -406,7 +406,9 @@ cvweno_status cvweno_features(cvweno_mesh m, const float* u, float* feats, float
 cvweno_status cvweno_mesh_set_surrogate(cvweno_mesh m, cvweno_mlp n, float conf_min);
 
 /* Cells that fell back to the plain sensor since the last reset, over every mesh n is
- * attached to (device counter read back: synchronises); reset != 0 zeroes it. */
+ * attached to and every evaluation of the sensor: each stage, residual and wave-speed call,
+ * so four per CFL-controlled step (device counter read back: synchronises); reset != 0
+ * zeroes it. */
 cvweno_status cvweno_mlp_fallbacks(cvweno_mlp n, uint64_t* count, int reset, void* stream);
 
 /* One SSP-RK3 step of fixed size dt > 0, in place on the caller's state u (device,

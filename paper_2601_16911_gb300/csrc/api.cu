@@ -918,9 +918,10 @@ cvweno_status cvweno_max_wavespeed(cvweno_mesh m, const float* u, double* lam, v
   a.u_in = u;
   cudaError_t e;
   double* out = m->d_red + kRedOut;
-  if (m->kind == CVWENO_CG || (m->desc.system != CVWENO_EULER && m->desc.params.lambda_const > 0.0)) {
+  if (m->kind == CVWENO_CG || (m->desc.system != CVWENO_EULER && m->desc.params.lambda_const > 0.0) || m->surrogate) {
     // CG cells' polynomials come from the stage kernel; a constant speed needs no pass, but takes
-    // this way for the same answer on an empty status
+    // this way for the same answer on an empty status; with the network attached the call is one
+    // more evaluation of the sensor, whose fallbacks are counted
     a.lambda_out = m->d_lambda;
     a.mode = kModeSensorOnly;
     e = launch(m, a, s);

@@ -200,3 +200,27 @@ def test_totals(system, nx, ny, p):
     # FP64 sums of the same numbers in another order
     assert np.abs(np.array(got[0]) - np.asarray(ref)).max() <= 1e-12 * np.abs(u[:, :, 0]).sum()
     mesh.close()
+
+
+@pytest.mark.parametrize("p", [1, 2, 4])
+def test_a_wave_speed_call_counts_its_fallbacks(p):
+    # conf_min = 1: every cell that is not flat falls back in every evaluation of the sensor, the one of
+    # a wave-speed call among them: a CFL-controlled step counts four times what a residual does
+    d = I.mesh(2, 21, 17, degree=p, system=I.BURGERS)
+    rng = np.random.default_rng(p)
+    u = to_gpu(rounded(rng.standard_normal(O.state_shape(d)) * 0.5))
+    net = cv.Mlp(np.array(I.mlp_init(5)))
+    mesh = cv.Mesh(d)
+    plain = mesh.max_wavespeed(u)
+    mesh.set_surrogate(net, conf_min=1.0)
+    mesh.residual(u)
+    once = net.fallbacks(reset=True)
+    assert once == d["nx"] * d["ny"]
+    speed = mesh.max_wavespeed(u)
+    assert net.fallbacks(reset=True) == once
+    assert abs(speed - plain) <= 1e-6 * plain
+    mesh.step(u, cfl=0.01)
+    assert net.fallbacks(reset=True) == 4 * once
+    mesh.set_surrogate(None)
+    mesh.close()
+    net.close()
