@@ -943,10 +943,19 @@ __global__ void __launch_bounds__(kCellThreads)
     if (!CVW_SPAN(a.status, ((NV - 1) * ncell + cell) * ND, ND, a.lim_in)) continue;
     f2 c[NV][N][MP];
     load_state<P>(a, a.u_in, cell, ncell, c);
-    for_node_groups<N, MP>(img, c, [&](const f2 (&ua)[NV], const f2 (&ub)[NV], bool mid) {
-      f2 vn, cs;
-      lam = fmaxf(lam, euler_wave(a.gas_gamma, ua, 0, vn, cs, bad));
-      if (!mid) lam = fmaxf(lam, euler_wave(a.gas_gamma, ub, 0, vn, cs, bad));
+    // mean + deviation, as in the stage: one rounding at the size of the mean
+    float Ubar[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Ubar[v] = c[v][0][0].x, c[v][0][0].x = 0.0f;
+    for_node_groups<N, MP>(img, c, [&](const f2 (&da)[NV], const f2 (&db)[NV], bool mid) {
+      f2 U[NV], vn, cs;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) U[v] = add2(dup2(Ubar[v]), da[v]);
+      lam = fmaxf(lam, euler_wave(a.gas_gamma, U, 0, vn, cs, bad));
+      if (mid) return;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) U[v] = add2(dup2(Ubar[v]), db[v]);
+      lam = fmaxf(lam, euler_wave(a.gas_gamma, U, 0, vn, cs, bad));
     });
   }
   if (bad) atomicOr(a.status, kStatPositivity);

@@ -224,3 +224,25 @@ def test_a_wave_speed_call_counts_its_fallbacks(p):
     mesh.set_surrogate(None)
     mesh.close()
     net.close()
+
+
+@pytest.mark.parametrize("direction", [0, 1])
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_euler_wave_speed_keeps_modes_below_an_ulp_of_the_mean(p, direction):
+    # p modes of 0.49 ulp of the mean each: their sum at one side of the cell is added to the mean
+    # there, so the speed is, to the bit, that of a cell whose mean has the rounded sum
+    d = I.mesh(2, 5, 3, degree=p, system=I.EULER, bc=I.TRANSMISSIVE)
+    n, mesh = p + 1, cv.Mesh(d)
+    rho, E = np.float32(1.0 + 8 * 2.0 ** -23), np.float32(2.0 + 8 * 2.0 ** -22)
+    base = np.zeros(O.state_shape(d), np.float32)
+    base[0, :, 0], base[3, :, 0] = rho, E
+    modes, whole = base.copy(), base.copy()
+    for v, mean, sign in ((0, rho, -1.0), (3, E, 1.0)):  # less dense and hotter: faster
+        part = np.float32(sign * 0.49 * np.spacing(mean))
+        for m in range(1, n):
+            modes[v, 7, m if direction == 0 else n * m] = part
+        whole[v, 7, 0] = np.float32(np.float64(mean) + p * np.float64(part))
+    still, got, want = (mesh.max_wavespeed(to_gpu(u)) for u in (base, modes, whole))
+    assert want > still
+    assert got == want
+    mesh.close()
