@@ -72,7 +72,6 @@ struct PackedTables {
 // FP32, passed to the kernels by value (__grid_constant__), so that every warp reads
 // them through the constant bank with uniform addresses (the entries read with per-lane
 // indices come from PackedImage instead).
-//   E[k][m]     = P_m^(k)(+1); the value at -1 is (-1)^(m+k) E[k][m]
 //   B[q][m]     = P_m(xi_q), Bd[q][m] = P_m'(xi_q) at the n Gauss-Legendre nodes xi_q
 //   Bk[k][q][m] = P_m^(k)(xi_q) (pointwise semi-norm at quadrature nodes, stage d)
 //   w[q]        Gauss weights on [-1,1]
@@ -89,7 +88,6 @@ struct DgTables {
   static constexpr int ND = DIM == 2 ? N * N : N;
   static constexpr int NS = ND - 1;
   static constexpr int NC = 1 << DIM;
-  float E[N][N];
   float B[N][N];
   float Bd[N][N];
   float Bk[N][N][N];
@@ -166,25 +164,16 @@ inline int packed_image_floats(int dim, int p) {
 
 // CG tabulations (Gauss-Lobatto-Legendre nodal basis l_a on [-1,1]):
 //   V[m][a]   Legendre mode m of l_a: (2m+1)/2 int P_m l_a      (nodal -> modal)
-//   Lq[q][a]  l_a(xi_q) and Ldq[q][a] = l_a'(xi_q) at the Gauss nodes
 //   M1[a][b]  int l_a l_b (1D reference mass), wl[a] = int l_a (GLL weight)
-//   xg[a]     GLL nodes
-//   Em[a][m]  int l_a P_m and Dm[a][m] = int l_a P_m' (local integrals of a Legendre
-//             expansion against the nodal basis)
 //   iml[a]    1 / (m_a wl[a]), m_a = 2 for the vertex node a = 0 (shared by two cells
 //             along the line), else 1: the inverse 1D lumped mass of local node a
 template <int DIM, int P>
 struct CgTables {
   static constexpr int N = P + 1;
   float V[N][N];
-  float Lq[N][N];
-  float Ldq[N][N];
   float M1[N][N];
-  float Em[N][N];
-  float Dm[N][N];
   float wl[N];
   float iml[N];
-  float xg[N];
 };
 
 // Run-time arguments of one stage launch.

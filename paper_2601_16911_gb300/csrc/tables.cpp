@@ -125,10 +125,6 @@ cvweno_status fill_into(DgTables<DIM, P>* t, double dx, double dy) {
   double gx[N], gw[N];
   gauss_golub_welsch(N, gx, gw);
   double tab[N * N];
-  // E at +1
-  legendre_derivs(1.0, P, P, tab);
-  for (int k = 0; k < N; ++k)
-    for (int mm = 0; mm < N; ++mm) t->E[k][mm] = (float)tab[k * N + mm];
   for (int q = 0; q < N; ++q) {
     legendre_derivs(gx[q], P, P, tab);
     for (int mm = 0; mm < N; ++mm) {
@@ -263,17 +259,12 @@ void gll_nodes(int p, double* x) {
   for (int i = 0; i < n; ++i) x[i + 1] = srt[i];
 }
 
-// Lagrange basis on nodes x[0..p]: value and first derivative of l_a at y (product rule)
-void lagrange_eval(int p, const double* x, int a, double y, double* val, double* der) {
-  double v = 1.0, d = 0.0;
-  for (int b = 0; b <= p; ++b) {
-    if (b == a) continue;
-    const double f = (y - x[b]) / (x[a] - x[b]);
-    d = d * f + v / (x[a] - x[b]);
-    v *= f;
-  }
-  *val = v;
-  *der = d;
+// Lagrange basis on nodes x[0..p]: l_a at y
+double lagrange(int p, const double* x, int a, double y) {
+  double v = 1.0;
+  for (int b = 0; b <= p; ++b)
+    if (b != a) v *= (y - x[b]) / (x[a] - x[b]);
+  return v;
 }
 
 template <int DIM, int P>
@@ -282,66 +273,33 @@ cvweno_status fill_cg(cvweno_mesh m) {
   constexpr int N = P + 1;
   C* t = (C*)calloc(1, sizeof(C));
   if (!t) return CVWENO_ERR_NOMEM;
-  double xg[N], gx[N], gw[N];
+  double xg[N];
   gll_nodes(P, xg);
-  gauss_golub_welsch(N, gx, gw);
   const int NG = 8;
   double qx[NG], qw[NG];
   gauss_golub_welsch(NG, qx, qw);
   for (int a = 0; a < N; ++a) {
-    t->xg[a] = (float)xg[a];
     m->cg_xg[a] = xg[a];
-    for (int q = 0; q < N; ++q) {
-      double v, d;
-      lagrange_eval(P, xg, a, gx[q], &v, &d);
-      t->Lq[q][a] = (float)v;
-      t->Ldq[q][a] = (float)d;
-    }
     double wl = 0.0;
-    for (int q = 0; q < NG; ++q) {
-      double va, da;
-      lagrange_eval(P, xg, a, qx[q], &va, &da);
-      wl += qw[q] * va;
-    }
+    for (int q = 0; q < NG; ++q) wl += qw[q] * lagrange(P, xg, a, qx[q]);
     t->wl[a] = (float)wl;
     t->iml[a] = (float)(1.0 / ((a == 0 ? 2.0 : 1.0) * wl));
     m->cg_wl[a] = wl;
   }
-  // Em[a][m] = int l_a P_m, Dm[a][m] = int l_a P_m' (exact: degree <= 2p < 2 NG)
-  for (int a = 0; a < N; ++a)
-    for (int mm = 0; mm < N; ++mm) {
-      double e = 0.0, dd = 0.0, tab[2 * N];
-      for (int q = 0; q < NG; ++q) {
-        double va, da;
-        lagrange_eval(P, xg, a, qx[q], &va, &da);
-        legendre_derivs(qx[q], P, 1, tab);
-        e += qw[q] * va * tab[mm];
-        dd += qw[q] * va * tab[N + mm];
-      }
-      t->Em[a][mm] = (float)e;
-      t->Dm[a][mm] = (float)dd;
-    }
   // V[m][a] = (2m+1)/2 int P_m l_a and M1[a][b] = int l_a l_b, in FP64 then rounded once
   for (int mm = 0; mm < N; ++mm)
     for (int a = 0; a < N; ++a) {
       double acc = 0.0, tab[N * N];
       for (int q = 0; q < NG; ++q) {
-        double va, da;
-        lagrange_eval(P, xg, a, qx[q], &va, &da);
         legendre_derivs(qx[q], P, 0, tab);
-        acc += qw[q] * tab[mm] * va;
+        acc += qw[q] * tab[mm] * lagrange(P, xg, a, qx[q]);
       }
       t->V[mm][a] = (float)(0.5 * (2 * mm + 1) * acc);
     }
   for (int a = 0; a < N; ++a)
     for (int b = 0; b < N; ++b) {
       double acc = 0.0;
-      for (int q = 0; q < NG; ++q) {
-        double va, da, vb, db;
-        lagrange_eval(P, xg, a, qx[q], &va, &da);
-        lagrange_eval(P, xg, b, qx[q], &vb, &db);
-        acc += qw[q] * va * vb;
-      }
+      for (int q = 0; q < NG; ++q) acc += qw[q] * lagrange(P, xg, a, qx[q]) * lagrange(P, xg, b, qx[q]);
       t->M1[a][b] = (float)acc;
     }
   m->cg_tables = t;
