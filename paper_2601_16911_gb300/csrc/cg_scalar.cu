@@ -61,8 +61,9 @@ struct CgLayout {
   static constexpr int NNXP = (NNX + 3 + 3) / 4 * 4;
   static constexpr int OFF_C = 0;                                              // cells
   static constexpr int OFF_ST = (L::VS * NH + 3) / 4 * 4;                      // vertex data, then stage (d)
-  static constexpr int OFF_NQ = OFF_ST, OFF_S12 = OFF_NQ + ND * NT;            // as the DG tile's
-  static constexpr int OFF_IMG = (OFF_ST + imax(L::VS * L::NVT, L::SCF) + 3) / 4 * 4;
+  // as the DG tile's; in 1D, where no barrier parts the sensor from stage (d), behind the vertex data
+  static constexpr int OFF_NQ = DIM == 1 ? OFF_ST + L::VS * L::NVT : OFF_ST, OFF_S12 = OFF_NQ + ND * NT;
+  static constexpr int OFF_IMG = ((DIM == 1 ? OFF_S12 : OFF_ST + imax(L::VS * L::NVT, L::SCF)) + 3) / 4 * 4;
   static constexpr int OFF_VIMG = OFF_IMG + Img::FLOATS;
   // The nodal tile is dead once the halo cells are converted to modes, the local integrals
   // (pairs (x, y), [ND][NH]) once P_h grad u is gathered; then its modes
@@ -214,6 +215,18 @@ __device__ __forceinline__ void projection_values(const f2 (&b)[MP], const f2* s
     f2 s = mul2(b[0], sp[my * MP * NT]);
 #pragma unroll
     for (int p = 1; p < MP; ++p) s = fma2(b[p], sp[(my * MP + p) * NT], s);
+    t[my] = mk2(s.x + s.y, s.x - s.y);
+  }
+}
+
+// The same of modes in registers.
+template <int NY1, int MP>
+__device__ __forceinline__ void projection_values(const f2 (&b)[MP], const f2 (&c)[NY1][MP], f2 (&t)[NY1]) {
+#pragma unroll
+  for (int my = 0; my < NY1; ++my) {
+    f2 s = mul2(b[0], c[my][0]);
+#pragma unroll
+    for (int p = 1; p < MP; ++p) s = fma2(b[p], c[my][p], s);
     t[my] = mk2(s.x + s.y, s.x - s.y);
   }
 }
@@ -417,11 +430,37 @@ __global__ void __launch_bounds__((cg_block_threads<DIM, P, TX, TY, FEW>()), (cg
     }
   }
   const bool need_sc = troubled && gam < 1.0f;
+  f2* sP = reinterpret_cast<f2*>(smem + G::OFF_PH);
+  if constexpr (DIM == 1) {
+    // by the cell's own thread, with the projection in its registers: cells of two to five nodes have
+    // less to share than the tile's barriers cost (300 cells P1: 27.9 us per step shared, 26.6 so with
+    // unrolled loops)
+    if (need_sc) {
+      float s1 = 0.0f, s2 = 0.0f;
+#pragma unroll 1
+      for (int g = 0; g < NG; ++g) {
+        f2 b[MP], d[MP], tb[1], td[1], tp[1], g1, g2, nq;
+        sc_node_group<DIM, P, TX, TY, false, L>(a, T, img, sNq, sc, nullptr, threadIdx.x, g, 0, g1, g2, &nq);
+        load_pairs<MP>(img + Img::BX + 2 * MP * g, b);
+        load_pairs<MP>(img + Img::DX + 2 * MP * g, d);
+        f2 cc[1][MP];
+        load_cell<L>(sc, L::cell(nullptr, hcx, 0), cc);
+        cc[0][0].x = 0.0f;
+        x_values<N, 1, MP>(b, d, cc, tb, td);
+        projection_values<1, MP>(b, px, tp);
+        const f2 f = mul2(dup2(-gam * a.two_dx * img[Img::WX + g]), mul2(td[0], tp[0]));
+        g1 = add2(g1, f);
+        g2 = fma2(nq, f, g2);
+        s1 += g1.x + g1.y;
+        s2 += g2.x + g2.y;
+      }
+      if (s1 > 0.0f && s2 > 0.0f) afac = s1 / s2;
+    }
+  } else {
   if (need_sc) sc_cell[atomicAdd(&sc_count, 1)] = (short)threadIdx.x;
   const bool any_sc = __syncthreads_or(need_sc);  // (and every cell has gathered the local integrals)
   // the projection's modes wait in shared memory: held in registers over the volume flux they
   // would cost the kernel a resident CTA
-  f2* sP = reinterpret_cast<f2*>(smem + G::OFF_PH);
   if (active) {
 #pragma unroll
     for (int my = 0; my < NY1; ++my)
@@ -493,6 +532,7 @@ __global__ void __launch_bounds__((cg_block_threads<DIM, P, TX, TY, FEW>()), (cg
       if (s1 > 0.0f && s2 > 0.0f) afac = s1 / s2;
     }
   }
+  }  // DIM == 2
   if (!active) return;
   if (a.troubled_out) a.troubled_out[cell] = troubled ? 1 : 0;
   if (a.alpha_out) {
@@ -524,7 +564,7 @@ __global__ void __launch_bounds__((cg_block_threads<DIM, P, TX, TY, FEW>()), (cg
       float even = 0.0f, odd = 0.0f;  // sums of the even and odd modes so far
 #pragma unroll
       for (int p = 0; p < MP; ++p) {
-        const f2 v = sP[(my * MP + p) * NT + threadIdx.x];
+        const f2 v = DIM == 1 ? px[my][p] : sP[(my * MP + p) * NT + threadIdx.x];
         const float e1 = even + v.x;
         R[my][p] = fma2(dup2(kx * sy), mk2(odd, e1), R[my][p]);
         even = e1;
@@ -553,7 +593,8 @@ __global__ void __launch_bounds__((cg_block_threads<DIM, P, TX, TY, FEW>()), (cg
       load_pairs<MP>(img + Img::BX + 2 * MP * g, b);
       load_pairs<MP>(img + Img::DX + 2 * MP * g, d);
       x_values<N, NY1, MP>(b, d, c, tb, td);
-      projection_values<NY1, MP, NT>(b, sP + threadIdx.x, tp);
+      if constexpr (DIM == 1) projection_values<NY1, MP>(b, px, tp);
+      else projection_values<NY1, MP, NT>(b, sP + threadIdx.x, tp);
       if (DIM == 2) projection_values<NY1, MP, NT>(b, sP + NY1 * MP * NT + threadIdx.x, tq);
 #pragma unroll
       for (int my = 0; my < NY1; ++my) hx[my] = hy[my] = mk2(0.0f, 0.0f);
@@ -677,7 +718,10 @@ __device__ __forceinline__ float mass_apply(const CgTables<DIM, P>& C, const flo
         const int lx = ax == 0 ? (kx == 0 ? P : 0) : ax;
         const int I0x = I - lx;
 #pragma unroll
-        for (int b = 0; b <= P; ++b) w = fmaf(C.M1[lx][b], rowp[((I0x + b) % nnx + nnx) % nnx], w);
+        for (int b = 0; b <= P; ++b) {
+          const int i = I0x + b;  // at most p <= nnx beyond either end (two modulos instead: P3 28.5 us per step, 26.5 so)
+          w = fmaf(C.M1[lx][b], rowp[i < 0 ? i + nnx : i >= nnx ? i - nnx : i], w);
+        }
       }
       acc = DIM == 2 ? fmaf(C.M1[ly][d], w, acc) : w;
     }

@@ -35,7 +35,8 @@
 // the batch 4.66 -> 3.36 ms, linear advection 330 x 170 Q4 residual 42.8 -> 31.3 us.
 //
 // Code-size discipline: the loops over vertex slots, corners and node groups are rolled
-// and read their tabulations (staged in shared memory) with uniform, broadcast loads, so
+// (not in 1D, where they are one to three short rounds of a latency-bound chain: CG P1 of 300
+// cells 23.6 -> 23.4 us per step, P3 28.2 -> 27.7) and read their tabulations (staged in shared memory) with uniform, broadcast loads, so
 // the kernel body stays within the instruction cache; only the short loops over modes are
 // unrolled into registers.  All arithmetic is FP32.
 #pragma once
@@ -887,7 +888,7 @@ __device__ __forceinline__ float cell_speed(const float* img, const Law& law, fl
   constexpr int N = Img::N, NY1 = Img::NY1, MP = Img::MP, NG = Img::NG;
   float lam = 0.0f;
   auto take = [&](f2 d) { lam = fmaxf(lam, fmaxf(law.speed(ubar + d.x), law.speed(ubar + d.y))); };
-#pragma unroll 1
+#pragma unroll (DIM == 1 ? 4 : 1)
   for (int g = 0; g <= NG; ++g) {
     f2 b[MP], tb[NY1];
     load_pairs<MP>(img + Img::BX + 2 * MP * (g < NG ? g : 0), b);
@@ -945,7 +946,7 @@ __device__ __forceinline__ void volume_flux(const StageArgs& a, const float* img
                                             f2 (&r)[PackedTables<DIM, P>::NY1][PackedTables<DIM, P>::MP]) {
   using Img = PackedImage<DIM, P>;
   constexpr int N = Img::N, NY1 = Img::NY1, MP = Img::MP, NG = Img::NG, NGY = DIM == 2 ? NG : 1;
-#pragma unroll 1
+#pragma unroll (DIM == 1 ? 3 : 1)
   for (int g = 0; g < NG; ++g) {
     f2 b[MP], tb[NY1];
     load_pairs<MP>(img + Img::BX + 2 * MP * g, b);
@@ -1089,7 +1090,7 @@ __device__ __forceinline__ void sc_node_group(const StageArgs& a, const PackedTa
   // squares of the derivatives at the nodes, (a) at +eta_h, (b) at -eta_h: the sum of all
   // weighted by sigma, and |grad u|^2; the signs (-1)^k at the mirrored nodes drop out
   f2 na = mk2(0.0f, 0.0f), nb = na, ga = na, gb = na;
-#pragma unroll 1
+#pragma unroll (DIM == 1 ? 5 : 1)
   for (int kx = 0; kx < N; ++kx) {
     f2 b[MP], X[NY1];
     load_pairs<MP>(img + Img::KX + 2 * MP * (kx * NG + g), b);
