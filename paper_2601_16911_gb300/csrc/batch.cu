@@ -380,22 +380,13 @@ void free_batch(cvweno_batch b) {
 }
 
 template <int P>
-bool same_tables(const PackedTables<2, P>& x, const PackedTables<2, P>& y) {
-  // everything but tscale (vertex-output scaling, not read by the batch)
-  PackedTables<2, P> a = x, c = y;
-  memset(a.tscale, 0, sizeof(a.tscale));
-  memset(c.tscale, 0, sizeof(c.tscale));
-  return memcmp(&a, &c, sizeof(a)) == 0;
-}
-
-template <int P>
 bool take_tables(PackedTables<2, P>& dst, bool have, const cvweno_mesh m) {
   const PackedTables<2, P>& src = static_cast<const DgTables<2, P>*>(m->tables)->pk;
   if (!have) {
     dst = src;
     return true;
   }
-  return same_tables<P>(dst, src);
+  return same_norms(dst, src);  // (tscale, the vertex-output scaling, is not read by the batch)
 }
 
 }  // namespace

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/cvweno.h"
 
@@ -119,6 +120,13 @@ inline void pack_tables(DgTables<DIM, P>& t) {
         }
     }
   for (int m = 0; m < ND; ++m) k.tscale[m] = t.tscale[m];
+}
+
+// Equal sigma2 and R2 (everything but tscale, which depends on the cell size).  Member by member: the
+// object has padding behind an odd tscale, which copies need not preserve.
+template <int DIM, int P>
+inline bool same_norms(const PackedTables<DIM, P>& x, const PackedTables<DIM, P>& y) {
+  return memcmp(x.sigma2, y.sigma2, sizeof(x.sigma2)) == 0 && memcmp(x.R2, y.R2, sizeof(x.R2)) == 0;
 }
 
 constexpr int imax(int a, int b) { return a > b ? a : b; }
