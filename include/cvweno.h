@@ -249,10 +249,13 @@ cvweno_status cvweno_positivity(cvweno_mesh m, const float* u, float* out, float
  * captured from such a step times each of its replays.  cvweno_kernel_times waits for
  * the last recorded event and writes the durations (ms) of the kernels of the most
  * recent step into ms[capacity] (host), in launch order: DG and Euler one per stage
- * (two with the HWENO or positivity limiter; with timing on, a one-tile 1D mesh also
- * launches stage by stage), CG two per stage in 2D (cells, then the
+ * (two with the HWENO or positivity limiter), CG two per stage in 2D (cells, then the
  * node phase: assembly and both defect-correction sweeps) and four in 1D (cells, node
- * right-hand side, two sweeps); *count receives how many were written.  Timing
+ * right-hand side, two sweeps); *count receives how many were written.  Two kinds of
+ * mesh launch more kernels with timing on than without, so there the durations are not
+ * those of an untimed step's kernels: the positivity limiter becomes a launch of its own
+ * (untimed steps limit inside the stage kernel), and a one-tile 1D mesh launches stage by
+ * stage (untimed: one launch for all steps).  Timing
  * costs one event record per kernel; turn it off (enable 0) for production runs.  Turning it off keeps the events
  * of the last timed step (and of graphs captured while it was on) readable. */
 cvweno_status cvweno_mesh_set_kernel_timing(cvweno_mesh m, int enable);

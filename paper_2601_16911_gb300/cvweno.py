@@ -347,7 +347,9 @@ class Mesh:
                "cvweno_mesh_set_check_extents")
 
     def kernel_times(self):
-        """Durations (ms) of the kernels of the most recent step, in launch order."""
+        """Durations (ms) of the kernels of the most recent timed step, in launch order.  With the
+        positivity limiter, and on a one-tile 1D mesh, an untimed step launches fewer, fused kernels
+        whose times these are not (include/cvweno.h)."""
         buf = (ctypes.c_float * 64)()
         n = ctypes.c_int(0)
         _check(load().cvweno_kernel_times(self._h, buf, 64, ctypes.byref(n)), "cvweno_kernel_times")
