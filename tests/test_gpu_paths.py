@@ -246,3 +246,49 @@ def test_euler_wave_speed_keeps_modes_below_an_ulp_of_the_mean(p, direction):
     assert want > still
     assert got == want
     mesh.close()
+
+
+def limited_step(d, u, dt, without=None):
+    """One limited SSP-RK3 step by the oracle (the limiter left out after stage `without`) and the
+    number of cells limited after each stage."""
+    plain, w, limited = dict(d, positivity=0), u, []
+    for k, (a, b) in enumerate(((0.0, 1.0), (0.75, 0.25), (1.0 / 3.0, 2.0 / 3.0))):
+        w = a * u + b * (w + dt * O.residual(plain, w)["dudt"].reshape(w.shape))
+        if k != without:
+            w, theta, _ = O.positivity(d, w)
+            limited.append(int((theta < 1.0).sum()))
+    return w, limited
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("nx,ny,seed", [(35, 19, 0), (20, 33, 1)])
+def test_positivity_in_the_stage_limits_in_every_stage(p, nx, ny, seed):
+    # pressures at the limiter's floor in many cells of several tiles: it acts after all three stages
+    d = I.mesh(2, nx, ny, degree=p, system=I.EULER, bc=I.TRANSMISSIVE, positivity=1)
+    u0 = rounded(O.positivity(d, random_state(d, np.random.default_rng(20 + p + seed), 1.6))[0])
+    dt = 0.2 / (max(nx, ny) * O.max_wavespeed(d, u0) * (2 * p + 1) * p)
+    ref, limited = limited_step(d, u0, dt)
+    assert min(limited) > 10
+    norm = np.abs(ref).max()
+    # near vacuum the step amplifies rounding: the bar is 32 times what one FP32 rounding of every input
+    # coefficient does to the FP64 step (some ten roundings of that size in each of three stages)
+    sens = 2.0 ** -23
+    for s in range(2):
+        noise = np.random.default_rng(s).uniform(-1.0, 1.0, u0.shape)
+        sens = max(sens, np.abs(limited_step(d, u0 * (1.0 + 2.0 ** -23 * noise), dt)[0] - ref).max() / norm)
+    tol = 32.0 * sens
+    assert np.abs(limited_step(d, u0, dt, without=2)[0] - ref).max() > 8.0 * tol * norm  # a lost limiter shows
+    fused, own = cv.Mesh(d), cv.Mesh(d)
+    own.set_kernel_timing(True)  # the limiter as a launch of its own
+    got = []
+    for m in (fused, own):
+        u = to_gpu(u0)
+        m.advance(u, dt, 1)
+        m.status_check()
+        got.append(u.cpu().numpy().astype(np.float64).reshape(u0.shape))
+    assert len(own.kernel_times()) == 6
+    fused.close()
+    own.close()
+    assert np.abs(got[0] - ref).max() <= tol * norm
+    assert np.abs(got[1] - ref).max() <= tol * norm
+    assert np.abs(got[0] - got[1]).max() <= tol * norm
