@@ -12,7 +12,7 @@ import torch
 from oracle import oracle as O
 from paper_2601_16911_gb300 import cvweno as cv
 from paper_2601_16911_gb300 import inputs as I
-from tests.gpu_common import ALPHA_TOL, RES_TOL, rel_err, rounded, to_gpu
+from tests.gpu_common import ALPHA_TOL, GAMMA_TOL, RES_TOL, rel_err, rounded, to_gpu
 from tests.test_gpu_alignment import misaligned_copy
 from tests.test_oracle_positivity import random_state
 
@@ -292,3 +292,41 @@ def test_positivity_in_the_stage_limits_in_every_stage(p, nx, ny, seed):
     assert np.abs(got[0] - ref).max() <= tol * norm
     assert np.abs(got[1] - ref).max() <= tol * norm
     assert np.abs(got[0] - got[1]).max() <= tol * norm
+
+
+def test_cg_q2_cell_kernels_on_both_sides_of_one_block_per_sm():
+    # as the node tiles above: 15 blocks, and 200 for the same state repeated 4 x 4 times
+    d = I.mesh(2, 40, 39, degree=2, system=I.BURGERS, kind=I.CG)
+    big = dict(d, nx=160, ny=156, x1=4.0, y1=4.0)
+    m, mb = cv.Mesh(d), cv.Mesh(big)
+    u = m.project(I.IC_FOURIER, FOURIER["fifteen"])
+    ub = u.view(78, 80).repeat(4, 4).contiguous().view(mb.empty_state().shape)
+    ov = torch.from_numpy((np.random.default_rng(2).uniform(size=(39, 40)) < 0.1).astype(np.int32)).cuda()
+    out = m.residual_ex(u, troubled_override=ov.view(-1))
+    outb = mb.residual_ex(ub, troubled_override=ov.repeat(4, 4).contiguous().view(-1))
+    m.status_check()
+    mb.status_check()
+    r, rb = out["dudt"].view(78, 80).repeat(4, 4), outb["dudt"].view(312, 320)
+    assert (r - rb).abs().max().item() <= RES_TOL * r.abs().max().item()
+    g, gb = out["gamma"].view(39, 40).repeat(4, 4), outb["gamma"].view(156, 160)
+    assert (g - gb).abs().max().item() <= GAMMA_TOL
+    m.close()
+    mb.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(192, 96), (208, 104)])  # 144 and 169 blocks
+@pytest.mark.parametrize("system", [I.BURGERS, I.KPP, I.LINADV])
+def test_cg_q2_cell_kernels_against_the_oracle(system, nx, ny):
+    d = I.mesh(2, nx, ny, degree=2, system=system, kind=I.CG)
+    rng = np.random.default_rng(nx)
+    u = rounded(rng.standard_normal(O.state_shape(d)) * 0.5)
+    ov = (rng.uniform(size=O.counts(d)["ncell"]) < 0.1).astype(np.int32)
+    ref = O.residual(d, u, ov)
+    mesh = cv.Mesh(d)
+    out = mesh.residual_ex(to_gpu(u), troubled_override=torch.from_numpy(ov).cuda())
+    mesh.status_check()
+    got = {k: v.cpu().numpy() for k, v in out.items()}
+    mesh.close()
+    assert np.array_equal(got["troubled"], ref["troubled"])
+    assert np.abs(got["alpha"] - ref["alpha"]).max() <= ALPHA_TOL * np.abs(ref["alpha"]).max()
+    assert rel_err(got["dudt"], ref["dudt"]) < RES_TOL
