@@ -315,9 +315,12 @@ __global__ void __launch_bounds__((cg_block_threads<DIM, P, TX, TY, FEW>()), (cg
   cp_async_wait_all();
   __syncthreads();
   // ---- every halo cell: nodal -> Legendre modes c = (V x V) u_loc -------------------------
-  // The transform is applied to u_loc - u_ref (u_ref = the cell's first node): every mode
-  // but the mean is unchanged (the rows of V beyond the mean sum to zero), the mean gets
-  // u_ref back, and a constant cell yields exactly zero non-mean modes.
+  // The transform is applied to u_loc - u_ref: every mode but the mean is unchanged (the rows of V
+  // beyond the mean sum to zero), the mean gets u_ref back, and a constant cell yields exactly zero
+  // non-mean modes.  u_ref is a middle node: the even modes come from sums of mirrored nodes,
+  // which about the middle nearly cancel on smooth data (about the first node they do not, and
+  // round at their own size: RMS error of the second and higher even modes 2 to 5 times as large at
+  // p = 2 and 4, 1.7 times at p = 3).
   for (int h = threadIdx.x; h < NH; h += NB) {
     const int hx = h % HX, hy = DIM == 2 ? h / HX : 0;
     float u[NY1][N];
@@ -325,7 +328,7 @@ __global__ void __launch_bounds__((cg_block_threads<DIM, P, TX, TY, FEW>()), (cg
     for (int b = 0; b < NY1; ++b)
 #pragma unroll
       for (int aa = 0; aa < N; ++aa) u[b][aa] = snode[sph[P * hy + b] + (P * hx + aa) + NNXP * (P * hy + b)];
-    const float uref = u[0][0];
+    const float uref = u[DIM == 2 ? P / 2 : 0][P / 2];
 #pragma unroll
     for (int b = 0; b < NY1; ++b)
 #pragma unroll

@@ -330,3 +330,26 @@ def test_cg_q2_cell_kernels_against_the_oracle(system, nx, ny):
     assert np.array_equal(got["troubled"], ref["troubled"])
     assert np.abs(got["alpha"] - ref["alpha"]).max() <= ALPHA_TOL * np.abs(ref["alpha"]).max()
     assert rel_err(got["dudt"], ref["dudt"]) < RES_TOL
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("p", [2, 4])
+def test_cg_cells_odd_about_their_middle_have_no_even_modes(p, dim):
+    # Nodal values c - d_g, ..., c, ..., c + d_g in x with arbitrary d_g, six cells rising and six falling: the
+    # even modes beyond the mean are zero, and sums of mirrored nodes about the middle one exactly so.
+    # The vertex candidates' highest x-derivative has the highest mode alone.
+    n = 12
+    d = I.mesh(dim, n, 5 if dim == 2 else 1, degree=p, system=I.BURGERS, kind=I.CG)
+    off = np.sort(np.random.default_rng(p).uniform(0.05, 0.4, p // 2))
+    off = np.round(off * 2.0 ** 20) / 2.0 ** 20  # every value below is an FP32 number
+    shape = np.concatenate([-off[::-1], [0.0], off])
+    middles = 1.0 + off[-1] * np.array([1, 3, 5, 7, 9, 11, 11, 9, 7, 5, 3, 1])
+    line = np.concatenate([(c + (shape if k < 6 else -shape))[:-1] for k, c in enumerate(middles)])
+    assert np.array_equal(line, line.astype(np.float32))
+    u = np.tile(line, (p * d["ny"] if dim == 2 else 1, 1))
+    mesh = cv.Mesh(d)
+    t = mesh.vertex_data(to_gpu(u.reshape(O.state_shape(d))))
+    mesh.status_check()
+    assert t[:, p].abs().max().item() == 0.0
+    assert t[:, 1].abs().max().item() > 1.0
+    mesh.close()
