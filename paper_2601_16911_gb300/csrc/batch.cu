@@ -84,9 +84,12 @@ constexpr size_t batch_smem(int psel) {
 // b, b + G, b + 2G, ...; otherwise sched[0] is the next unclaimed tile and sched[1]
 // counts CTAs that have left -- the last one resets both for the next launch in stream
 // order.  No CTA ever waits on another.
-// Register caps (CTAs per SM at 128 threads) at the single-mesh kernels' allocation:
-// without them the per-tile argument loads and the degree switch inflate the fused
-// kernel to the 255-register ceiling.
+// Register caps (CTAs per SM at 128 threads): without any, the per-tile argument loads and the
+// degree switch inflate the fused kernel to the 255-register ceiling.  Their values come from a
+// sweep of the scalar-FMA kernels and have not been swept for the two-wide ones, which they fit less
+// well: p = 2 is held to 80 registers and spills 232 B of stores and 296 B of loads (the single-mesh
+// kernel takes 92-94 and none), p = 3 has 128 and spills 92 / 76 B (96, at most 32 / 64 B), p = 4 168 and
+// 264-300 / 100-152 B (152-158, none), the fused kernel 168 and 1.1 KB each way.
 template <int PSEL, int TX, int TY>
 constexpr int batch_min_ctas() {
   return (PSEL == 0 || PSEL == 4 ? 3 : PSEL == 3 ? 4 : PSEL == 2 ? 6 : 8) * (128 / (TX * TY));

@@ -261,7 +261,9 @@ struct EulerLayout {
 // Minimum resident CTAs the register allocation must allow, from sweeps (us per step).
 // p = 1, 512^2: 4 CTAs of 160 threads 108.7, 3 CTAs 114, 6 CTAs 114.  p = 2, 512^2: 3 CTAs 321,
 // 2 CTAs 352 (but 5 % faster on meshes of one wave), 4 CTAs 360.  p = 3, 512^2: 2 CTAs at
-// 255 registers 415, 3 CTAs at 168 (spills) 496.  p = 4 (8x8 tiles), 300^2: 2 CTAs 494.
+// 255 registers 415, 3 CTAs at 168 496.  p = 4 (8x8 tiles), 300^2: 2 CTAs 494.  All forms from p = 2 on
+// spill; the ones in use, stores / loads: p = 2 (168 registers) 0.45 / 0.85 KB, p = 3 0.2 / 0.5 KB, p = 4
+// 1.3 / 2.3 KB, so at p = 3 what 3 CTAs lose is more spilling, not the first.
 template <int P, int TX, int TY>
 constexpr int euler_min_ctas() {
   return P == 1 ? 4 : P == 2 ? 3 : 2;
