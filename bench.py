@@ -276,14 +276,16 @@ def bytes_per_dof_stage() -> float:
 
 # Sources of each profiled kernel: a recorded DRAM traffic figure is used only while the
 # hash of these files matches the one stored beside it.
-COMMON = ["stage_common.cuh", "dg_packed.cuh"]
+# (Every header that a source includes is listed, the layouts of the tabulations among them.)
+COMMON = ["cvweno_internal.cuh", "stage_common.cuh", "dg_packed.cuh", "mlp_mma.cuh", "tc_tf32.cuh",
+          "dg_scalar_kernel.cuh"]
 KERNEL_SOURCES = {
-    "dg_scalar_stage_q3_kpp256": COMMON + ["dg_scalar_kernel.cuh", "dg_scalar_launch.cuh", "dg_scalar_2d.cu"],
-    "dg_scalar_steps_tile_p2_burgers1d": COMMON + ["dg_scalar_kernel.cuh", "dg_scalar_launch.cuh", "dg_scalar_1d.cu"],
-    "dg_euler_stage_q3_euler512": COMMON + ["dg_scalar_kernel.cuh", "dg_euler.cu"],
-    "dg_scalar_batch_burgers64": COMMON + ["dg_scalar_kernel.cuh", "batch.cu"],
-    "dg_scalar_stage_q2_surrogate_kpp1024": COMMON + ["dg_scalar_kernel.cuh", "mlp_mma.cuh", "dg_scalar_2d_mlp.cu"],
-    "cg_stage_cells_q3_kpp256": COMMON + ["dg_scalar_kernel.cuh", "cg_scalar.cu"],
+    "dg_scalar_stage_q3_kpp256": COMMON + ["dg_scalar_launch.cuh", "dg_scalar_2d.cu"],
+    "dg_scalar_steps_tile_p2_burgers1d": COMMON + ["dg_scalar_launch.cuh", "dg_scalar_1d.cu"],
+    "dg_euler_stage_q3_euler512": COMMON + ["dg_euler.cu"],
+    "dg_scalar_batch_burgers64": COMMON + ["batch.cu"],
+    "dg_scalar_stage_q2_surrogate_kpp1024": COMMON + ["dg_scalar_launch.cuh", "dg_scalar_2d_mlp.cu"],
+    "cg_stage_cells_q3_kpp256": COMMON + ["cg_scalar.cu"],
 }
 
 
