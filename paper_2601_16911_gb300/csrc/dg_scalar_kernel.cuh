@@ -1593,7 +1593,7 @@ __global__ void __launch_bounds__(128, 4)
 // other; u_n in the registers of the cell's thread) and goes back to global memory at the end;
 // a block barrier stands in for the kernel boundary.  Each stage is the stage kernel's code
 // with the same block, so the results are bitwise those of three launches per step.  Bound by
-// the latency of one cell's chain on 5 warps: Burgers P2, 128 cells, 10 steps 58.9 us (77.9 with
+// the latency of one cell's chain on 5 warps: Burgers P2, 128 cells, 10 steps 57.3 us (77.9 with
 // every stage's halo through global memory).
 template <int P, int SYS, int TX>
 __global__ void __launch_bounds__(stage_block_threads<1, P, TX, 1>())
