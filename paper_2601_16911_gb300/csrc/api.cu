@@ -347,7 +347,9 @@ __global__ void sum_cg_partial(const float* __restrict__ u, int nnx, int nny, in
 
 // DG conservation totals in one launch: block (b, v) sums mode 0 of a grid-stride slice of
 // variable v (FP64) into partial[v][b]; the last block to finish adds each variable's partials
-// in a fixed order into out[v] and leaves the counter zero for the next call.
+// in a fixed order into out[v].  The counter wraps to zero with the call's last block: calls that
+// overlap on one mesh (which share the partials, so their own totals are undefined) leave it
+// zero all the same, where a reset by the last block could leave a remainder for every later call.
 __global__ void __launch_bounds__(kRedThreads) sum_mode0_kernel(const float* __restrict__ u, int64_t n, int stride,
                                                                 double* __restrict__ partial, double* __restrict__ out,
                                                                 unsigned* done) {
@@ -369,7 +371,7 @@ __global__ void __launch_bounds__(kRedThreads) sum_mode0_kernel(const float* __r
     for (int w = 1; w < kRedThreads / 32; ++w) acc += sh[w];
     partial[v * kRedBlocks + blockIdx.x] = acc;
     __threadfence();
-    last = atomicAdd(done, 1u) == (unsigned)(nb * nvar) - 1;
+    last = atomicInc(done, (unsigned)(nb * nvar) - 1) == (unsigned)(nb * nvar) - 1;  // back to zero by itself
   }
   __syncthreads();
   if (!last) return;
@@ -380,7 +382,6 @@ __global__ void __launch_bounds__(kRedThreads) sum_mode0_kernel(const float* __r
     acc = warp_sum(acc);
     if (lane == 0) out[warp] = acc;
   }
-  if (threadIdx.x == 0) *done = 0;
 }
 
 __global__ void max_partial(const float* __restrict__ x, int64_t n, double* __restrict__ partial) {

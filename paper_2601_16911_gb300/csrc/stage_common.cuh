@@ -374,11 +374,10 @@ __device__ __forceinline__ void finish_max(float x, int* status, const MaxSlots&
   if (threadIdx.x == 0) {
     atomicMax(out.best, best);
     __threadfence();
-    if (atomicAdd(out.done, 1u) == gridDim.x - 1) {
+    if (atomicInc(out.done, gridDim.x - 1) == gridDim.x - 1) {  // back to zero by itself (sum_mode0_kernel)
       __threadfence();
       *out.max = (double)__uint_as_float(atomicExch(out.best, 0u));
       *out.status = atomicOr(status, 0);
-      *out.done = 0;
     }
   }
 }
